@@ -269,27 +269,55 @@ __device__ __forceinline__ double dkey_inv(uint64_t k) {
     return __longlong_as_double(b);
 }
 
-// Excess attitude noise (Sect. 5.2.5): eps_a^2 of the three components (AL, AC in the
-// preceding field, AC in the following field) per time bucket [t0 + j dt, t0 + (j+1) dt),
-// stored eps2[comp * n_b + j].  eps2 null: off.
-// 1/d for d > 0 by Newton's iteration for the reciprocal, y <- y + y (1 - d y), two steps
-// from an FP32 seed (rcp.approx of d rounded to FP32).  The seed's relative error e0 (below
-// 2^-22: the FP32 rounding of d plus the approximate reciprocal) becomes e0^2 after one step
-// and e0^4 < 2^-88 after two, so the result differs from 1/d by the rounding of the last
-// FMA: at most one FP64 ulp (the GPU unit test measures the largest difference from the
-// correctly rounded 1.0 / d over random and edge values).  d outside [2^-100, 2^101)
-// (exponent bits) takes the plain division.
+// 1/d for d > 0 from rcp.approx.ftz.f64, whose relative error e = 1 - d y is below 1.0e-6
+// (measured over [1, 4)), by the geometric series 1/d = y (1 + e + e^2 + e^3 + ...) to e^3: the
+// remainder e^4 < 2^-79 leaves the rounding of the last FMA, so the result is within one FP64
+// ulp of 1/d (the GPU unit test measures the largest difference from the correctly rounded
+// 1.0 / d over random and edge values).  An FP64 instruction holds a sub-partition's FP64 unit
+// for 64 cycles: four of them after an 18-cycle approximation, against four and two conversions
+// (104 + 64 cycles) from an FP32 seed.  d outside [2^-100, 2^101) (exponent bits) takes the
+// plain division.
 __device__ __forceinline__ double rcp_pos(double d) {
     const int ex = (__double2hiint(d) >> 20) & 0x7ff;
     if (ex < 1023 - 100 || ex > 1023 + 100) return 1.0 / d;
-    float y0;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(__double2float_rn(d)));
-    double y = (double)y0;
-    y = fma(y, fma(-d, y, 1.0), y);
-    y = fma(y, fma(-d, y, 1.0), y);
-    return y;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+    const double e = fma(-d, y, 1.0);
+    double t = fma(e, e, e);
+    t = fma(t, e, e);
+    return fma(y, t, y);
 }
 
+// 1/d for d > 0 in integer arithmetic (a few cycles per step where FP64 takes 64): with D the
+// 53-bit significand of d as a 64-bit fraction in [1/2, 1) and Y0 the FP32 approximation of 1/D
+// to 31 bits, e = 1 - D Y0 is exact to 82 fractional bits and |e| < 2^-21, and 1/D = Y0 (1 + e +
+// e^2) to e^3 < 2^-63, rounded to the nearest 53 bits: within one FP64 ulp (the GPU unit test
+// measures it against the correctly rounded 1.0 / d).  d outside [2^-100, 2^101) takes the division.
+__device__ __forceinline__ double rcp_pos_int(double d) {
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const int ex = (int)(hi >> 20);
+    if (ex < 1023 - 100 || ex > 1023 + 100) return 1.0 / d;
+    const unsigned Dh = 0x80000000u | (hi << 11) | (lo >> 21), Dl = lo << 11;
+    float y0;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(__uint_as_float(0x3f000000u | ((Dh >> 8) & 0x7fffffu))));
+    const unsigned Y0 = 0x40000000u | ((__float_as_uint(fminf(y0, 1.99999988f)) & 0x7fffffu) << 7);   // 30 fractional bits
+    const unsigned long long Pl = (unsigned long long)Dl * Y0;
+    const unsigned long long Ph = (unsigned long long)Dh * Y0 + (Pl >> 32);
+    const long long A = (long long)(0x4000000000000000ull - Ph);
+    const long long e = (A << 20) - (long long)((unsigned)Pl >> 12);                    // 82 bits
+    const int eh = (int)(e >> 32);                                                      // 50 bits
+    const long long s = e + (((long long)eh * eh) >> 18);                               // e + e^2, 82 bits
+    const long long c = (s >> 32) * (long long)(int)Y0 +
+                        (long long)(((unsigned long long)(unsigned)s * Y0) >> 32);      // Y0 (e + e^2), 80 bits
+    const unsigned long long Y = ((unsigned long long)Y0 << 33) + (unsigned long long)(c >> 17);   // 63 bits
+    unsigned long long R = (Y + 1024) >> 11;                                            // 52 bits
+    if (Dh == 0x80000000u && Dl == 0) R = 1ull << 53;                                   // a power of two: 1/D = 2
+    return __longlong_as_double((long long)(((unsigned long long)(2045 - ex) << 52) + (R - (1ull << 52))));
+}
+
+// Excess attitude noise (Sect. 5.2.5): eps_a^2 of the three components (AL, AC in the
+// preceding field, AC in the following field) per time bucket [t0 + j dt, t0 + (j+1) dt),
+// stored eps2[comp * n_b + j].  eps2 null: off.
 struct AttNoise {
     const double* eps2 = nullptr;
     int64_t t0 = 0, dt = 1;

@@ -196,33 +196,58 @@ __global__ void __launch_bounds__(32 * kAsmWarps) k_att_assemble(int n_seg, int 
 // Robust factorisation of each segment's band (Algorithm C.1 on the envelope, in the
 // square-root-free form N = V' D V with V unit upper triangular: U = sqrt(D) V, the same pivot
 // test on D and the same zeroed rows for a failing pivot) with the forward substitution (C.2)
-// fused, then the back substitution (C.3).  Without the square root the per-row chain that
-// bounds the recurrence (pivot, reciprocal, V_{r,r+1}, the next pivot's update) is about a
-// third as long.  One segment per group of 8 lanes, four per warp.  The 16x16 window W[a][b] = N'[r+a][r+b] (a <= b) of the
-// partly reduced matrix lives in shared memory, addressed by absolute row and column modulo
-// 16, so that moving the window by one row moves no data.  Per row the 120 window entries
-// below the pivot row are updated 15 per lane (every lane the same count, so one FP64
-// instruction of the warp does useful work in all its lanes), and the column that enters
-// the window comes from a ring filled by cp.async kColAhead rows ahead, each lane copying
-// and later consuming the same two entries.  Every entry receives the same FMAs in the
-// same order whatever the lane mapping, and the back substitution sums its 15 products in a
-// fixed tree.  Row r of urow holds 1/D_r and V_{r, r+1..r+15}; yv holds w_r / D_r.
-constexpr int kSegLanes = 8;
-constexpr int kSegsPerWarp = kWarp / kSegLanes;
-constexpr int kSolveSegWarps = 2;
-constexpr int kColAhead = 8;
+// fused, then the back substitution (C.3).  One segment per block of two warps.
+//
+// What bounds it: an FP64 instruction of a warp holds its SM sub-partition's FP64 unit for 64
+// cycles, however many lanes it has active, and takes as long to its result, so a row costs 64
+// cycles for every FP64 instruction that is issued or waited for.  Hence few instructions over
+// full warps, and two warps that work at the same time:
+//   pivot warp   V_{r,.} (one product over the 17 lanes of the pivot row), the next pivot row
+//                ahead of the rest (one FMA), and its reciprocal in integer arithmetic
+//   update warp  the rest of the window: the 136 entries of the 16x16 window of the partly
+//                reduced matrix and its 16 right-hand sides are 152 unordered pairs of slots
+//                (slot = row or column mod 16, 16 = right-hand side), five to a lane, in
+//                registers: the window moves by one row without moving data, because a pair of
+//                slots names one entry (row = early slot, column = late slot) at any time.  Five
+//                FMAs update every pair; the pairs of the pivot's slot then take the column that
+//                enters, from a ring filled by cp.async a knot (four rows) at a time.
+// The pivot row, the row after it and V pass through shared memory, one barrier per row.
+// Every entry receives the FMAs of the plain row-by-row elimination in its order.
+// The back substitution (pivot warp) goes column by column: one FMA and one shuffle per row.
+//
+// Measured: 183 segments of 2988 rows 6.47 -> 1.29 ms (2.0 -> 0.43 us per row), 1827 segments of
+// 11628 rows 26.5 -> 12.4 ms (before: one segment per 8 lanes, the window in shared memory, 15
+// window instructions per row for four segments and an FP64 reciprocal from an FP32 seed).  With
+// an FP64 reciprocal in this layout: 1.40 and 18.2 ms; with one warp for both parts: 2.1 and 13.5 ms.
+constexpr int kColAhead = 16;      // ring slots of incoming columns
+constexpr int kBackRows = 32;      // ring rows of the back substitution
+constexpr int kPairs = 152;        // 136 of the matrix, 16 right-hand sides
+constexpr int kPairSlots = 5;      // pairs per lane
 struct __align__(16) SegWin {
-    double Wf[256];              // W[row mod 16][col mod 16] at row * 16 + (col + row) mod 16 (a
-                                 // diagonal skew: a column's entries fall in distinct banks)
-    double z[16];                // partly reduced right-hand side per row slot
-    double dg[16];               // original diagonal per row slot (the pivot test of C.1)
-    double U[16];                // the current row of V: U[b] = V_{r, r+b} (b >= 1)
-    double xs[16];               // back substitution: x of the rows r+1 .. r+15 by slot
-    double ring[kColAhead][18];  // incoming columns: 16 band values, rhs, pad
-    double pad[8];               // 3776 B: consecutive segments start 64 B apart modulo 128 B,
-                                 // so the two segments of a half warp use disjoint banks
+    union {
+        struct {
+            double ring[kColAhead][16];  // incoming columns: 16 band values
+            double rring[kColAhead];     // and their right-hand sides
+            double A[2][18];             // pivot row by slot (16: right-hand side), alternating
+            double B[2][18];             // the row after it, before this step's update
+            double V[2][18];             // V_{r, .} by slot (16: w_r / D_r)
+            double tdg[32];              // pivot tolerance times the original diagonal, row mod 32
+        } f;
+        struct {
+            double U[kBackRows][16];     // rows of V (entry 0 unused), row mod kBackRows
+            double y[kBackRows];
+        } b;
+    };
 };
-static_assert(sizeof(SegWin) % 128 == 64, "segment windows must alternate between bank halves");
+// order-preserving map of a double (not NaN) to a signed integer: comparing two of these takes a
+// few integer cycles, an FP64 comparison 115
+__device__ __forceinline__ long long ord_bits(double x) {
+    const long long b = __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ bool is_nan_bits(double x) {
+    return ((unsigned long long)__double_as_longlong(x) << 1) > 0xffe0000000000000ull;
+}
 
 __device__ __forceinline__ void cp_async16_att(void* smem, const void* gmem) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
@@ -238,174 +263,194 @@ __device__ __forceinline__ void cp_async_wait_att() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
-__device__ __forceinline__ double& win(SegWin& sm, int row, int col) {
-    return sm.Wf[row * 16 + ((col + row) & 15)];
-}
-
-__global__ void __launch_bounds__(32 * kSolveSegWarps) k_att_solve(int n_seg, const int64_t* __restrict__ seg_row,
+__device__ __forceinline__ void seg_barrier() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
+__global__ void __launch_bounds__(64) k_att_solve(int n_seg, const int64_t* __restrict__ seg_row,
                                                   const double* __restrict__ bandc, const double* __restrict__ rhs,
                                                   double* __restrict__ urow, double* __restrict__ yv,
                                                   double* __restrict__ x, double tol, int* __restrict__ seg_rd) {
-    __shared__ SegWin win_all[kSolveSegWarps][kSegsPerWarp];
+    __shared__ SegWin sm;
     const int lane = threadIdx.x & 31;
-    const int wib = threadIdx.x >> 5;
-    const int grp = lane / kSegLanes;
-    const int sub = lane % kSegLanes;
-    const unsigned gmask = ((1u << kSegLanes) - 1u) << (grp * kSegLanes);
-    SegWin& sm = win_all[wib][grp];
-    const int sg = (blockIdx.x * kSolveSegWarps + wib) * kSegsPerWarp + grp;
-    const bool seg_ok = sg < n_seg;
-    const int64_t base = seg_ok ? seg_row[sg] : 0;
-    const int64_t n = seg_ok ? seg_row[sg + 1] - base : 0;
-    int64_t n_max = n;
-#pragma unroll
-    for (int o = kSegLanes; o < kWarp; o <<= 1) {
-        const int64_t v = __shfl_xor_sync(0xffffffffu, n_max, o);
-        n_max = v > n_max ? v : n_max;
+    // the update warp issues five FP64 instructions per row, the pivot warp two: which warp of the
+    // block is which alternates between waves of two blocks per SM, so that the SM's sub-partitions
+    // carry both (1827 segments: 12.4 ms, 14.4 without)
+    const bool pivot_warp = ((threadIdx.x >> 5) ^ ((blockIdx.x / (2 * 152)) & 1)) == 0;
+    const int sg = blockIdx.x;
+    const int64_t base = seg_row[sg];
+    const int n = (int)(seg_row[sg + 1] - base);
+    const double* bc = bandc + base * 16;
+    const double* rh = rhs + base;
+    double* ur = urow + base * 16;
+    double* yr = yv + base;
+    // pivot row 0 and row 1 by slot, right-hand side at 16, zero at 17
+    if (threadIdx.x < 18) {
+        sm.f.A[0][lane] = lane < 16 ? bc[(int64_t)lane * 16 + lane] : lane == 16 ? rh[0] : 0.0;
+        sm.f.B[0][lane] = lane >= 1 && lane < 16 ? bc[(int64_t)lane * 16 + lane - 1] : lane == 16 ? rh[1] : 0.0;
+        sm.f.A[1][lane] = sm.f.B[1][lane] = sm.f.V[0][lane] = sm.f.V[1][lane] = 0.0;
+        if (lane < 16) sm.f.tdg[lane] = tol * bc[(int64_t)lane * 16];
     }
-    if (n_max == 0) return;
-    // this lane's 15 window entries per row, (a, b) with 1 <= a <= b <= 15 in row-major
-    // order: pair p = 8 t + sub (the a = 1 row, which the next pivot needs, comes first)
-    int pa[15], pb[15];
+    __syncthreads();
+    if (pivot_warp) {
+        int rd = 0;
+        // 1 / D_r for the pivot of row r; a failing pivot zeroes the row (rank defect)
+        auto pivot_inverse = [&](double piv, double td) -> double {
+            const bool pos = ord_bits(piv) > ord_bits(td) && !is_nan_bits(piv) && !is_nan_bits(td);
+            rd += !pos;
+            const double y = rcp_pos_int(piv);
+            return pos && __double_as_longlong(piv) > 0 ? y : 0.0;
+        };
+        double invd = pivot_inverse(sm.f.A[0][0], sm.f.tdg[0]);
+        const int l17 = lane < 17 ? lane : 17;
+        double a0 = sm.f.A[0][l17];   // the pivot row (lane = slot; 16: right-hand side)
+        double* up = ur;
+        for (int r0 = 0; r0 < n; r0 += 4) {
 #pragma unroll
-    for (int t = 0; t < 15; t++) {
-        int p = kSegLanes * t + sub, a = 1;
-        while (p >= 16 - a) { p -= 16 - a; a++; }
-        pa[t] = a;
-        pb[t] = a + p;
-    }
-    // initial window: rows and columns 0..15 (lane sub loads columns 2 sub and 2 sub + 1)
-#pragma unroll
-    for (int h = 0; h < 2; h++) {
-        const int b = 2 * sub + h;
-        for (int a = 0; a < 16; a++)
-            win(sm, a, b) = (a <= b && b < n) ? bandc[(base + b) * 16 + (b - a)] : 0.0;
-        sm.dg[b] = b < n ? bandc[(base + b) * 16] : 0.0;
-        sm.z[b] = b < n ? rhs[base + b] : 0.0;
-    }
-    // the columns 16 .. 16 + kColAhead - 1 into the ring (lane sub: band entries 2 sub, 2 sub + 1;
-    // lane 0 also the right-hand side)
-#pragma unroll
-    for (int q = 0; q < kColAhead; q++) {
-        const int64_t c = 16 + q;
-        if (c < n) {
-            cp_async16_att(&sm.ring[q][2 * sub], bandc + (base + c) * 16 + 2 * sub);
-            if (sub == 0) cp_async8_att(&sm.ring[q][16], rhs + base + c);
+            for (int h = 0; h < 4; h++) {
+                const int r = r0 + h, s0 = r & 15, s1 = (r + 1) & 15;
+                // V_{r, .} = W[0][.] / D_r and w_r / D_r
+                const double v = invd * a0;
+                if (lane < 17) sm.f.V[h & 1][lane] = v;
+                const double v1 = __shfl_sync(0xffffffffu, v, s1);
+                seg_barrier();   // V_r is out; row r + 1 (before this step's update) and column r + 16 are in
+                const double* col = sm.f.ring[(r + 16) % kColAhead];
+                const double b0 = sm.f.B[h & 1][l17];
+                const double c15 = col[15], c0 = col[0], td = sm.f.tdg[(r + 1) & 31];
+                // look ahead: the next pivot row, complete (lane s0: the entry of the column that enters)
+                a0 = lane == s0 ? c15 : fma(-v1, a0, b0);
+                const double piv = __shfl_sync(0xffffffffu, a0, s1);
+                if (lane < 17) sm.f.A[(h + 1) & 1][lane] = a0;
+                if (lane < 16) up[h * 16 + ((lane - s0) & 15)] = v;
+                else if (lane == 16) yr[r] = v;
+                else if (lane == 17) sm.f.tdg[(r + 16) & 31] = tol * c0;
+                if (r + 1 < n) invd = pivot_inverse(piv, td);
+            }
+            up += 64;
         }
-        cp_async_commit_att();
-    }
-    __syncwarp();
-    int rd = 0;
-    for (int64_t r = 0; r < n_max; r++) {
-        const bool live = r < n;
-        const int s0 = (int)(r & 15);
-        const double piv = win(sm, s0, s0);
-        const double dg0 = sm.dg[s0];
-        // the pivot test of Algorithm C.1; a failing pivot zeroes the row (rank defect)
-        const bool pos = piv > tol * dg0;
-        const double invd = (pos && piv > 0.0) ? rcp_pos(piv) : 0.0;
-        if (live) rd += !pos;
-        const double wr = sm.z[s0];
-        const double yr = wr * invd;
-        // V_{r, r+b} = W[0][b] / D_r and the forward substitution z_b -= V_b w_r, b = sub + 1, sub + 9
+        if (lane == 0) seg_rd[sg] = rd;
+        seg_barrier();
+    } else {
+        // this lane's pairs by early slot and late slot of the rows in the window, as byte offsets into
+        // a row by slot, and their entries of the first window.  Pairs 0-135 are the matrix's (four for
+        // every lane and a fifth in lanes 0-7), the right-hand sides of slots 0-15 are the fifth of
+        // lanes 8-23 (late slot 16)
+        int oe[kPairSlots], ol[kPairSlots];
+        double e[kPairSlots];
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int b = sub + 1 + kSegLanes * h;
-            if (b <= 15) {
-                const int sb = (int)((r + b) & 15);
-                double v = win(sm, s0, sb) * invd;
-                if (r + b >= n) v = 0.0;
-                sm.U[b] = v;
-                sm.z[sb] -= v * wr;
+        for (int t = 0; t < kPairSlots; t++) {
+            int k = lane + kWarp * t, p = 0;
+            oe[t] = ol[t] = 8 * 17;   // no pair: an entry that nothing uses
+            e[t] = 0.0;
+            if (k < 136) {
+                while (k >= 16 - p) { k -= 16 - p; p++; }
+                oe[t] = 8 * p;
+                ol[t] = 8 * (p + k);
+                e[t] = bc[(int64_t)(p + k) * 16 + k];   // n >= 16: a segment has 4 knots or more
+            } else if (k < kPairs) {
+                oe[t] = 8 * (k - 136);
+                ol[t] = 8 * 16;
+                e[t] = rh[k - 136];
             }
         }
-        __syncwarp(gmask);
-        if (live) {
-            const double v0 = sub == 0 ? invd : sm.U[2 * sub];
-            *reinterpret_cast<double2*>(urow + (base + r) * 16 + 2 * sub) = make_double2(v0, sm.U[2 * sub + 1]);
-            if (sub == 0) yv[base + r] = yr;
-        }
-        // the window below the pivot row: W[a][b] -= V_a W[0][b] (= W[0][a] W[0][b] / D_r);
-        // row r's slot is not written in this step.  All 45 operands are loaded before the
-        // first product and the 15 results stored after the last, so that the loads of one
-        // entry do not wait for the store of another.
-        {
-            int adr[15];
-            double wv[15], uv[15], pv[15];
-#pragma unroll
-            for (int t = 0; t < 15; t++) {
-                const int ra = (int)((r + pa[t]) & 15), sb = (int)((r + pb[t]) & 15);
-                adr[t] = ra * 16 + ((sb + ra) & 15);
-                wv[t] = sm.Wf[adr[t]];
-                pv[t] = sm.Wf[s0 * 16 + ((sb + s0) & 15)];
-                uv[t] = sm.U[pa[t]];
+        const bool z_lane = lane >= 8 && lane < 24;
+        // the four columns of a knot (c a multiple of 4) into ring slots c mod kColAhead ..: a lane
+        // copies 16 bytes of the 512, lanes 0 and 1 also 16 of the right-hand sides; zeros beyond the
+        // segment (whose length is a multiple of 4)
+        auto fetch = [&](int c) {
+            double* slot = &sm.f.ring[c % kColAhead][0] + 2 * lane;
+            double* rslot = &sm.f.rring[c % kColAhead] + 2 * lane;
+            if (c < n) {
+                cp_async16_att(slot, bc + (int64_t)c * 16 + 2 * lane);
+                if (lane < 2) cp_async16_att(rslot, rh + c + 2 * lane);
+            } else {
+                slot[0] = slot[1] = 0.0;
+                if (lane < 2) rslot[0] = rslot[1] = 0.0;
             }
+            cp_async_commit_att();
+        };
+        constexpr int kKnotsAhead = kColAhead / 4 - 1;
 #pragma unroll
-            for (int t = 0; t < 15; t++) wv[t] -= uv[t] * pv[t];
+        for (int q = 0; q < kKnotsAhead; q++) fetch(16 + 4 * q);
+        for (int r0 = 0; r0 < n; r0 += 4) {
+            cp_async_wait_att<kKnotsAhead - 1>();   // the columns r0 + 16 .. r0 + 19 have arrived
 #pragma unroll
-            for (int t = 0; t < 15; t++) sm.Wf[adr[t]] = wv[t];
-        }
-        // the column r + 16 enters in the slot of column r (row r's entries are no longer read)
-        cp_async_wait_att<kColAhead - 1>();
-        const int64_t c = r + 16;
-        const int q = (int)(r % kColAhead);
+            for (int h = 0; h < 4; h++) {
+                const int r = r0 + h, s0 = r & 15, s2 = (r + 2) & 15;
+                seg_barrier();   // V_r and the pivot row are in; row r + 1 is out
+                // the slots of the columns taken in the previous four steps are free
+                if (h == 0) fetch(r0 + 12 + kColAhead);
+                const char* A0 = (const char*)sm.f.A[h & 1];
+                const char* V0 = (const char*)sm.f.V[h & 1];
+                const char* col = (const char*)sm.f.ring[(r + 16) % kColAhead];
+                // pairs of the other slots: W[a][b] -= V_a W[0][b]; pairs of slot s0 (their early one): the
+                // entering column r + 16 (band entry N[c - k][c] or the right-hand side), the late slot of its pairs
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int k = 2 * sub + h;   // band entry N[c - k][c]: window row a = 15 - k
-            const int a = 15 - k;
-            win(sm, (int)((r + 1 + a) & 15), s0) = c < n ? sm.ring[q][k] : 0.0;
+                for (int t = 0; t < kPairSlots; t++) {
+                    const double ve = *(const double*)(V0 + oe[t]);
+                    const double wl = *(const double*)(A0 + ol[t]);
+                    const bool mine = oe[t] == 8 * s0;
+                    const char* src = col + ((8 * s0 - ol[t]) & 120);
+                    if (t == 4) src = z_lane ? (const char*)&sm.f.rring[(r + 16) % kColAhead] : src;
+                    const double in = *(const double*)src;
+                    const double upd = fma(-ve, wl, e[t]);
+                    e[t] = mine ? in : upd;
+                    const bool turn = t == 4 ? mine && !z_lane : mine;
+                    oe[t] = turn ? ol[t] : oe[t];
+                    ol[t] = turn ? 8 * s0 : ol[t];
+                }
+                // publish row r + 2 for the next look-ahead: its slot is the early one of its pairs
+                char* B1 = (char*)sm.f.B[(h + 1) & 1];
+#pragma unroll
+                for (int t = 0; t < kPairSlots; t++)
+                    if (oe[t] == 8 * s2) *(double*)(B1 + ol[t]) = e[t];
+            }
         }
-        if (sub == 0) {
-            sm.dg[s0] = c < n ? sm.ring[q][0] : 0.0;
-            sm.z[s0] = c < n ? sm.ring[q][16] : 0.0;
-        }
-        __syncwarp(gmask);
-        // refill the ring slot (read above by this lane only) with the column kColAhead on
-        const int64_t cn = c + kColAhead;
-        if (cn < n) {
-            cp_async16_att(&sm.ring[q][2 * sub], bandc + (base + cn) * 16 + 2 * sub);
-            if (sub == 0) cp_async8_att(&sm.ring[q][16], rhs + base + cn);
-        }
-        cp_async_commit_att();
+        cp_async_wait_att<0>();
+        seg_barrier();
+        return;
     }
     cp_async_wait_att<0>();
-    // back substitution: x_r = y_r - sum_k V_{r,r+k} x_{r+k}, k = 1..15, y_r = w_r / D_r; lane
-    // sub forms the products k = sub and sub + 8 and the group adds them in a fixed tree
-    for (int k = 0; k < 16; k++)
-        if (sub == 0) sm.xs[k] = 0.0;
     __syncwarp();
-    // the row's V entries and y are loaded one row ahead (they do not depend on the x chain)
-    double u_lo = 0.0, u_hi = 0.0, y_r = 0.0;
-    if (n - 1 >= 0) {
-        const double* ur = urow + (base + n - 1) * 16;
-        u_lo = ur[sub];
-        u_hi = ur[sub + 8];
-        y_r = yv[base + n - 1];
-    }
-    for (int64_t kk = 0; kk < n_max; kk++) {
-        const int64_t r = n - 1 - kk;
-        const bool live = r >= 0;
-        const double c_lo = u_lo, c_hi = u_hi, c_y = y_r;
-        if (r - 1 >= 0) {
-            const double* un = urow + (base + r - 1) * 16;
-            u_lo = un[sub];
-            u_hi = un[sub + 8];
-            y_r = yv[base + r - 1];
+    // back substitution x_r = y_r - sum_k V_{r,r+k} x_{r+k}, column by column: lane j < 16 keeps the
+    // partial sum of the row i = j mod 16 among the 16 rows at or below r; once x_r is known it is
+    // broadcast and every pending row subtracts its product (one FMA per row and step).  Rows are
+    // fetched a knot (four rows) at a time.
+    auto fetch_rows = [&](int i) {   // i a multiple of 4
+        if (i >= 0) {
+            cp_async16_att(&sm.b.U[i % kBackRows][0] + 2 * lane, ur + (int64_t)i * 16 + 2 * lane);
+            if (lane < 2) cp_async16_att(&sm.b.y[i % kBackRows] + 2 * lane, yr + i + 2 * lane);
         }
-        const double p_lo = (live && sub >= 1) ? c_lo * sm.xs[(r + sub) & 15] : 0.0;
-        const double p_hi = live ? c_hi * sm.xs[(r + sub + 8) & 15] : 0.0;
-        double part = p_lo + p_hi;
+        cp_async_commit_att();
+    };
+    constexpr int kBackAhead = kBackRows / 4 - 5;   // knots fetched beyond the five that a step reads
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o, kSegLanes);
-        const double xr = live ? c_y - part : 0.0;
-        __syncwarp(gmask);
-        if (live && sub == 0) {
-            x[base + r] = xr;
-            sm.xs[r & 15] = xr;
+    for (int q = 1; q <= 4 + kBackAhead; q++) fetch_rows(n - 4 * q);
+    cp_async_wait_att<kBackAhead>();
+    __syncwarp();
+    const int j = lane & 15;
+    double acc = sm.b.y[(n - 16 + ((j - (n - 16)) & 15)) % kBackRows];   // rows n-16 .. n-1 by slot
+    double* xo = x + base;
+    for (int r0 = n - 4; r0 >= 0; r0 -= 4) {
+        cp_async_wait_att<kBackAhead - 1>();   // the rows r0 - 16 .. r0 - 13 have arrived
+        __syncwarp();
+        double u[4], yn[4];
+#pragma unroll
+        for (int h = 3; h >= 0; h--) {
+            const int r = r0 + h, k = (r - j) & 15, i = r - k;
+            u[h] = i >= 0 ? sm.b.U[i & (kBackRows - 1)][k] : 0.0;
+            yn[h] = r >= 16 ? sm.b.y[(r - 16) & (kBackRows - 1)] : 0.0;
         }
-        __syncwarp(gmask);
+#pragma unroll
+        for (int h = 3; h >= 0; h--) {
+            const int r = r0 + h;
+            const double xr = __shfl_sync(0xffffffffu, acc, r & 15);
+            const bool mine = j == (r & 15);
+            if (lane == (r & 15)) xo[r] = xr;
+            const double upd = fma(-u[h], xr, acc);
+            acc = mine ? yn[h] : upd;
+        }
+        fetch_rows(r0 - 16 - 4 * kBackAhead);
     }
-    if (sub == 0 && seg_ok) seg_rd[sg] = rd;
+    cp_async_wait_att<0>();
+
 }
 
 // a_n += x for the coefficients each segment owns (n in [u_lo, u_hi]); one thread per
@@ -454,9 +499,7 @@ void launch_att_solve(int n_seg, int max_seg_knots, int n_coef, int64_t n_rows, 
     if (blocks > 152 * 16) blocks = 152 * 16;
     if (blocks < 1) blocks = 1;
     k_att_assemble<<<blocks, 32 * kAsmWarps, 0, s>>>(n_seg, runs_per_seg, seg_row, seg_l, seg_n, blk, bandc, rhs);
-    const int seg_warps = (n_seg + kSegsPerWarp - 1) / kSegsPerWarp;
-    k_att_solve<<<(seg_warps + kSolveSegWarps - 1) / kSolveSegWarps, 32 * kSolveSegWarps, 0, s>>>(
-        n_seg, seg_row, bandc, rhs, urow, yv, x, tol, seg_rd);
+    k_att_solve<<<n_seg, 64, 0, s>>>(n_seg, seg_row, bandc, rhs, urow, yv, x, tol, seg_rd);
     k_att_apply<<<(n_coef + 255) / 256, 256, 0, s>>>(n_coef, n_seg, seg_u, seg_n, seg_row, x, att, d_att, dx);
 }
 
