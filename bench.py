@@ -33,14 +33,15 @@ WORKLOADS = {
     "uneven5yr": "3M sources, 5 yr, 30-s knots, G ~ U(12, 18) with sigma_AL 50-500 uas, 40-250 transits",
 }
 # kernels launched by one iteration, (with a full FP64 evaluation, with the linearized pass):
-# FP64 form: S (source geometry, observation pass, per-source solve, stats in two stages,
-# update-history push), A (accumulate, assemble, solve, apply, rank-defect sum), C
+# FP64 form: S (source geometry, observation pass, first sums, 5 rounds of 5x5 algebra, 4 rounds
+# of sums, final pass, per-observation path, stats in two stages, update-history push) = 17, A
+# (accumulate, assemble, solve, apply, rank-defect sum), C
 # (accumulate, project, rank-defect sum), frame (normals, solve, apply sources, apply
-# attitude) = 18.  Mixed form: the S pass is source geometry + full evaluation, or the one
+# attitude) = 29.  Mixed form: the S pass is source geometry + full evaluation, or the one
 # linearized-correction kernel; the S solves are scale/round-0 sums, 5 rounds of 5x5 algebra,
 # 4 rounds of sums, final pass, per-observation path, stats (two), history push = 15 (default
 # 4 reweighting rounds); A, C and frame as above.
-KERNELS_PER_STEP = {"fp64": (18, 18), "mixed": (2 + 15 + 12, 1 + 15 + 12)}
+KERNELS_PER_STEP = {"fp64": (29, 29), "mixed": (2 + 15 + 12, 1 + 15 + 12)}
 # with the excess attitude noise on: x values, per-bucket selection, attitude weights
 KERNELS_ATTNOISE = 3
 FALLBACK_HBM_GBS = 6800.0
@@ -50,7 +51,7 @@ MIX_PASS_BYTES = 8 + 16 + 4 + 8 + 8
 # of 2.47e7 observations, scaled per observation; profiles/k_*_kernels_30k.md): the S block of
 # the FP64 form (observation pass + solves) and the mixed form's linearized pass.  None once
 # the kernel has changed since its capture.
-TRAFFIC_PER_OBS = {"fp64_s_block": 780.0, "mixed_correct": 47.6}
+TRAFFIC_PER_OBS = {"fp64_s_block": None, "mixed_correct": 47.6}
 
 
 def parse():

@@ -438,8 +438,8 @@ int agis_solve_exchange(agis_ctx* ctx, int32_t which, agis_block_stats* out, dou
  *   AGIS_KNOB_OBS_PASS    observation pass (FP64 model in the FP64 form, the linearized
  *                         correction in the mixed form): a threads per block (128, 256),
  *                         b blocks per SM of the grid-stride grid (1..64)
- *   AGIS_KNOB_SRC_BATCH   FP64 form, per-source solves: a sources per work fetch of the
- *                         persistent kernel (1..32; 0: n_src / 2432 within 1..32); b unused
+ *   AGIS_KNOB_SRC_BATCH   FP64 form, passes of the per-source solves: a consecutive sources per
+ *                         warp and grid-stride step (1..32; 0: one); b unused
  *   AGIS_KNOB_MIX_SUMS    mixed form, S-block sums and final pass: a warps per block
  *                         (2, 4, 8), b blocks per SM (1..64)
  *   AGIS_KNOB_MIX_SOLVE5  mixed form, 5x5 solves (a thread per source): a threads per block

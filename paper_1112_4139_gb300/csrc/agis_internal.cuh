@@ -195,6 +195,18 @@ struct SrcOutPtrs {
     int* rankdef;
 };
 
+// Per-source state of the FP64 S block between its kernels (class-sum path).
+struct __align__(16) SrcWork {
+    double T[2][21];   // unit-weight sums per class: 15 AA, 5 Ah, hh
+    double C[2][21];   // what the round's weights take off: sums of (1 - w) times the same products
+    double s2c[2];     // sigma^2 of the AL and AC observations (one value per class)
+    double s2min, vs;  // smallest sigma^2; robust scale of x = h / sigma
+    double d[5];       // solution of the latest round
+    double isd[2];     // 1 / sqrt(sigma_c^2 + eps^2); after the last round 1 / (sigma_c^2 + eps^2)
+    int32_t flags;     // 1: one sigma per class, 2: no observations, 0: the general path
+    int32_t nout;      // observations with w < 0.2
+};
+
 struct Settings {
     int robust, n_rounds, n_eps, weight_fn;
     double lambda2;
@@ -208,7 +220,7 @@ struct Settings {
 // arithmetic whatever the shape, so the results do not depend on them.
 struct Shapes {
     int obs_threads = 256, obs_bps = 64;  // observation pass: threads per block, blocks per SM (grid cap)
-    int src_batch = 0;                    // FP64 S solves: sources per work fetch (0: n_src / 2432 in 1..32)
+    int src_batch = 0;                    // FP64 S passes: sources per warp and step (0: one)
     int sums_warps = 4, sums_bps = 16;    // mixed S sums and final pass: warps per block, blocks per SM
     int solve5_threads = 128;             // mixed 5x5 solves: threads per block
     int att_bps = 0;                      // A accumulation: blocks per SM (0: 32 FP64 form, 64 mixed form)
@@ -269,23 +281,21 @@ __device__ __forceinline__ double dkey_inv(uint64_t k) {
     return __longlong_as_double(b);
 }
 
-// 1/d for d > 0 from rcp.approx.ftz.f64, whose relative error e = 1 - d y is below 1.0e-6
-// (measured over [1, 4)), by the geometric series 1/d = y (1 + e + e^2 + e^3 + ...) to e^3: the
-// remainder e^4 < 2^-79 leaves the rounding of the last FMA, so the result is within one FP64
-// ulp of 1/d (the GPU unit test measures the largest difference from the correctly rounded
-// 1.0 / d over random and edge values).  An FP64 instruction holds a sub-partition's FP64 unit
-// for 64 cycles: four of them after an 18-cycle approximation, against four and two conversions
-// (104 + 64 cycles) from an FP32 seed.  d outside [2^-100, 2^101) (exponent bits) takes the
-// plain division.
+// 1/d for d > 0 by Newton's iteration for the reciprocal, y <- y + y (1 - d y), two steps from
+// rcp.approx.ftz.f64, whose relative error is below 1.0e-6 (measured over [1, 4)): e0 becomes
+// e0^2 after one step and e0^4 < 2^-79 after two, so the result differs from 1/d by the rounding
+// of the last FMA: at most one FP64 ulp (the GPU unit test measures the largest difference from
+// the correctly rounded 1.0 / d over random and edge values).  An FP64 instruction holds a
+// sub-partition's FP64 unit for 64 cycles: four of them after an 18-cycle approximation, against
+// four and two conversions (104 + 64 cycles) from an FP32 seed.  d outside [2^-100, 2^101)
+// (exponent bits) takes the plain division.
 __device__ __forceinline__ double rcp_pos(double d) {
     const int ex = (__double2hiint(d) >> 20) & 0x7ff;
     if (ex < 1023 - 100 || ex > 1023 + 100) return 1.0 / d;
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-    const double e = fma(-d, y, 1.0);
-    double t = fma(e, e, e);
-    t = fma(t, e, e);
-    return fma(y, t, y);
+    y = fma(y, fma(-d, y, 1.0), y);
+    return fma(y, fma(-d, y, 1.0), y);
 }
 
 // 1/d for d > 0 in integer arithmetic (a few cycles per step where FP64 takes 64): with D the

@@ -1,12 +1,27 @@
 // k_source.cu -- the observation pass in source order and the S block (Sect. 5.1).
 //
-// One warp per source (persistent warps take sources from a work counter, largest first).
-// The warp evaluates every observation of the source once (residual h_l, design row A_l,
-// attitude partial g_l), keeps (h, A, w, sigma^2) in a per-warp scratch slice that stays in
-// L2 during the inner iteration, and runs the inner iteration of Sect. 5.1.2 with
-// butterfly (xor-shuffle) reductions, so every lane holds the same 5x5 system and solves it
-// redundantly.  At the end it writes the hand-over record (t, R = h - A d, W, g, meta) that
-// the time-ordered attitude pass and the calibration pass gather.
+// The observation pass (one thread per observation) leaves residual h, design row A and sigma^2
+// in a 64-byte scratch row.  The inner iteration of Sect. 5.1.2 then runs as passes over the
+// rows (one warp per source, largest first) and 5x5 solves (one thread per source) in turn:
+//   k_src_first   sigma per class, robust scale and round 0's class sums
+//   k_src_solve5  the 5x5 algebra of the excess-noise steps
+//   k_src_round   the next round's class sums, and the weights of the last round
+//   k_src_final   the hand-over records (t, R = h - A d, W, g, meta) that the time-ordered
+//                 attitude pass and the calibration pass gather
+//   k_src_general sources whose sigma differs within a class: all rounds in one warp
+//
+// What bounds it: FP64 issue (2 FMA per clock and SM).  A 5x5 solve of one lane costs a warp as
+// many FP64 cycles as 32 of them, hence a thread per source there.  Downweighting leaves w = 1
+// wherever |z| <= 2 (Eqs. dw, dwH), about 95% of the observations, so for long sources the 21
+// products of a row are summed once, with unit weights; a round evaluates z in FP32 (with a bound
+// on its error), and only the rows that may exceed 2 are gathered, 32 to a warp, for the FP64
+// weight and the 27 products that (1 - w) takes off again: a round then costs about a fifth of
+// the FP64 work of the direct sums.
+// Measured, source solves of the S block: 24.7M observations of 30,000 sources 14.2 -> 4.5 ms (9.9
+// with direct sums), 0.5M of 3000 sources 1.68 -> 0.7 ms (direct sums).  Before, one persistent
+// kernel ran all rounds of a batch of sources in a warp, with the 5x5 solves in one lane each.
+#include <type_traits>
+
 #include "agis_internal.cuh"
 
 namespace agis {
@@ -163,103 +178,6 @@ __device__ __forceinline__ void pass_q(const double* scr, int n, int lane, const
     S2 = warp_sum(s);
 }
 
-// Weight of one row in the class-sum path.  mode 0 (initial downweighting): w = wfun(x / vs)
-// with x = h / sigma_c, evaluated as h * rx with rx = 1 / (sigma_c vs) (rx = 0: vs = 0, w = 1);
-// mode 1 (later rounds): w = wfun(R / sqrt(sigma_c^2 + y_prev)) with R = h - A d_prev; mode 2
-// (plain weights): w = 1.
-__device__ __forceinline__ double class_w(int mode, double h, const double* A, const double* dp, double rx,
-                                          double inv_sd, int wfn) {
-    if (mode == 2) return 1.0;
-    if (mode == 0) return rx > 0.0 ? wfun(h * rx, wfn) : 1.0;
-    double Ad = A[0] * dp[0];
-    Ad = fma(A[1], dp[1], Ad);
-    Ad = fma(A[2], dp[2], Ad);
-    Ad = fma(A[3], dp[3], Ad);
-    Ad = fma(A[4], dp[4], Ad);
-    return wfun((h - Ad) * inv_sd, wfn);
-}
-
-// Per-class inputs of one round of a source: sigma_c, rx = 1 / (sigma_c vs), 1 / sqrt(s2_c + y)
-struct RoundIn {
-    double rx[2], isd[2];
-};
-__device__ __forceinline__ RoundIn round_in(const double* s2c, double y, double vs) {
-    RoundIn r;
-#pragma unroll
-    for (int c = 0; c < 2; c++) {
-        const double sig = sqrt(s2c[c]);
-        r.rx[c] = vs > 0.0 ? 1.0 / (sig * vs) : 0.0;
-        r.isd[c] = 1.0 / sqrt(s2c[c] + y);
-    }
-    return r;
-}
-
-// Lane partial sums of one class over its contiguous range [lo, hi) of the source's rows (AL
-// rows come first), with the weights of class_w, written to column `lane` of the warp's
-// reduction buffer red[21][kRedStride] (15 AA, 5 Ah, hh); the last round (store) keeps w in
-// the scratch row for the hand-over records.
-constexpr int kRedVals = 42;      // both classes
-constexpr int kRedStride = 33;    // doubles per value row (odd: the column sums read distinct banks)
-__device__ __forceinline__ void pass_class1(double* scr, int lo, int hi, int lane, int mode, double rx,
-                                            const double* dp, double inv_sd, int wfn, bool store, double* red,
-                                            int& nout) {
-    double AA[15], Ah[5];
-#pragma unroll
-    for (int i = 0; i < 15; i++) AA[i] = 0.0;
-#pragma unroll
-    for (int i = 0; i < 5; i++) Ah[i] = 0.0;
-    double hs = 0.0;
-    int cnt = 0;
-    for (int j = lo + lane; j < hi; j += kWarp) {
-        double* e = scr + (size_t)j * kScr;
-        const double h = e[0];
-        const double A[5] = {e[1], e[2], e[3], e[4], e[5]};
-        const double w = class_w(mode, h, A, dp, rx, inv_sd, wfn);
-        if (store) e[6] = w;
-        cnt += (w < 0.2);
-#pragma unroll
-        for (int a = 0; a < 5; a++) {
-            const double wa = w * A[a];
-#pragma unroll
-            for (int b = a; b < 5; b++) AA[up5(a, b)] += wa * A[b];
-            Ah[a] += wa * h;
-        }
-        hs += w * h * h;
-    }
-#pragma unroll
-    for (int i = 0; i < 15; i++) red[i * kRedStride + lane] = AA[i];
-#pragma unroll
-    for (int i = 0; i < 5; i++) red[(15 + i) * kRedStride + lane] = Ah[i];
-    red[20 * kRedStride + lane] = hs;
-    nout = warp_sum_int(cnt);
-}
-
-// both classes: the 42 lane partials go to the warp's reduction buffer, and lane v adds the
-// 32 partials of value v in lane order (31 additions per value instead of 5 per value in every
-// lane for butterflies); the sums go to the warp's shared-memory slot S, so that they do not
-// occupy registers during the 5x5 algebra
-__device__ __forceinline__ void pass_class(double* scr, int n, int nal, int lane, int mode, const RoundIn& ri,
-                                           const double* dp, int wfn, bool store, ClassSums& S, int& nout,
-                                           double* red) {
-    int nc[2];
-    for (int c = 0; c < 2; c++)
-        pass_class1(scr, c ? nal : 0, c ? n : nal, lane, mode, ri.rx[c], dp, ri.isd[c], wfn, store,
-                    red + c * 21 * kRedStride, nc[c]);
-    __syncwarp();
-    for (int v = lane; v < kRedVals; v += kWarp) {
-        const double* col = red + v * kRedStride;
-        double t = col[0];
-#pragma unroll
-        for (int k = 1; k < kWarp; k++) t += col[k];
-        const int c = v / 21, i = v % 21;
-        if (i < 15) S.AA[c][i] = t;
-        else if (i < 20) S.Ah[c][i - 15] = t;
-        else S.hh[c] = t;
-    }
-    __syncwarp();
-    nout = nc[0] + nc[1];
-}
-
 // Per-source geometry for the observation pass: p, q, r (Eq. normal-triad), parameters, cos(delta).
 __global__ void k_src_geo(int32_t n_src, const double* __restrict__ src, double* __restrict__ geo) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_src; i += gridDim.x * blockDim.x) {
@@ -396,203 +314,695 @@ __device__ __noinline__ void solve_general(const Settings& st, int i, int64_t o0
     __syncwarp();
 }
 
-// Per-source solve, batched: a warp takes `batch` consecutive sources of the largest-first
-// order.  The warp sweeps each source's observations cooperatively (robust sigma, per-class
-// sums, hand-over records); lane k keeps source k's state and class sums, so the 5x5
-// algebra of the excess-noise steps runs for the whole batch in parallel instead of
-// redundantly in every lane.  Sources whose observations do not have one sigma per class use
-// the general per-observation path.
-constexpr int kSolveWarps = 2;
-__global__ void __launch_bounds__(32 * kSolveWarps, 1) k_source_solve(
-    Settings st, const uint32_t* __restrict__ meta, const int64_t* __restrict__ src_off,
-    const int32_t* __restrict__ src_nal, const int32_t* __restrict__ src_order, int32_t n_src, int batch,
-    SrcOutPtrs out, ObsRec* __restrict__ rec, double* __restrict__ scratch, const uint64_t* __restrict__ skey,
-    int* work_counter) {
-    __shared__ int hist_all[kSolveWarps * 256];
-    __shared__ ClassSums sums_all[kSolveWarps][kWarp];
-    __shared__ double red_all[kSolveWarps][kRedVals * kRedStride];
-    const int lane = threadIdx.x & 31;
-    const int wib = threadIdx.x >> 5;
-    int* hist = hist_all + wib * 256;
-    ClassSums* sums = sums_all[wib];
-    double* red = red_all[wib];
-    const int rounds = st.robust ? st.n_rounds + 1 : 1;
-    for (;;) {
-        int base = 0;
-        if (lane == 0) base = atomicAdd(work_counter, batch);
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (base >= n_src) break;
-        const int nb = min(batch, n_src - base);
-        // ---- this lane's source
-        const bool mine = lane < nb;
-        const int my_i = mine ? src_order[base + lane] : 0;
-        const int64_t my_o0 = mine ? src_off[my_i] : 0;
-        const int my_n = mine ? (int)(src_off[my_i + 1] - my_o0) : 0;
-        const int my_nal = mine ? src_nal[my_i] : 0;
-        double s5[5] = {0, 0, 0, 0, 0};
-        if (mine)
-            for (int k = 0; k < 5; k++) s5[k] = out.src[5 * (size_t)my_i + k];
-        const double cosd = cos(s5[1]);
-        double my_s2c[2] = {1.0, 1.0}, my_s2min = 1.0, my_vs = 0.0;
-        bool my_uniform = false;
-        // ---- per source: sigma per class, robust sigma
-        for (int k = 0; k < nb; k++) {
-            const int64_t o0 = __shfl_sync(0xffffffffu, my_o0, k);
-            const int n = __shfl_sync(0xffffffffu, my_n, k);
-            if (n == 0) continue;
+// ---------------------------------------------------------------------------------------
+// class-sum path (one sigma per class and source)
+// ---------------------------------------------------------------------------------------
+constexpr int kSumVals = 21;       // 15 AA, 5 Ah, hh of one class
+constexpr int kPassWarps = 4;      // warps per block of the passes over the rows
+constexpr int kKeyCap64 = 1024;    // keys of a source kept in shared memory
+constexpr int kSelCap = 96;        // keys around a quantile that are ranked directly
+
+// float of a double by its bit pattern, truncated (relative error below 2^-23): values below the
+// FP32 range are 0, above it (and NaN) infinite.  Integer instructions: a conversion holds the
+// FP64 unit.
+__device__ __forceinline__ float trunc_f32(double x) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t ex = (hi >> 20) & 0x7ffu;
+    uint32_t f = __funnelshift_l(lo, hi, 3) ^ 0x40000000u;   // exponent - 896, 23 bits of the significand
+    f = ex < 897u ? 0u : (ex > 1150u ? 0x7f800000u : f & 0x7fffffffu);
+    return __uint_as_float(f | (hi & 0x80000000u));
+}
+
+// Sums of kSumVals lane values over the warp by recursive halving: in each step a lane gives one
+// half of its values to its partner and adds the partner's other half, 23 additions instead of
+// the 105 of butterflies.  out[i] (i < kSumVals) is written by the lane that ends up with it.
+__device__ __forceinline__ void reduce_vals(double* v, int lane, double* out) {
+    int off = 0, cnt = kSumVals;   // this lane's values are off .. off + cnt - 1
+    auto step = [&](auto nc, int bit) {
+        constexpr int n = decltype(nc)::value, h = (n + 1) / 2;
+        const bool up = lane & bit;
+#pragma unroll
+        for (int k = 0; k < h; k++) {
+            const double lo = v[k], hi = k + h < n ? v[k + h] : 0.0;
+            const double got = __shfl_xor_sync(0xffffffffu, up ? lo : hi, bit);
+            v[k] = (up ? hi : lo) + got;
+        }
+        off += up ? h : 0;
+        cnt = up ? cnt - h : (cnt < h ? cnt : h);
+    };
+    step(std::integral_constant<int, 21>{}, 16);
+    step(std::integral_constant<int, 11>{}, 8);
+    step(std::integral_constant<int, 6>{}, 4);
+    step(std::integral_constant<int, 3>{}, 2);
+    step(std::integral_constant<int, 2>{}, 1);
+    if (cnt > 0) out[off] = v[0];
+}
+
+__device__ __forceinline__ void row_load(const double* __restrict__ e, double& h, double A[5]) {
+    const double2 a = *reinterpret_cast<const double2*>(e), b = *reinterpret_cast<const double2*>(e + 2),
+                  c = *reinterpret_cast<const double2*>(e + 4);
+    h = a.x; A[0] = a.y; A[1] = b.x; A[2] = b.y; A[3] = c.x; A[4] = c.y;
+}
+__device__ __forceinline__ double row_dot(const double A[5], const double* d) {
+    double Ad = A[0] * d[0];
+    Ad = fma(A[1], d[1], Ad);
+    Ad = fma(A[2], d[2], Ad);
+    Ad = fma(A[3], d[3], Ad);
+    return fma(A[4], d[4], Ad);
+}
+
+// What a round subtracts from the unit-weight sums of one class: (1 - w) times the products of
+// the rows listed in shared memory (m <= 32 of them), lane by lane.  first: w = wfun(h rx), the
+// initial downweighting by the robust scale; else w = wfun((h - A d) isd).  last: w goes to the
+// scratch row for the hand-over records.
+__device__ __forceinline__ void subtract_rows(double* scr, const uint32_t* list, int m, int lane, bool first,
+                                              const double* d, double scale, int wfn, bool last, double* corr,
+                                              int& nout) {
+    if (lane >= m) return;
+    double* e = scr + (size_t)list[lane] * kScr;
+    double h, A[5];
+    row_load(e, h, A);
+    const double w = wfun((first ? h : h - row_dot(A, d)) * scale, wfn);
+    if (last) e[6] = w;
+    nout += w < 0.2;
+    const double u = 1.0 - w;
+#pragma unroll
+    for (int a = 0; a < 5; a++) {
+        const double ua = u * A[a];
+#pragma unroll
+        for (int b = a; b < 5; b++) corr[up5(a, b)] = fma(ua, A[b], corr[up5(a, b)]);
+        corr[15 + a] = fma(ua, h, corr[15 + a]);
+    }
+    corr[20] = fma(u * h, h, corr[20]);
+}
+
+// Direct class sums of one round: every row weighted (w = wfun(h rx) first, wfun((h - A d) isd)
+// later, 1 for plain weights), lane partials over the rows lane, lane + 32, ... of each class to
+// red[value][lane], then lane v adds the 32 partials of value v in lane order.  last: w goes to
+// the scratch row for the hand-over records.
+constexpr int kRedVals = 2 * kSumVals;
+constexpr int kRedStride = 33;    // doubles per value row (odd: the column sums read distinct banks)
+__device__ __forceinline__ void direct_sums(double* scr, int n, int nal, int lane, int mode, const double* rx,
+                                            const double* isd, const double* d, int wfn, bool last, double* red,
+                                            double* out, int& nout) {
+    int cnt = 0;
+    for (int c = 0; c < 2; c++) {
+        const int hi = c ? n : nal;
+        double AA[15], Ah[5], hs = 0.0;
+#pragma unroll
+        for (int i = 0; i < 15; i++) AA[i] = 0.0;
+#pragma unroll
+        for (int i = 0; i < 5; i++) Ah[i] = 0.0;
+        for (int j = (c ? nal : 0) + lane; j < hi; j += kWarp) {
+            double* e = scr + (size_t)j * kScr;
+            double h, A[5];
+            row_load(e, h, A);
+            double w = 1.0;
+            if (mode == 0) {
+                if (rx[c] > 0.0) w = wfun(h * rx[c], wfn);
+            } else if (mode == 1) {
+                w = wfun((h - row_dot(A, d)) * isd[c], wfn);
+            }
+            if (last) e[6] = w;
+            cnt += (w < 0.2);
+#pragma unroll
+            for (int a = 0; a < 5; a++) {
+                const double wa = w * A[a];
+#pragma unroll
+                for (int b = a; b < 5; b++) AA[up5(a, b)] += wa * A[b];
+                Ah[a] += wa * h;
+            }
+            hs += w * h * h;
+        }
+        double* rc = red + c * kSumVals * kRedStride;
+#pragma unroll
+        for (int i = 0; i < 15; i++) rc[i * kRedStride + lane] = AA[i];
+#pragma unroll
+        for (int i = 0; i < 5; i++) rc[(15 + i) * kRedStride + lane] = Ah[i];
+        rc[20 * kRedStride + lane] = hs;
+    }
+    nout = warp_sum_int(cnt);
+    __syncwarp();
+    for (int v = lane; v < kRedVals; v += kWarp) {
+        const double* col = red + v * kRedStride;
+        double t = col[0];
+#pragma unroll
+        for (int k = 1; k < kWarp; k++) t += col[k];
+        out[v] = t;
+    }
+    __syncwarp();
+}
+
+// Appends the row j of every lane with cand set to the list (n entries so far); a full list of 32
+// is worked off by `flush`.
+template <class F>
+__device__ __forceinline__ void append_rows(bool cand, int j, uint32_t* list, int& n, int lane, F flush) {
+    const unsigned ball = __ballot_sync(0xffffffffu, cand);
+    if (!ball) return;
+    const int pos = n + __popc(ball & ((1u << lane) - 1u));
+    if (cand && pos < 32) list[pos] = (uint32_t)j;
+    n += __popc(ball);
+    if (n < 32) return;
+    __syncwarp();
+    flush(32);
+    __syncwarp();
+    if (cand && pos >= 32) list[pos - 32] = (uint32_t)j;
+    n -= 32;
+}
+
+// The k-th and (k+1)-th smallest keys (k + 1 capped at n - 1) for k = k1 and k = k5 at once: a
+// histogram of the values on 256 equal steps between their extremes finds the steps that hold
+// those ranks, and the few keys in them are ranked against one another.  False if a step holds
+// too many keys (heavy ties, a wild outlier) or a value is not finite: the caller then uses the
+// radix select.
+struct SelWork {
+    uint64_t keys[kKeyCap64];
+    int hist[256];
+    uint64_t list[2][kSelCap];
+    uint64_t res[4];
+    int cnt[2];
+};
+__device__ bool select_quantiles(const uint64_t* __restrict__ keys, int n, int k1, int k5, float lo, float hi,
+                                 SelWork& sw, int lane, double out[4]) {
+    if (!(hi > lo) || !isfinite(lo) || !isfinite(hi)) return false;
+    const float scale = 256.0f / (hi - lo);
+    if (!isfinite(scale)) return false;
+#pragma unroll
+    for (int i = 0; i < 8; i++) sw.hist[lane + 32 * i] = 0;
+    if (lane < 2) sw.cnt[lane] = 0;
+    __syncwarp();
+    auto bin_of = [&](uint64_t key) {
+        const int b = (int)((trunc_f32(dkey_inv(key)) - lo) * scale);   // never decreasing in the key
+        return b > 255 ? 255 : b;
+    };
+    for (int j = lane; j < n; j += kWarp) atomicAdd(&sw.hist[bin_of(keys[j])], 1);
+    __syncwarp();
+    int c[8], tot = 0;
+#pragma unroll
+    for (int i = 0; i < 8; i++) { c[i] = sw.hist[lane * 8 + i]; tot += c[i]; }
+    int incl = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    // the steps of ranks k1, k1 + 1, k5, k5 + 1 and the keys below the first of each pair
+    int bin[4], below[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        int k = (q < 2 ? k1 : k5) + (q & 1);
+        if (k > n - 1) k = n - 1;
+        const unsigned ball = __ballot_sync(0xffffffffu, incl > k);
+        const int sl = __ffs(ball) - 1;
+        int acc = incl - tot, bs = 7;
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            if (bs == 7 && acc + c[i] > k) bs = i + 8;
+            if (bs < 8) acc += c[i];
+        }
+        if (bs == 7) acc -= c[7];   // not reached for the chosen lane
+        bin[q] = __shfl_sync(0xffffffffu, lane * 8 + (bs & 7), sl);
+        below[q] = __shfl_sync(0xffffffffu, acc, sl);
+    }
+    bool ok = true;
+#pragma unroll
+    for (int p = 0; p < 2; p++) {
+        const int m = sw.hist[bin[2 * p]] + (bin[2 * p + 1] != bin[2 * p] ? sw.hist[bin[2 * p + 1]] : 0);
+        ok = ok && m <= kSelCap;
+    }
+    if (!ok) return false;
+    for (int j = lane; j < n; j += kWarp) {
+        const uint64_t key = keys[j];
+        const int b = bin_of(key);
+        if (b >= bin[0] && b <= bin[1]) sw.list[0][atomicAdd(&sw.cnt[0], 1)] = key;
+        if (b >= bin[2] && b <= bin[3]) sw.list[1][atomicAdd(&sw.cnt[1], 1)] = key;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int p = 0; p < 2; p++) {
+        const int m = sw.cnt[p];
+        const int t0 = (p ? k5 : k1) - below[2 * p];
+        const int t1 = (p ? k5 : k1) + 1 > n - 1 ? t0 : t0 + 1;
+        for (int a = lane; a < m; a += kWarp) {
+            const uint64_t key = sw.list[p][a];
+            int less = 0, eq = 0;
+            for (int b = 0; b < m; b++) {
+                const uint64_t o = sw.list[p][b];
+                less += o < key;
+                eq += o == key;
+            }
+            // this value holds the ranks less .. less + eq - 1
+            if (t0 >= less && t0 < less + eq) sw.res[2 * p] = key;
+            if (t1 >= less && t1 < less + eq) sw.res[2 * p + 1] = key;
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 4; q++) out[q] = dkey_inv(sw.res[q]);
+    __syncwarp();
+    return true;
+}
+
+// Per source: sigma per class, robust scale of x = h / sigma (Sect. 5.1.2: half the intersextile
+// range), unit-weight class sums, and round 0's downweighting.
+template <bool kDirect>
+__global__ void __launch_bounds__(32 * kPassWarps) k_src_first(Settings st, const int64_t* __restrict__ src_off,
+                                                               const int32_t* __restrict__ src_nal,
+                                                               const int32_t* __restrict__ src_order, int32_t n_src,
+                                                               int batch, double* __restrict__ scratch,
+                                                               const uint64_t* __restrict__ skey,
+                                                               SrcWork* __restrict__ work) {
+    extern __shared__ __align__(16) unsigned char first_smem[];
+    union FirstWork {
+        SelWork sel;
+        double red[kDirect ? kRedVals * kRedStride : 1];
+    };
+    FirstWork& fw = reinterpret_cast<FirstWork*>(first_smem)[threadIdx.x >> 5];
+    SelWork& sw = fw.sel;
+    __shared__ uint32_t list_all[kPassWarps][32];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    uint32_t* list = list_all[wib];
+    const int step = gridDim.x * kPassWarps * batch;
+    for (int base = (blockIdx.x * kPassWarps + wib) * batch; base < n_src; base += step)
+        for (int q = base; q < min(base + batch, n_src); q++) {
+            const int i = src_order[q];
+            const int64_t o0 = src_off[i];
+            const int n = (int)(src_off[i + 1] - o0), nal = src_nal[i];
+            SrcWork& w = work[i];
+            if (n == 0) {
+                if (lane == 0) w.flags = 2;
+                continue;
+            }
             double* scr = scratch + (size_t)o0 * kScr;
-            double s2min = 1e300;
-            double s2lo[2] = {1e300, 1e300}, s2hi[2] = {-1e300, -1e300};
-            for (int j = lane; j < n; j += kWarp) {
-                const double s2 = scr[(size_t)j * kScr + 7];
-                const int c = meta_kind(meta[o0 + j]);
-                s2lo[c] = fmin(s2lo[c], s2);
-                s2hi[c] = fmax(s2hi[c], s2);
-                s2min = fmin(s2min, s2);
+            // unit-weight sums and sigma of each class; sums only while its sigma is one value
+            double s2c[2] = {1.0, 1.0}, s2min = 1e300;
+            bool uni = true;
+            for (int c = 0; c < 2; c++) {
+                const int lo = c ? nal : 0, hi = c ? n : nal;
+                double v[kSumVals];
+#pragma unroll
+                for (int k = 0; k < kSumVals; k++) v[k] = 0.0;
+                if (lo < hi) {
+                    const double s2 = scr[(size_t)lo * kScr + 7];
+                    bool same = true;
+                    for (int j0 = lo; j0 < hi; j0 += kWarp) {
+                        const int j = j0 + lane;
+                        if (j < hi) {
+                            const double* e = scr + (size_t)j * kScr;
+                            const double sj = e[7];
+                            s2min = fmin(s2min, sj);
+                            same = same && sj == s2;
+                            if (!kDirect && uni) {
+                                double h, A[5];
+                                row_load(e, h, A);
+#pragma unroll
+                                for (int a = 0; a < 5; a++) {
+#pragma unroll
+                                    for (int b = a; b < 5; b++) v[up5(a, b)] = fma(A[a], A[b], v[up5(a, b)]);
+                                    v[15 + a] = fma(A[a], h, v[15 + a]);
+                                }
+                                v[20] = fma(h, h, v[20]);
+                            }
+                        }
+                        uni = __all_sync(0xffffffffu, uni && same);
+                    }
+                    s2c[c] = s2;
+                }
+                if (!kDirect && uni) reduce_vals(v, lane, w.T[c]);
             }
             s2min = warp_min(s2min);
-            for (int c = 0; c < 2; c++) {
-                s2lo[c] = warp_min(s2lo[c]);
-                s2hi[c] = -warp_min(-s2hi[c]);
-            }
-            const bool uni = (s2lo[0] == s2hi[0] || s2lo[0] == 1e300) && (s2lo[1] == s2hi[1] || s2lo[1] == 1e300);
-            __syncwarp();
             double vs = 0.0;
+            const bool in_smem = n <= kKeyCap64;
+            const uint64_t* keys = in_smem ? sw.keys : skey + o0;
             if (st.robust) {
-                const double p1 = 1.0 / 6.0, p5 = 5.0 / 6.0;
-                const double h1 = p1 * (double)(n - 1), h5 = p5 * (double)(n - 1);
+                float lo = INFINITY, hi = -INFINITY;
+                bool nan = false;
+                for (int j = lane; j < n; j += kWarp) {
+                    const uint64_t key = skey[o0 + j];
+                    if (in_smem) sw.keys[j] = key;
+                    const float x = trunc_f32(dkey_inv(key));
+                    nan = nan || !isfinite(x);
+                    lo = fminf(lo, x);
+                    hi = fmaxf(hi, x);
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+                    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+                }
+                nan = __any_sync(0xffffffffu, nan);
+                __syncwarp();
+                const double h1 = __dmul_rn(1.0 / 6.0, (double)(n - 1)), h5 = __dmul_rn(5.0 / 6.0, (double)(n - 1));
                 const int lo1 = (int)floor(h1), lo5 = (int)floor(h5);
-                double a0, a1, b0, b1;
-                warp_select_pair(skey + o0, n, lo1, hist, lane, a0, a1);
-                warp_select_pair(skey + o0, n, lo5, hist, lane, b0, b1);
-                vs = 0.5 * ((b0 + (h5 - lo5) * (b1 - b0)) - (a0 + (h1 - lo1) * (a1 - a0)));
+                double x[4];
+                if (nan || !select_quantiles(keys, n, lo1, lo5, lo, hi, sw, lane, x)) {
+                    warp_select_pair(keys, n, lo1, sw.hist, lane, x[0], x[1]);
+                    warp_select_pair(keys, n, lo5, sw.hist, lane, x[2], x[3]);
+                }
+                // products and differences rounded one by one (h - floor(h) is exact)
+                const double g1 = __dadd_rn(h1, -(double)lo1), g5 = __dadd_rn(h5, -(double)lo5);
+                vs = 0.5 * ((x[2] + g5 * (x[3] - x[2])) - (x[0] + g1 * (x[1] - x[0])));
                 __syncwarp();
             }
-            __syncwarp();
-            if (lane == k) {
-                my_uniform = uni;
-                my_s2c[0] = s2lo[0] == 1e300 ? 1.0 : s2lo[0];
-                my_s2c[1] = s2lo[1] == 1e300 ? 1.0 : s2lo[1];
-                my_s2min = s2min;
-                my_vs = vs;
+            if (lane == 0) {
+                w.s2c[0] = s2c[0];
+                w.s2c[1] = s2c[1];
+                w.s2min = s2min;
+                w.vs = vs;
+                w.flags = uni ? 1 : 0;
             }
-        }
-        // ---- inner iteration, class-sum path (lane k solves source k)
-        double d[5] = {0, 0, 0, 0, 0};
-        double U[kU5];
-        for (int q = 0; q < kU5; q++) U[q] = 0.0;
-        double y = 0.0, Q = 0.0, Q0 = 0.0, S2 = 0.0;
-        int nu = 0, nout = 0, rd = 0;
-        for (int rnd = 0; rnd < rounds; rnd++) {
-            const int mode = !st.robust ? 2 : (rnd == 0 ? 0 : 1);
-            for (int k = 0; k < nb; k++) {
-                const int n = __shfl_sync(0xffffffffu, my_n, k);
-                const int uni = __shfl_sync(0xffffffffu, (int)my_uniform, k);
-                if (n == 0 || !uni) continue;
-                const int64_t o0 = __shfl_sync(0xffffffffu, my_o0, k);
-                const int nal = __shfl_sync(0xffffffffu, my_nal, k);
-                double dk[5];
-                for (int a = 0; a < 5; a++) dk[a] = __shfl_sync(0xffffffffu, d[a], k);
-                const double yk = __shfl_sync(0xffffffffu, y, k);
-                const double s2c[2] = {__shfl_sync(0xffffffffu, my_s2c[0], k), __shfl_sync(0xffffffffu, my_s2c[1], k)};
-                const double vsk = __shfl_sync(0xffffffffu, my_vs, k);
-                const RoundIn ri = round_in(s2c, yk, vsk);
-                double* scr = scratch + (size_t)o0 * kScr;
-                int no = 0;
-                pass_class(scr, n, nal, lane, mode, ri, dk, st.weight_fn, rnd == rounds - 1, sums[k], no, red);
-                if (lane == k) nout = no;
+            if (!uni) continue;
+            const bool last = st.robust ? st.n_rounds == 0 : true;
+            int nout = 0;
+            if (kDirect) {
+                double rx[2];
+                for (int c = 0; c < 2; c++) rx[c] = vs > 0.0 ? 1.0 / (sqrt(s2c[c]) * vs) : 0.0;
+                direct_sums(scr, n, nal, lane, st.robust ? 0 : 2, rx, nullptr, nullptr, st.weight_fn, last, fw.red,
+                            &w.T[0][0], nout);
+                if (lane == 0) w.nout = nout;
+                for (int k = lane; k < kRedVals; k += kWarp) (&w.C[0][0])[k] = 0.0;
+                __syncwarp();
+                continue;
             }
-            __syncwarp();
-            if (mine && my_n > 0 && my_uniform) {
-                nu = my_n - nout - 5;
-                y = 0.0;
-                class_solve(sums[lane], my_s2c, 0.0, st.pivot_tol, U, d, rd, Q, S2);
-                Q0 = Q;
-                if (st.robust && nu > 0 && Q0 > (double)nu) {
-                    const double tol = 1e-12 * my_s2min;
-                    for (int it = 0; it < st.n_eps; it++) {
-                        const double dy = (1.0 - Q / (double)nu) * Q / (-S2);
-                        y = fmax(0.0, y + dy);
-                        class_solve(sums[lane], my_s2c, y, st.pivot_tol, U, d, rd, Q, S2);
-                        if (fabs(dy) <= tol) break;
+            for (int c = 0; c < 2; c++) {
+                const int lo = c ? nal : 0, hi = c ? n : nal;
+                double corr[kSumVals];
+#pragma unroll
+                for (int k = 0; k < kSumVals; k++) corr[k] = 0.0;
+                int m = 0;
+                bool any = false;
+                const double rx = vs > 0.0 ? 1.0 / (sqrt(s2c[c]) * vs) : 0.0;
+                const float ivs = (float)(1.0 / vs);
+                auto flush = [&](int k) {
+                    subtract_rows(scr, list, k, lane, true, nullptr, rx, st.weight_fn, last, corr, nout);
+                    any = true;
+                };
+                if (st.robust && rx > 0.0)
+                    for (int j0 = lo; j0 < hi; j0 += kWarp) {
+                        const int j = j0 + lane;
+                        // x of the key, to 2^-22 relative: at or above 2 within that, or not finite
+                        const bool cand = j < hi && !(fabsf(trunc_f32(dkey_inv(keys[j])) * ivs) < 1.99999f);
+                        if (last && j < hi && !cand) scr[(size_t)j * kScr + 6] = 1.0;
+                        append_rows(cand, j, list, m, lane, flush);
                     }
-                }
+                else if (last)
+                    for (int j = lo + lane; j < hi; j += kWarp) scr[(size_t)j * kScr + 6] = 1.0;
+                __syncwarp();
+                if (m > 0) flush(m);
+                __syncwarp();
+                if (any) reduce_vals(corr, lane, w.C[c]);
+                else if (lane < kSumVals) w.C[c][lane] = 0.0;
             }
+            nout = warp_sum_int(nout);
+            if (lane == 0) w.nout = nout;
             __syncwarp();
         }
-        // ---- hand-over records and per-source results
-        double my_chi = 0.0;
-        for (int k = 0; k < nb; k++) {
-            const int n = __shfl_sync(0xffffffffu, my_n, k);
-            const int uni = __shfl_sync(0xffffffffu, (int)my_uniform, k);
-            if (n == 0 || !uni) continue;
-            const int64_t o0 = __shfl_sync(0xffffffffu, my_o0, k);
-            const int nal = __shfl_sync(0xffffffffu, my_nal, k);
-            double dk[5];
-            for (int a = 0; a < 5; a++) dk[a] = __shfl_sync(0xffffffffu, d[a], k);
-            const double yk = __shfl_sync(0xffffffffu, y, k);
-            const double iw[2] = {1.0 / (__shfl_sync(0xffffffffu, my_s2c[0], k) + yk),
-                                  1.0 / (__shfl_sync(0xffffffffu, my_s2c[1], k) + yk)};
+}
+
+// Class sums of a later round: w = wfun((h - A d) / sqrt(sigma_c^2 + y)) with the previous round's
+// (d, y).  z = (h - A d) isd in FP32 from truncated values: its error is below
+// 2^-19 isd (|h| + sum |A_k d_k|) (truncation 2^-23 of each factor, ten roundings of 2^-24).
+__global__ void __launch_bounds__(32 * kPassWarps) k_src_round(Settings st, int last, const int64_t* __restrict__ src_off,
+                                                               const int32_t* __restrict__ src_nal,
+                                                               const int32_t* __restrict__ src_order, int32_t n_src,
+                                                               int batch, double* __restrict__ scratch,
+                                                               SrcWork* __restrict__ work) {
+    __shared__ uint32_t list_all[kPassWarps][32];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    uint32_t* list = list_all[wib];
+    const int step = gridDim.x * kPassWarps * batch;
+    for (int base = (blockIdx.x * kPassWarps + wib) * batch; base < n_src; base += step)
+        for (int q = base; q < min(base + batch, n_src); q++) {
+            const int i = src_order[q];
+            SrcWork& w = work[i];
+            if (w.flags != 1) continue;
+            const int64_t o0 = src_off[i];
+            const int n = (int)(src_off[i + 1] - o0), nal = src_nal[i];
+            double* scr = scratch + (size_t)o0 * kScr;
+            double d[5];
+            float df[5];
+#pragma unroll
+            for (int k = 0; k < 5; k++) { d[k] = w.d[k]; df[k] = (float)d[k]; }
+            int nout = 0;
+            for (int c = 0; c < 2; c++) {
+                const int lo = c ? nal : 0, hi = c ? n : nal;
+                const double isd = w.isd[c];
+                const float isf = (float)isd;
+                double corr[kSumVals];
+#pragma unroll
+                for (int k = 0; k < kSumVals; k++) corr[k] = 0.0;
+                int m = 0;
+                bool any = false;
+                auto flush = [&](int k) {
+                    subtract_rows(scr, list, k, lane, false, d, isd, st.weight_fn, last, corr, nout);
+                    any = true;
+                };
+                auto screen = [&](double h, const double A[5]) {
+                    const float hf = trunc_f32(h);
+                    float Rf = hf, S = fabsf(hf);
+#pragma unroll
+                    for (int k = 0; k < 5; k++) {
+                        const float t = trunc_f32(A[k]) * df[k];
+                        Rf -= t;
+                        S += fabsf(t);
+                    }
+                    return !((fabsf(Rf) + S * 1.9073486e-6f) * isf < 2.0f);
+                };
+                for (int j0 = lo; j0 < hi; j0 += 2 * kWarp) {   // two rows in flight per lane
+                    const int ja = j0 + lane, jb = ja + kWarp;
+                    double ha = 0.0, hb = 0.0, Aa[5], Ab[5];
+                    if (ja < hi) row_load(scr + (size_t)ja * kScr, ha, Aa);
+                    if (jb < hi) row_load(scr + (size_t)jb * kScr, hb, Ab);
+                    const bool ca = ja < hi && screen(ha, Aa);
+                    const bool cb = jb < hi && screen(hb, Ab);
+                    if (last) {
+                        if (ja < hi && !ca) scr[(size_t)ja * kScr + 6] = 1.0;
+                        if (jb < hi && !cb) scr[(size_t)jb * kScr + 6] = 1.0;
+                    }
+                    append_rows(ca, ja, list, m, lane, flush);
+                    append_rows(cb, jb, list, m, lane, flush);
+                }
+                __syncwarp();
+                if (m > 0) flush(m);
+                __syncwarp();
+                if (any) reduce_vals(corr, lane, w.C[c]);
+                else if (lane < kSumVals) w.C[c][lane] = 0.0;
+            }
+            nout = warp_sum_int(nout);
+            if (lane == 0) w.nout = nout;
+        }
+}
+
+__global__ void __launch_bounds__(32 * kPassWarps) k_src_round_direct(Settings st, int last,
+                                                                      const int64_t* __restrict__ src_off,
+                                                                      const int32_t* __restrict__ src_nal,
+                                                                      const int32_t* __restrict__ src_order,
+                                                                      int32_t n_src, int batch,
+                                                                      double* __restrict__ scratch,
+                                                                      SrcWork* __restrict__ work) {
+    __shared__ double red_all[kPassWarps][kRedVals * kRedStride];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int step = gridDim.x * kPassWarps * batch;
+    for (int base = (blockIdx.x * kPassWarps + wib) * batch; base < n_src; base += step)
+        for (int q = base; q < min(base + batch, n_src); q++) {
+            const int i = src_order[q];
+            SrcWork& w = work[i];
+            if (w.flags != 1) continue;
+            const int64_t o0 = src_off[i];
+            double d[5];
+#pragma unroll
+            for (int k = 0; k < 5; k++) d[k] = w.d[k];
+            const double isd[2] = {w.isd[0], w.isd[1]};
+            int nout;
+            direct_sums(scratch + (size_t)o0 * kScr, (int)(src_off[i + 1] - o0), src_nal[i], lane, 1, nullptr, isd, d,
+                        st.weight_fn, last, red_all[wib], &w.T[0][0], nout);
+            if (lane == 0) w.nout = nout;
+        }
+}
+
+// class_solve by two neighbouring lanes of a warp: each forms half of the 15 + 5 entries of N and b,
+// both factor and solve, and each sums Q's numerator of one class.  Every value is formed by the
+// operations of class_solve in their order.
+struct HalfSums {
+    double E[2][10];             // entries 10 h .. 10 h + 9 of (AA, Ah) of both classes
+    double AA[15], Ah[5], hh;    // class h
+};
+__device__ __forceinline__ double lane_pair(double v) { return __shfl_xor_sync(0xffffffffu, v, 1); }
+static __device__ __noinline__ void class_solve_pair(const HalfSums& S, int h, const double* s2c, double y, double tol_piv,
+                                                     double* U, double* d, int& rd, double& Q, double& S2) {
+    const double im = 1.0 / (s2c[h] + y), io = lane_pair(im);
+    const double i0 = h ? io : im, i1 = h ? im : io;
+    double NB[20];
+#pragma unroll
+    for (int k = 0; k < 10; k++) {
+        const double v = S.E[0][k] * i0 + S.E[1][k] * i1, o = lane_pair(v);
+        NB[k] = h ? o : v;
+        NB[10 + k] = h ? v : o;
+    }
+    rd = chol5(NB, U, tol_piv);
+    chol5_solve(U, NB + 15, d);
+    double dMd = 0.0, db = 0.0;
+#pragma unroll
+    for (int a = 0; a < 5; a++) {
+        db += d[a] * S.Ah[a];
+        dMd += S.AA[up5(a, a)] * d[a] * d[a];
+#pragma unroll
+        for (int k = a + 1; k < 5; k++) dMd += 2.0 * S.AA[up5(a, k)] * d[a] * d[k];
+    }
+    const double nm = S.hh - 2.0 * db + dMd, no = lane_pair(nm);
+    const double num[2] = {h ? no : nm, h ? nm : no};
+    Q = num[0] * i0 + num[1] * i1;
+    S2 = num[0] * i0 * i0 + num[1] * i1 * i1;
+}
+
+// the 5x5 algebra of one round, one thread (kPair: two neighbouring lanes) per source: y = 0 first,
+// then the rational steps of the excess variance.  Leaves (d, 1 / sqrt(sigma_c^2 + y)) for the next
+// round; after the last round the update, 1 / (sigma_c^2 + y) and the per-source results.
+template <bool kPair>
+__global__ void __launch_bounds__(128) k_src_solve5(Settings st, int last, const int64_t* __restrict__ src_off,
+                                                    int32_t n_src, SrcOutPtrs out, SrcWork* __restrict__ work) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int h = kPair ? t & 1 : 0;
+    const int it_ = kPair ? t >> 1 : t;
+    const int i = it_ < n_src ? it_ : n_src - 1;   // lanes beyond the sources repeat the last one for the shuffles
+    const bool mine = it_ < n_src && h == 0;
+    if (!kPair && !mine) return;
+    SrcWork& w = work[i];
+    const int flags = w.flags;
+    if (mine && (flags & 2) && last) {
+        for (int k = 0; k < 5; k++) out.d[5 * (size_t)i + k] = 0.0;
+        for (int k = 0; k < 25; k++) out.cov[25 * (size_t)i + k] = 0.0;
+        out.eps2[i] = out.q[i] = out.dsig[i] = out.chi2[i] = 0.0;
+        out.nu[i] = out.nout[i] = out.rankdef[i] = 0;
+    }
+    if (!kPair && flags != 1) return;
+    const int n = (int)(src_off[i + 1] - src_off[i]);
+    ClassSums S;
+    HalfSums H;
+    if (kPair) {
+        for (int c = 0; c < 2; c++)
+            for (int k = 0; k < 10; k++) H.E[c][k] = w.T[c][10 * h + k] - w.C[c][10 * h + k];
+        for (int k = 0; k < 15; k++) H.AA[k] = w.T[h][k] - w.C[h][k];
+        for (int k = 0; k < 5; k++) H.Ah[k] = w.T[h][15 + k] - w.C[h][15 + k];
+        H.hh = w.T[h][20] - w.C[h][20];
+    } else {
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+#pragma unroll
+            for (int k = 0; k < 15; k++) S.AA[c][k] = w.T[c][k] - w.C[c][k];
+#pragma unroll
+            for (int k = 0; k < 5; k++) S.Ah[c][k] = w.T[c][15 + k] - w.C[c][15 + k];
+            S.hh[c] = w.T[c][20] - w.C[c][20];
+        }
+    }
+    const double s2c[2] = {w.s2c[0], w.s2c[1]};
+    const int nout = w.nout, nu = n - nout - 5;
+    double U[kU5], d[5], y = 0.0, Q, S2;
+    int rd;
+    auto solve = [&](double yy) {
+        if (kPair) class_solve_pair(H, h, s2c, yy, st.pivot_tol, U, d, rd, Q, S2);
+        else class_solve(S, s2c, yy, st.pivot_tol, U, d, rd, Q, S2);
+    };
+    solve(0.0);
+    const double Q0 = Q;
+    // the two lanes of a pair hold the same values; the pairs of a warp leave the loop together
+    bool go = st.robust && flags == 1 && nu > 0 && Q0 > (double)nu;
+    const double tol = 1e-12 * w.s2min;
+    for (int it = 0; it < st.n_eps; it++) {
+        if (kPair ? !__any_sync(0xffffffffu, go) : !go) break;
+        const double dy = (1.0 - Q / (double)nu) * Q / (-S2);
+        if (kPair) {
+            // a pair that is done keeps its solution: solve again at its y (the same values)
+            y = go ? fmax(0.0, y + dy) : y;
+            solve(y);
+            go = go && !(fabs(dy) <= tol);
+        } else {
+            y = fmax(0.0, y + dy);
+            solve(y);
+            if (fabs(dy) <= tol) break;
+        }
+    }
+    if (!mine || flags != 1) return;
+#pragma unroll
+    for (int k = 0; k < 5; k++) w.d[k] = d[k];
+    if (!last) {
+        for (int c = 0; c < 2; c++) w.isd[c] = 1.0 / sqrt(s2c[c] + y);
+        return;
+    }
+    for (int c = 0; c < 2; c++) w.isd[c] = 1.0 / (s2c[c] + y);
+    double* sp = out.src + 5 * (size_t)i;
+    const double cosd = cos(sp[1]);
+    sp[0] += d[0] / cosd;
+    for (int k = 1; k < 5; k++) sp[k] += d[k];
+    for (int k = 0; k < 5; k++) out.d[5 * (size_t)i + k] = d[k];
+    for (int c = 0; c < 5; c++) {
+        double e[5] = {0, 0, 0, 0, 0};
+        e[c] = 1.0;
+        double x[5];
+        chol5_solve(U, e, x);
+        for (int k = 0; k < 5; k++) out.cov[25 * (size_t)i + 5 * k + c] = x[k];
+    }
+    out.eps2[i] = y;
+    out.q[i] = Q;
+    out.nu[i] = nu;
+    out.nout[i] = nout;
+    out.dsig[i] = nu > 0 ? (Q0 - (double)nu) / sqrt(2.0 * (double)nu) : 0.0;
+    out.rankdef[i] = rd;
+}
+
+// hand-over records R = h - A d, W = w / (sigma_c^2 + y) and chi^2 of the class-sum sources
+__global__ void __launch_bounds__(32 * kPassWarps) k_src_final(Settings st, const int64_t* __restrict__ src_off,
+                                                               const int32_t* __restrict__ src_nal,
+                                                               const int32_t* __restrict__ src_order, int32_t n_src,
+                                                               int batch, const double* __restrict__ scratch,
+                                                               const SrcWork* __restrict__ work, SrcOutPtrs out,
+                                                               ObsRec* __restrict__ rec) {
+    const int lane = threadIdx.x & 31;
+    const int step = gridDim.x * kPassWarps * batch;
+    for (int base = (blockIdx.x * kPassWarps + (threadIdx.x >> 5)) * batch; base < n_src; base += step)
+        for (int q = base; q < min(base + batch, n_src); q++) {
+            const int i = src_order[q];
+            const SrcWork& w = work[i];
+            if (w.flags != 1) continue;
+            const int64_t o0 = src_off[i];
+            const int n = (int)(src_off[i + 1] - o0), nal = src_nal[i];
             const double* scr = scratch + (size_t)o0 * kScr;
+            const double d[5] = {w.d[0], w.d[1], w.d[2], w.d[3], w.d[4]};
+            const double iw[2] = {w.isd[0], w.isd[1]};
             double chi = 0.0;
             for (int j = lane; j < n; j += kWarp) {
                 const double* e = scr + (size_t)j * kScr;
-                const double R = e[0] - (e[1] * dk[0] + e[2] * dk[1] + e[3] * dk[2] + e[4] * dk[3] + e[5] * dk[4]);
+                double h, A[5];
+                row_load(e, h, A);
+                const double R = h - (A[0] * d[0] + A[1] * d[1] + A[2] * d[2] + A[3] * d[3] + A[4] * d[4]);
                 const double W = e[6] * (j < nal ? iw[0] : iw[1]);
                 ObsRec* r = rec + (o0 + j);
-                r->R = st.handover_h ? e[0] : R;
+                r->R = st.handover_h ? h : R;
                 r->W = W;
                 chi += W * R * R;
             }
             chi = warp_sum(chi);
-            if (lane == k) my_chi = chi;
+            if (lane == 0) out.chi2[i] = chi;
         }
-        if (mine && (my_n == 0 || my_uniform)) {
-            const int i = my_i;
-            if (my_n == 0) {
-                for (int k = 0; k < 5; k++) out.d[5 * (size_t)i + k] = 0.0;
-                for (int k = 0; k < 25; k++) out.cov[25 * (size_t)i + k] = 0.0;
-                out.eps2[i] = out.q[i] = out.dsig[i] = out.chi2[i] = 0.0;
-                out.nu[i] = out.nout[i] = out.rankdef[i] = 0;
-            } else {
-                double* sp = out.src + 5 * (size_t)i;
-                sp[0] = s5[0] + d[0] / cosd;
-                sp[1] = s5[1] + d[1];
-                sp[2] = s5[2] + d[2];
-                sp[3] = s5[3] + d[3];
-                sp[4] = s5[4] + d[4];
-                for (int k = 0; k < 5; k++) out.d[5 * (size_t)i + k] = d[k];
-                for (int c = 0; c < 5; c++) {
-                    double e[5] = {0, 0, 0, 0, 0};
-                    e[c] = 1.0;
-                    double x[5];
-                    chol5_solve(U, e, x);
-                    for (int k = 0; k < 5; k++) out.cov[25 * (size_t)i + 5 * k + c] = x[k];
-                }
-                out.eps2[i] = y;
-                out.q[i] = Q;
-                out.nu[i] = nu;
-                out.nout[i] = nout;
-                out.dsig[i] = nu > 0 ? (Q0 - (double)nu) / sqrt(2.0 * (double)nu) : 0.0;
-                out.chi2[i] = my_chi;
-                out.rankdef[i] = rd;
-            }
-        }
-        __syncwarp();
-        // ---- sources without one sigma per class: general path, one at a time
-        for (int k = 0; k < nb; k++) {
-            const int n = __shfl_sync(0xffffffffu, my_n, k);
-            const int uni = __shfl_sync(0xffffffffu, (int)my_uniform, k);
-            if (n == 0 || uni) continue;
-            const int i = __shfl_sync(0xffffffffu, my_i, k);
-            const int64_t o0 = __shfl_sync(0xffffffffu, my_o0, k);
-            double sk[5];
-            for (int a = 0; a < 5; a++) sk[a] = __shfl_sync(0xffffffffu, s5[a], k);
-            const double ck = __shfl_sync(0xffffffffu, cosd, k);
-            const double s2m = __shfl_sync(0xffffffffu, my_s2min, k);
-            const double vsk = __shfl_sync(0xffffffffu, my_vs, k);
-            solve_general(st, i, o0, n, sk, ck, scratch + (size_t)o0 * kScr, s2m, vsk, out, rec, lane);
-        }
+}
+
+// sources whose sigma differs within a class: all rounds by per-observation passes
+__global__ void __launch_bounds__(32 * kPassWarps) k_src_general(Settings st, const int64_t* __restrict__ src_off,
+                                                                 const int32_t* __restrict__ src_order, int32_t n_src,
+                                                                 SrcOutPtrs out, ObsRec* __restrict__ rec,
+                                                                 double* __restrict__ scratch,
+                                                                 const SrcWork* __restrict__ work) {
+    const int lane = threadIdx.x & 31;
+    const int nw = gridDim.x * kPassWarps;
+    for (int q = blockIdx.x * kPassWarps + (threadIdx.x >> 5); q < n_src; q += nw) {
+        const int i = src_order[q];
+        const SrcWork& w = work[i];
+        if (w.flags != 0) continue;
+        const int64_t o0 = src_off[i];
+        const int n = (int)(src_off[i + 1] - o0);
+        double s5[5];
+        for (int k = 0; k < 5; k++) s5[k] = out.src[5 * (size_t)i + k];
+        solve_general(st, i, o0, n, s5, cos(s5[1]), scratch + (size_t)o0 * kScr, w.s2min, w.vs, out, rec, lane);
     }
 }
 
@@ -625,22 +1035,43 @@ void launch_obs_pass(const DevGeo& G, const AttNoise& an, const int64_t* t_ns, c
                                               rec);
 }
 
-// the per-source solves of the S block on the scratch rows of the observation pass
-void launch_source_solve(const Settings& st, const uint32_t* meta, const int64_t* src_off, const int32_t* src_nal,
+// The inner iteration of the S block on the scratch rows of the observation pass.  corrections:
+// rounds subtract (1 - w) terms from unit-weight sums; else each round sums every row.
+void launch_source_solve(const Settings& st, bool corrections, const int64_t* src_off, const int32_t* src_nal,
                          const int32_t* src_order, int32_t n_src, const SrcOutPtrs& out, ObsRec* rec, double* scratch,
-                         const uint64_t* skey, int* work_counter, int n_blocks, const Shapes& sh, cudaStream_t stream) {
-    cudaMemsetAsync(work_counter, 0, sizeof(int), stream);
-    // batch size: 32 sources per warp when there are enough sources to keep ~16 warps per SM
-    // busy, unless the autotuner chose one
-    int batch = n_src / (152 * 16);
-    batch = batch < 1 ? 1 : (batch > 32 ? 32 : batch);
-    if (sh.src_batch > 0) batch = sh.src_batch;
-    int warps = (n_src + batch - 1) / batch;
-    int blocks = (warps + kSolveWarps - 1) / kSolveWarps;
-    if (blocks > n_blocks * 4) blocks = n_blocks * 4;
-    if (blocks < 1) blocks = 1;
-    k_source_solve<<<blocks, 32 * kSolveWarps, 0, stream>>>(st, meta, src_off, src_nal, src_order, n_src, batch, out,
-                                                            rec, scratch, skey, work_counter);
+                         const uint64_t* skey, SrcWork* work, const Shapes& sh, cudaStream_t stream) {
+    if (n_src == 0) return;
+    // consecutive sources of the largest-first order per warp and step: one, unless the autotuner
+    // chose more (grids of at most 16 blocks per SM, a warp per source up to 9728 sources)
+    const int batch = sh.src_batch > 0 ? sh.src_batch : 1;
+    const int64_t warps = ((int64_t)n_src + batch - 1) / batch;
+    int64_t blocks = (warps + kPassWarps - 1) / kPassWarps;
+    if (blocks > 152 * 16) blocks = 152 * 16;
+    const int nb = (int)blocks, th = 32 * kPassWarps;
+    const int rounds = st.robust ? st.n_rounds + 1 : 1;
+    // a warp of 5x5 algebra is a chain of FP64 instructions (64 cycles each): two lanes per source and
+    // one warp per block while that leaves sub-partitions idle (800 sources: 38 us a round, one
+    // lane 48), one lane beyond (30,000 sources: 100 us)
+    const bool pair = n_src <= 152 * 4 * 16;
+    constexpr size_t first_smem = kPassWarps * sizeof(SelWork);
+    static_assert(sizeof(SelWork) <= kRedVals * kRedStride * sizeof(double), "shared memory of the direct first pass");
+    for (int r = 0; r < rounds; r++) {
+        const int last = r == rounds - 1;
+        if (r == 0 && corrections)
+            k_src_first<false><<<nb, th, first_smem, stream>>>(st, src_off, src_nal, src_order, n_src, batch, scratch, skey,
+                                                               work);
+        else if (r == 0)
+            k_src_first<true><<<nb, th, kPassWarps * kRedVals * kRedStride * sizeof(double), stream>>>(
+                st, src_off, src_nal, src_order, n_src, batch, scratch, skey, work);
+        else if (corrections)
+            k_src_round<<<nb, th, 0, stream>>>(st, last, src_off, src_nal, src_order, n_src, batch, scratch, work);
+        else
+            k_src_round_direct<<<nb, th, 0, stream>>>(st, last, src_off, src_nal, src_order, n_src, batch, scratch, work);
+        if (pair) k_src_solve5<true><<<(2 * n_src + 31) / 32, 32, 0, stream>>>(st, last, src_off, n_src, out, work);
+        else k_src_solve5<false><<<(n_src + 127) / 128, 128, 0, stream>>>(st, last, src_off, n_src, out, work);
+    }
+    k_src_final<<<nb, th, 0, stream>>>(st, src_off, src_nal, src_order, n_src, batch, scratch, work, out, rec);
+    k_src_general<<<nb, th, 0, stream>>>(st, src_off, src_order, n_src, out, rec, scratch, work);
 }
 
 void launch_src_geo(int32_t n_src, const double* src, double* geo, cudaStream_t s) {
