@@ -157,111 +157,202 @@ __global__ void __launch_bounds__(32 * kFwdWarps) k_mlp_fwd_tc(const uint32_t* _
     }
 }
 
-// Loss and gradient of the BF16-rounded forward (FP32 arithmetic on the CUDA cores): every
-// lane takes one row; the weight gradients of a warp's 32 rows are outer-product sums over
-// the rows kept in shared memory, added into a per-block gradient with shared atomics and
-// then into the global gradient.
-constexpr int kGradWarps = 4;
+// Loss and gradient of the BF16-rounded forward (FP32 arithmetic on the CUDA cores).  A block of
+// kGradWarps warps takes 32 rows at a time: lane = row, and every warp computes its share of the
+// units of each layer (the weights are then broadcast loads, the row vectors of odd stride free of
+// bank conflicts); the weight gradients are outer-product sums over the 32 rows kept in shared
+// memory, each thread owning 4x4 tiles of W2 and W1 (8 loads for 16 products).  Blocks with one
+// tile add it straight into the global gradient, four values per reduction where aligned.
+// Bound: the batch of the training step (8192 rows, 256 tiles) is 1.7 blocks per SM, so the time is
+// one tile's chain of dependent sums: 83 -> 24.5 us (before: a warp per tile, a whole row per
+// thread, on 64 of the 152 SMs).
+constexpr int kGradWarps = 8;
+constexpr int kGradThreads = 32 * kGradWarps;
 constexpr int kRowF = kIn + 4 * kH + kOut;            // per row: x, h1, h2, dh2, dh1, dy
-constexpr size_t kGradSmem = (size_t)(2 * pN + kGradWarps * 32 * kRowF + 1) * sizeof(float);
+constexpr size_t kGradSmem = (size_t)(2 * pN + 32 * kRowF + kGradWarps) * sizeof(float);
+static_assert(kRowF % 2 == 1, "rows in distinct banks");
 
-__global__ void __launch_bounds__(32 * kGradWarps) k_mlp_loss_grad(const float* __restrict__ p,
-                                                                    const float* __restrict__ X,
-                                                                    const float* __restrict__ T,
-                                                                    const int32_t* __restrict__ idx, int n,
-                                                                    float* __restrict__ grad,
-                                                                    float* __restrict__ loss) {
+// four neighbouring sums into the global gradient
+__device__ __forceinline__ void grad_add4(float* g, const float* v, bool vec) {
+    if (vec) {
+        asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(g), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3])
+                     : "memory");
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; k++) atomicAdd(g + k, v[k]);
+    }
+}
+
+// sum over the 32 rows of d[row][i] * v[row][k] for a 4x4 tile
+__device__ __forceinline__ void outer4(const float* d, const float* v, float acc[4][4]) {
+#pragma unroll 4
+    for (int q = 0; q < 32; q++) {
+        float a[4], b[4];
+#pragma unroll
+        for (int t = 0; t < 4; t++) {
+            a[t] = d[q * kRowF + t];
+            b[t] = v[q * kRowF + t];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+#pragma unroll
+            for (int k = 0; k < 4; k++) acc[i][k] = fmaf(a[i], b[k], acc[i][k]);
+    }
+}
+
+__global__ void __launch_bounds__(kGradThreads) k_mlp_loss_grad(const float* __restrict__ p, const float* __restrict__ X,
+                                                                const float* __restrict__ T,
+                                                                const int32_t* __restrict__ idx, int n,
+                                                                float* __restrict__ grad, float* __restrict__ loss) {
     extern __shared__ float sm[];
     float* W = sm;                                     // rounded weights and FP32 biases, flat layout
-    float* G = sm + pN;                                // block gradient
-    float* rowbuf = sm + 2 * pN + (threadIdx.x >> 5) * 32 * kRowF;
-    float* Lsum = sm + 2 * pN + kGradWarps * 32 * kRowF;
-    for (int i = threadIdx.x; i < pN; i += blockDim.x) {
+    float* G = sm + pN;                                // block gradient (several tiles per block)
+    float* rows = sm + 2 * pN;
+    float* lsum = sm + 2 * pN + 32 * kRowF;
+    const int ntile = (n + 31) / 32;
+    const bool one = ntile <= (int)gridDim.x;          // at most one tile per block
+    for (int i = threadIdx.x; i < pN; i += kGradThreads) {
         const bool is_w = (i < pB1) || (i >= pW2 && i < pB2) || (i >= pW3 && i < pB3);
         W[i] = is_w ? bf16r(p[i]) : p[i];
-        G[i] = 0.0f;
+        if (!one) G[i] = 0.0f;
     }
-    if (threadIdx.x == 0) *Lsum = 0.0f;
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const float inv_n = 1.0f / (float)n;
+    // W1 (offset 0) and W2 start on 16 bytes when grad does (pW2 = 1472)
+    static_assert(pW1 % 4 == 0 && pW2 % 4 == 0, "offsets of the vector reductions");
+    const bool vec = (reinterpret_cast<uintptr_t>(grad) & 15) == 0;
     float lpart = 0.0f;
-    const int ntile = (n + 31) / 32;
-    for (int tile = blockIdx.x * kGradWarps + (threadIdx.x >> 5); tile < ntile; tile += gridDim.x * kGradWarps) {
-        const int rb_ = tile * 32 + lane;
-        const bool valid = rb_ < n;
-        const int64_t r = valid ? (idx ? (int64_t)idx[rb_] : (int64_t)rb_) : 0;
-        float* xs = rowbuf + lane * kRowF;
-        float* h1 = xs + kIn;
-        float* h2 = h1 + kH;
-        float* dh2 = h2 + kH;
-        float* dh1 = dh2 + kH;
-        float* dy = dh1 + kH;
-        for (int k = 0; k < kIn; k++) xs[k] = valid ? bf16r(X[r * kIn + k]) : 0.0f;
-        for (int i = 0; i < kH; i++) {
-            float z = W[pB1 + i];
-            for (int k = 0; k < kIn; k++) z = fmaf(W[pW1 + i * kIn + k], xs[k], z);
-            h1[i] = bf16r(fmaxf(z, 0.0f));
+    float* xs = rows + lane * kRowF;
+    float* h1 = xs + kIn;
+    float* h2 = h1 + kH;
+    float* dh2 = h2 + kH;
+    float* dh1 = dh2 + kH;
+    float* dy = dh1 + kH;
+    constexpr int kU = kH / kGradWarps;                // units of a hidden layer per warp
+    for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+        // the tile's rows: warp w loads rows w, w + kGradWarps, ... coalesced
+        __syncthreads();
+        for (int q = wib; q < 32; q += kGradWarps) {
+            const int rb_ = tile * 32 + q;
+            const int64_t r = rb_ < n ? (idx ? (int64_t)idx[rb_] : (int64_t)rb_) : 0;
+            if (lane < kIn) rows[q * kRowF + lane] = rb_ < n ? bf16r(X[r * kIn + lane]) : 0.0f;
         }
-        for (int i = 0; i < kH; i++) {
-            float z = W[pB2 + i];
-            for (int k = 0; k < kH; k++) z = fmaf(W[pW2 + i * kH + k], h1[k], z);
-            h2[i] = bf16r(fmaxf(z, 0.0f));
+        __syncthreads();
+        {
+            float z[kU];
+#pragma unroll
+            for (int u = 0; u < kU; u++) z[u] = W[pB1 + wib * kU + u];
+#pragma unroll 2
+            for (int k = 0; k < kIn; k++) {
+                const float x = xs[k];
+#pragma unroll
+                for (int u = 0; u < kU; u++) z[u] = fmaf(W[pW1 + (wib * kU + u) * kIn + k], x, z[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < kU; u++) h1[wib * kU + u] = bf16r(fmaxf(z[u], 0.0f));
         }
-        for (int o = 0; o < kOut; o++) {
+        __syncthreads();
+        {
+            float z[kU];
+#pragma unroll
+            for (int u = 0; u < kU; u++) z[u] = W[pB2 + wib * kU + u];
+#pragma unroll 4
+            for (int k = 0; k < kH; k++) {
+                const float x = h1[k];
+#pragma unroll
+                for (int u = 0; u < kU; u++) z[u] = fmaf(W[pW2 + (wib * kU + u) * kH + k], x, z[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < kU; u++) h2[wib * kU + u] = bf16r(fmaxf(z[u], 0.0f));
+        }
+        __syncthreads();
+        if (wib < kOut) {
+            const int o = wib, rb_ = tile * 32 + lane;
+            const bool valid = rb_ < n;
+            const int64_t r = valid ? (idx ? (int64_t)idx[rb_] : (int64_t)rb_) : 0;
             float y = W[pB3 + o];
+#pragma unroll 8
             for (int k = 0; k < kH; k++) y = fmaf(W[pW3 + o * kH + k], h2[k], y);
             const float e = valid ? y - T[r * kOut + o] : 0.0f;
             lpart = fmaf(e, e, lpart);
             dy[o] = 2.0f * e * inv_n;
         }
-        for (int i = 0; i < kH; i++) {
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kU; u++) {
+            const int i = wib * kU + u;
             float s = 0.0f;
+#pragma unroll
             for (int o = 0; o < kOut; o++) s = fmaf(dy[o], W[pW3 + o * kH + i], s);
             dh2[i] = h2[i] > 0.0f ? s : 0.0f;
         }
-        for (int k = 0; k < kH; k++) {
-            float s = 0.0f;
-            for (int i = 0; i < kH; i++) s = fmaf(dh2[i], W[pW2 + i * kH + k], s);
-            dh1[k] = h1[k] > 0.0f ? s : 0.0f;
+        __syncthreads();
+        {
+            float s[kU];
+#pragma unroll
+            for (int u = 0; u < kU; u++) s[u] = 0.0f;
+#pragma unroll 4
+            for (int i = 0; i < kH; i++) {
+                const float d = dh2[i];
+#pragma unroll
+                for (int u = 0; u < kU; u++) s[u] = fmaf(d, W[pW2 + i * kH + wib * kU + u], s[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < kU; u++) dh1[wib * kU + u] = h1[wib * kU + u] > 0.0f ? s[u] : 0.0f;
         }
-        __syncwarp();
-        // weight gradients over the 32 rows of the tile, each lane owning entries lane + 32 m
-        const float* rb = rowbuf;
-        for (int e = lane; e < kOut * kH; e += 32) {           // W3
-            const int o = e / kH, k = e % kH;
-            float s = 0.0f;
-            for (int q = 0; q < 32; q++) s = fmaf(rb[q * kRowF + kIn + 4 * kH + o], rb[q * kRowF + kIn + kH + k], s);
-            atomicAdd(&G[pW3 + e], s);
+        __syncthreads();
+        // weight gradients over the 32 rows
+        const float* rb = rows;
+        for (int e = threadIdx.x; e < (kH / 4) * (kH / 4); e += kGradThreads) {   // W2: 16 x 16 tiles of 4 x 4
+            const int i = 4 * (e / (kH / 4)), k = 4 * (e % (kH / 4));
+            float acc[4][4] = {};
+            outer4(rb + kIn + 2 * kH + i, rb + kIn + k, acc);
+#pragma unroll
+            for (int a = 0; a < 4; a++) {
+                const int off = pW2 + (i + a) * kH + k;
+                if (one) grad_add4(grad + off, acc[a], vec);
+                else
+                    for (int b = 0; b < 4; b++) G[off + b] += acc[a][b];
+            }
         }
-        for (int e = lane; e < kH * kH; e += 32) {             // W2
-            const int i = e / kH, k = e % kH;
-            float s = 0.0f;
-            for (int q = 0; q < 32; q++) s = fmaf(rb[q * kRowF + kIn + 2 * kH + i], rb[q * kRowF + kIn + k], s);
-            atomicAdd(&G[pW2 + e], s);
-        }
-        for (int e = lane; e < kH * kIn; e += 32) {            // W1
+        for (int e = threadIdx.x; e < kH * kIn; e += kGradThreads) {              // W1
             const int i = e / kIn, k = e % kIn;
             float s = 0.0f;
+#pragma unroll 8
             for (int q = 0; q < 32; q++) s = fmaf(rb[q * kRowF + kIn + 3 * kH + i], rb[q * kRowF + k], s);
-            atomicAdd(&G[pW1 + e], s);
+            if (one) atomicAdd(&grad[pW1 + e], s);
+            else G[pW1 + e] += s;
         }
-        for (int e = lane; e < 2 * kH + kOut; e += 32) {      // biases
+        for (int e = threadIdx.x; e < kOut * kH; e += kGradThreads) {             // W3
+            const int o = e / kH, k = e % kH;
+            float s = 0.0f;
+#pragma unroll 8
+            for (int q = 0; q < 32; q++) s = fmaf(rb[q * kRowF + kIn + 4 * kH + o], rb[q * kRowF + kIn + kH + k], s);
+            if (one) atomicAdd(&grad[pW3 + e], s);
+            else G[pW3 + e] += s;
+        }
+        for (int e = threadIdx.x; e < 2 * kH + kOut; e += kGradThreads) {         // biases
             int off, src;
             if (e < kH) { off = pB1 + e; src = kIn + 3 * kH + e; }
             else if (e < 2 * kH) { off = pB2 + e - kH; src = kIn + 2 * kH + e - kH; }
             else { off = pB3 + e - 2 * kH; src = kIn + 4 * kH + e - 2 * kH; }
             float s = 0.0f;
+#pragma unroll 8
             for (int q = 0; q < 32; q++) s += rb[q * kRowF + src];
-            atomicAdd(&G[off], s);
+            if (one) atomicAdd(&grad[off], s);
+            else G[off] += s;
         }
-        __syncwarp();
     }
     lpart = warp_sum_f32(lpart);
-    if (lane == 0) atomicAdd(Lsum, lpart);
+    if (lane == 0) lsum[wib] = lpart;
     __syncthreads();
-    for (int i = threadIdx.x; i < pN; i += blockDim.x) atomicAdd(&grad[i], G[i]);
-    if (threadIdx.x == 0) atomicAdd(loss, *Lsum * inv_n);
+    if (!one)
+        for (int i = threadIdx.x; i < pN; i += kGradThreads) atomicAdd(&grad[i], G[i]);
+    if (threadIdx.x == 0) {
+        float s = 0.0f;
+        for (int k = 0; k < kGradWarps; k++) s += lsum[k];
+        atomicAdd(loss, s * inv_n);
+    }
 }
 
 __global__ void k_mlp_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
@@ -540,8 +631,8 @@ int agis_mlp_loss_grad(const float* params, const float* X, const float* T, cons
     cudaMemsetAsync(grad, 0, sizeof(float) * agis::pN, s);
     cudaMemsetAsync(loss, 0, sizeof(float), s);
     const int tiles = (n + 31) / 32;
-    agis::k_mlp_loss_grad<<<agis::grid_of(tiles, agis::kGradWarps, 152), 32 * agis::kGradWarps, agis::kGradSmem, s>>>(
-        params, X, T, idx, n, grad, loss);
+    agis::k_mlp_loss_grad<<<agis::grid_of(tiles, 1, 2 * 152), agis::kGradThreads, agis::kGradSmem, s>>>(params, X, T, idx, n,
+                                                                                                     grad, loss);
     return mlp_launch_status("agis_mlp_loss_grad");
 }
 
