@@ -317,21 +317,7 @@ __device__ __noinline__ void solve_general(const Settings& st, int i, int64_t o0
 // ---------------------------------------------------------------------------------------
 // class-sum path (one sigma per class and source)
 // ---------------------------------------------------------------------------------------
-constexpr int kSumVals = 21;       // 15 AA, 5 Ah, hh of one class
 constexpr int kPassWarps = 4;      // warps per block of the passes over the rows
-constexpr int kKeyCap64 = 1024;    // keys of a source kept in shared memory
-constexpr int kSelCap = 96;        // keys around a quantile that are ranked directly
-
-// float of a double by its bit pattern, truncated (relative error below 2^-23): values below the
-// FP32 range are 0, above it (and NaN) infinite.  Integer instructions: a conversion holds the
-// FP64 unit.
-__device__ __forceinline__ float trunc_f32(double x) {
-    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-    const uint32_t ex = (hi >> 20) & 0x7ffu;
-    uint32_t f = __funnelshift_l(lo, hi, 3) ^ 0x40000000u;   // exponent - 896, 23 bits of the significand
-    f = ex < 897u ? 0u : (ex > 1150u ? 0x7f800000u : f & 0x7fffffffu);
-    return __uint_as_float(f | (hi & 0x80000000u));
-}
 
 // Sums of kSumVals lane values over the warp by recursive halving: in each step a lane gives one
 // half of its values to its partner and adds the partner's other half, 23 additions instead of
@@ -356,19 +342,6 @@ __device__ __forceinline__ void reduce_vals(double* v, int lane, double* out) {
     step(std::integral_constant<int, 3>{}, 2);
     step(std::integral_constant<int, 2>{}, 1);
     if (cnt > 0) out[off] = v[0];
-}
-
-__device__ __forceinline__ void row_load(const double* __restrict__ e, double& h, double A[5]) {
-    const double2 a = *reinterpret_cast<const double2*>(e), b = *reinterpret_cast<const double2*>(e + 2),
-                  c = *reinterpret_cast<const double2*>(e + 4);
-    h = a.x; A[0] = a.y; A[1] = b.x; A[2] = b.y; A[3] = c.x; A[4] = c.y;
-}
-__device__ __forceinline__ double row_dot(const double A[5], const double* d) {
-    double Ad = A[0] * d[0];
-    Ad = fma(A[1], d[1], Ad);
-    Ad = fma(A[2], d[2], Ad);
-    Ad = fma(A[3], d[3], Ad);
-    return fma(A[4], d[4], Ad);
 }
 
 // What a round subtracts from the unit-weight sums of one class: (1 - w) times the products of
@@ -396,63 +369,6 @@ __device__ __forceinline__ void subtract_rows(double* scr, const uint32_t* list,
     corr[20] = fma(u * h, h, corr[20]);
 }
 
-// Direct class sums of one round: every row weighted (w = wfun(h rx) first, wfun((h - A d) isd)
-// later, 1 for plain weights), lane partials over the rows lane, lane + 32, ... of each class to
-// red[value][lane], then lane v adds the 32 partials of value v in lane order.  last: w goes to
-// the scratch row for the hand-over records.
-constexpr int kRedVals = 2 * kSumVals;
-constexpr int kRedStride = 33;    // doubles per value row (odd: the column sums read distinct banks)
-__device__ __forceinline__ void direct_sums(double* scr, int n, int nal, int lane, int mode, const double* rx,
-                                            const double* isd, const double* d, int wfn, bool last, double* red,
-                                            double* out, int& nout) {
-    int cnt = 0;
-    for (int c = 0; c < 2; c++) {
-        const int hi = c ? n : nal;
-        double AA[15], Ah[5], hs = 0.0;
-#pragma unroll
-        for (int i = 0; i < 15; i++) AA[i] = 0.0;
-#pragma unroll
-        for (int i = 0; i < 5; i++) Ah[i] = 0.0;
-        for (int j = (c ? nal : 0) + lane; j < hi; j += kWarp) {
-            double* e = scr + (size_t)j * kScr;
-            double h, A[5];
-            row_load(e, h, A);
-            double w = 1.0;
-            if (mode == 0) {
-                if (rx[c] > 0.0) w = wfun(h * rx[c], wfn);
-            } else if (mode == 1) {
-                w = wfun((h - row_dot(A, d)) * isd[c], wfn);
-            }
-            if (last) e[6] = w;
-            cnt += (w < 0.2);
-#pragma unroll
-            for (int a = 0; a < 5; a++) {
-                const double wa = w * A[a];
-#pragma unroll
-                for (int b = a; b < 5; b++) AA[up5(a, b)] += wa * A[b];
-                Ah[a] += wa * h;
-            }
-            hs += w * h * h;
-        }
-        double* rc = red + c * kSumVals * kRedStride;
-#pragma unroll
-        for (int i = 0; i < 15; i++) rc[i * kRedStride + lane] = AA[i];
-#pragma unroll
-        for (int i = 0; i < 5; i++) rc[(15 + i) * kRedStride + lane] = Ah[i];
-        rc[20 * kRedStride + lane] = hs;
-    }
-    nout = warp_sum_int(cnt);
-    __syncwarp();
-    for (int v = lane; v < kRedVals; v += kWarp) {
-        const double* col = red + v * kRedStride;
-        double t = col[0];
-#pragma unroll
-        for (int k = 1; k < kWarp; k++) t += col[k];
-        out[v] = t;
-    }
-    __syncwarp();
-}
-
 // Appends the row j of every lane with cand set to the list (n entries so far); a full list of 32
 // is worked off by `flush`.
 template <class F>
@@ -468,99 +384,6 @@ __device__ __forceinline__ void append_rows(bool cand, int j, uint32_t* list, in
     __syncwarp();
     if (cand && pos >= 32) list[pos - 32] = (uint32_t)j;
     n -= 32;
-}
-
-// The k-th and (k+1)-th smallest keys (k + 1 capped at n - 1) for k = k1 and k = k5 at once: a
-// histogram of the values on 256 equal steps between their extremes finds the steps that hold
-// those ranks, and the few keys in them are ranked against one another.  False if a step holds
-// too many keys (heavy ties, a wild outlier) or a value is not finite: the caller then uses the
-// radix select.
-struct SelWork {
-    uint64_t keys[kKeyCap64];
-    int hist[256];
-    uint64_t list[2][kSelCap];
-    uint64_t res[4];
-    int cnt[2];
-};
-__device__ bool select_quantiles(const uint64_t* __restrict__ keys, int n, int k1, int k5, float lo, float hi,
-                                 SelWork& sw, int lane, double out[4]) {
-    if (!(hi > lo) || !isfinite(lo) || !isfinite(hi)) return false;
-    const float scale = 256.0f / (hi - lo);
-    if (!isfinite(scale)) return false;
-#pragma unroll
-    for (int i = 0; i < 8; i++) sw.hist[lane + 32 * i] = 0;
-    if (lane < 2) sw.cnt[lane] = 0;
-    __syncwarp();
-    auto bin_of = [&](uint64_t key) {
-        const int b = (int)((trunc_f32(dkey_inv(key)) - lo) * scale);   // never decreasing in the key
-        return b > 255 ? 255 : b;
-    };
-    for (int j = lane; j < n; j += kWarp) atomicAdd(&sw.hist[bin_of(keys[j])], 1);
-    __syncwarp();
-    int c[8], tot = 0;
-#pragma unroll
-    for (int i = 0; i < 8; i++) { c[i] = sw.hist[lane * 8 + i]; tot += c[i]; }
-    int incl = tot;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    // the steps of ranks k1, k1 + 1, k5, k5 + 1 and the keys below the first of each pair
-    int bin[4], below[4];
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-        int k = (q < 2 ? k1 : k5) + (q & 1);
-        if (k > n - 1) k = n - 1;
-        const unsigned ball = __ballot_sync(0xffffffffu, incl > k);
-        const int sl = __ffs(ball) - 1;
-        int acc = incl - tot, bs = 7;
-#pragma unroll
-        for (int i = 0; i < 8; i++) {
-            if (bs == 7 && acc + c[i] > k) bs = i + 8;
-            if (bs < 8) acc += c[i];
-        }
-        if (bs == 7) acc -= c[7];   // not reached for the chosen lane
-        bin[q] = __shfl_sync(0xffffffffu, lane * 8 + (bs & 7), sl);
-        below[q] = __shfl_sync(0xffffffffu, acc, sl);
-    }
-    bool ok = true;
-#pragma unroll
-    for (int p = 0; p < 2; p++) {
-        const int m = sw.hist[bin[2 * p]] + (bin[2 * p + 1] != bin[2 * p] ? sw.hist[bin[2 * p + 1]] : 0);
-        ok = ok && m <= kSelCap;
-    }
-    if (!ok) return false;
-    for (int j = lane; j < n; j += kWarp) {
-        const uint64_t key = keys[j];
-        const int b = bin_of(key);
-        if (b >= bin[0] && b <= bin[1]) sw.list[0][atomicAdd(&sw.cnt[0], 1)] = key;
-        if (b >= bin[2] && b <= bin[3]) sw.list[1][atomicAdd(&sw.cnt[1], 1)] = key;
-    }
-    __syncwarp();
-#pragma unroll
-    for (int p = 0; p < 2; p++) {
-        const int m = sw.cnt[p];
-        const int t0 = (p ? k5 : k1) - below[2 * p];
-        const int t1 = (p ? k5 : k1) + 1 > n - 1 ? t0 : t0 + 1;
-        for (int a = lane; a < m; a += kWarp) {
-            const uint64_t key = sw.list[p][a];
-            int less = 0, eq = 0;
-            for (int b = 0; b < m; b++) {
-                const uint64_t o = sw.list[p][b];
-                less += o < key;
-                eq += o == key;
-            }
-            // this value holds the ranks less .. less + eq - 1
-            if (t0 >= less && t0 < less + eq) sw.res[2 * p] = key;
-            if (t1 >= less && t1 < less + eq) sw.res[2 * p + 1] = key;
-        }
-    }
-    __syncwarp();
-#pragma unroll
-    for (int q = 0; q < 4; q++) out[q] = dkey_inv(sw.res[q]);
-    __syncwarp();
-    return true;
 }
 
 // Per source: sigma per class, robust scale of x = h / sigma (Sect. 5.1.2: half the intersextile
@@ -818,41 +641,6 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_round_direct(Settings s
                         st.weight_fn, last, red_all[wib], &w.T[0][0], nout);
             if (lane == 0) w.nout = nout;
         }
-}
-
-// class_solve by two neighbouring lanes of a warp: each forms half of the 15 + 5 entries of N and b,
-// both factor and solve, and each sums Q's numerator of one class.  Every value is formed by the
-// operations of class_solve in their order.
-struct HalfSums {
-    double E[2][10];             // entries 10 h .. 10 h + 9 of (AA, Ah) of both classes
-    double AA[15], Ah[5], hh;    // class h
-};
-__device__ __forceinline__ double lane_pair(double v) { return __shfl_xor_sync(0xffffffffu, v, 1); }
-static __device__ __noinline__ void class_solve_pair(const HalfSums& S, int h, const double* s2c, double y, double tol_piv,
-                                                     double* U, double* d, int& rd, double& Q, double& S2) {
-    const double im = 1.0 / (s2c[h] + y), io = lane_pair(im);
-    const double i0 = h ? io : im, i1 = h ? im : io;
-    double NB[20];
-#pragma unroll
-    for (int k = 0; k < 10; k++) {
-        const double v = S.E[0][k] * i0 + S.E[1][k] * i1, o = lane_pair(v);
-        NB[k] = h ? o : v;
-        NB[10 + k] = h ? v : o;
-    }
-    rd = chol5(NB, U, tol_piv);
-    chol5_solve(U, NB + 15, d);
-    double dMd = 0.0, db = 0.0;
-#pragma unroll
-    for (int a = 0; a < 5; a++) {
-        db += d[a] * S.Ah[a];
-        dMd += S.AA[up5(a, a)] * d[a] * d[a];
-#pragma unroll
-        for (int k = a + 1; k < 5; k++) dMd += 2.0 * S.AA[up5(a, k)] * d[a] * d[k];
-    }
-    const double nm = S.hh - 2.0 * db + dMd, no = lane_pair(nm);
-    const double num[2] = {h ? no : nm, h ? nm : no};
-    Q = num[0] * i0 + num[1] * i1;
-    S2 = num[0] * i0 * i0 + num[1] * i1 * i1;
 }
 
 // the 5x5 algebra of one round, one thread (kPair: two neighbouring lanes) per source: y = 0 first,

@@ -210,18 +210,46 @@ __global__ void k_static_check(int64_t n_obs, ObsPtrs ob, int32_t n_src, int cap
     if (bad) atomicOr(&ctrl[1], bad);
 }
 
+// the updated parameters and the statistics of one source
+__device__ __forceinline__ void write_static(double* src, double* stats, int32_t n_src, int i, const double* s5,
+                                             double cosd, const double* d, double y, double Q, double Q0, int nu,
+                                             int nout) {
+    double* sp = src + 5 * (size_t)i;
+    sp[0] = s5[0] + d[0] / cosd;
+    for (int k = 1; k < 5; k++) sp[k] = s5[k] + d[k];
+    if (!stats) return;
+    stats[i] = y;
+    stats[(size_t)n_src + i] = Q;
+    stats[2 * (size_t)n_src + i] = (double)nu;
+    stats[3 * (size_t)n_src + i] = (double)nout;
+    stats[4 * (size_t)n_src + i] = nu > 0 ? (Q0 - (double)nu) / sqrt(2.0 * (double)nu) : 0.0;
+}
+
 // One warp per source: observation pass into the warp's slice of the static scratch, then the
-// inner iteration of Sect. 5.1.2 (per-observation form) and the outputs.
+// inner iteration of Sect. 5.1.2 and the outputs.  Where the AL and the AC observations of the
+// source have one sigma each, the rows are laid out AL first and the inner iteration works on
+// class sums (one pass over the rows per round, the 5x5 algebra by pairs of lanes); otherwise every
+// excess-noise step passes over the rows.
+// Bound: FP64 issue (64 cycles of a sub-partition per warp instruction).  2000 sources of 140
+// observations: 2.58 -> 1.29 ms (before: per-observation passes, two divisions each, for every step,
+// and 8-digit radix selects over the strided rows).
 __global__ void __launch_bounds__(128) k_source_static(DevGeo G, Settings st, ObsPtrs ob, int64_t n_obs,
                                                        int32_t n_src, CcdRows rows, int64_t cal_t0, int64_t cal_dt,
                                                        int32_t n_days, double* __restrict__ src,
                                                        const double* __restrict__ att, const double* __restrict__ cal,
                                                        double* __restrict__ R_out, double* __restrict__ W_out,
                                                        double* __restrict__ stats, int cap, double* scratch, int* ctrl) {
-    __shared__ int hist_all[4 * 256];
+    union WarpWork {
+        SelWork sel;
+        double red[kRedVals * kRedStride];
+    };
+    __shared__ __align__(16) unsigned char work_raw[4 * sizeof(WarpWork)];
+    __shared__ double sums_all[4][kRedVals];
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
-    int* hist = hist_all + wib * 256;
+    WarpWork& ww = reinterpret_cast<WarpWork*>(work_raw)[wib];
+    double* sums = sums_all[wib];
+    int* hist = ww.sel.hist;
     const size_t gw = (size_t)blockIdx.x * (blockDim.x >> 5) + wib;
     double* scr = scratch + gw * (size_t)cap * kScr;
     for (;;) {
@@ -246,8 +274,39 @@ __global__ void __launch_bounds__(128) k_source_static(DevGeo G, Settings st, Ob
         }
         SrcGeo S;
         source_geo(s5, S);
+        // one sigma per class?  and the AL observations, whose rows come first if so
         double s2min = 1e300;
+        float slo[2] = {INFINITY, INFINITY}, shi[2] = {0.0f, 0.0f};
+        int nal = 0;
         for (int j = lane; j < n; j += kWarp) {
+            const int k = ob.kind[o0 + j] ? 1 : 0;
+            const float sg = ob.sigma[o0 + j];
+            slo[k] = fminf(slo[k], sg);
+            shi[k] = fmaxf(shi[k], sg);
+            nal += !k;
+        }
+        nal = warp_sum_int(nal);
+#pragma unroll
+        for (int c = 0; c < 2; c++)
+#pragma unroll
+            for (int m = 16; m > 0; m >>= 1) {
+                slo[c] = fminf(slo[c], __shfl_xor_sync(0xffffffffu, slo[c], m));
+                shi[c] = fmaxf(shi[c], __shfl_xor_sync(0xffffffffu, shi[c], m));
+            }
+        const bool uni = (nal == 0 || slo[0] == shi[0]) && (nal == n || slo[1] == shi[1]);
+        int at[2] = {0, nal};   // next row of each class
+        for (int j0 = 0; j0 < n; j0 += kWarp) {
+            const int j = j0 + lane;
+            int row = j;
+            if (uni) {
+                const int k = j < n ? (ob.kind[o0 + j] ? 1 : 0) : 2;
+                const unsigned b0 = __ballot_sync(0xffffffffu, k == 0), b1 = __ballot_sync(0xffffffffu, k == 1);
+                const unsigned below = (1u << lane) - 1u;
+                row = k ? at[1] + __popc(b1 & below) : at[0] + __popc(b0 & below);
+                at[0] += __popc(b0);
+                at[1] += __popc(b1);
+            }
+            if (j >= n) continue;
             const int64_t o = o0 + j;
             const int c = ob.ccd[o], f = ob.fov[o], k = ob.kind[o];
             const int64_t t = ob.t_ns[o];
@@ -260,24 +319,93 @@ __global__ void __launch_bounds__(128) k_source_static(DevGeo G, Settings st, Ob
             ObsOut oo;
             observe<1>(G, S, t, m, k ? ob.mu[o] : 0.0, att, cal, oo);
             const double sg = (double)ob.sigma[o];
-            double* e = scr + (size_t)j * kScr;
+            double* e = scr + (size_t)row * kScr;
             e[0] = oo.R;
             e[1] = oo.A[0]; e[2] = oo.A[1]; e[3] = oo.A[2]; e[4] = oo.A[3]; e[5] = oo.A[4];
-            e[6] = __longlong_as_double((long long)skey(oo.R / sg));
-            e[7] = sg * sg;
+            const uint64_t key = skey(oo.R * rcp_pos(sg));
+            e[6] = __longlong_as_double((long long)key);
+            if (n <= kKeyCap64) ww.sel.keys[j] = key;
+            e[7] = uni ? __longlong_as_double((long long)j) : sg * sg;   // class path: the row's observation
             s2min = fmin(s2min, sg * sg);
         }
         s2min = warp_min(s2min);
         __syncwarp();
+        double vs = 0.0;
         if (st.robust) {
             const double p1 = 1.0 / 6.0, p5 = 5.0 / 6.0;
             const double h1 = p1 * (double)(n - 1), h5 = p5 * (double)(n - 1);
             const int lo1 = (int)floor(h1), lo5 = (int)floor(h5);
-            double a0, a1, b0, b1;
-            s_select_pair(scr, n, lo1, hist, lane, a0, a1);
-            s_select_pair(scr, n, lo5, hist, lane, b0, b1);
-            const double vs = 0.5 * ((b0 + (h5 - lo5) * (b1 - b0)) - (a0 + (h1 - lo1) * (a1 - a0)));
+            double q[4];
+            bool done = false;
+            if (n <= kKeyCap64) {
+                float lo = INFINITY, hi = -INFINITY;
+                bool bad = false;
+                for (int j = lane; j < n; j += kWarp) {
+                    const float x = trunc_f32(skey_inv(ww.sel.keys[j]));
+                    bad = bad || !isfinite(x);
+                    lo = fminf(lo, x);
+                    hi = fmaxf(hi, x);
+                }
+#pragma unroll
+                for (int m = 16; m > 0; m >>= 1) {
+                    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, m));
+                    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, m));
+                }
+                done = !__any_sync(0xffffffffu, bad) && select_quantiles(ww.sel.keys, n, lo1, lo5, lo, hi, ww.sel, lane, q);
+            }
+            if (!done) {
+                s_select_pair(scr, n, lo1, hist, lane, q[0], q[1]);
+                s_select_pair(scr, n, lo5, hist, lane, q[2], q[3]);
+            }
+            vs = 0.5 * ((q[2] + (h5 - lo5) * (q[3] - q[2])) - (q[0] + (h1 - lo1) * (q[1] - q[0])));
             __syncwarp();
+        }
+        if (uni) {
+            // class sums: AL rows [0, nal), AC rows [nal, n)
+            const double s2c[2] = {nal > 0 ? (double)slo[0] * (double)slo[0] : 1.0,
+                                   nal < n ? (double)slo[1] * (double)slo[1] : 1.0};
+            double rx[2], isd[2] = {0.0, 0.0}, d[5] = {0, 0, 0, 0, 0}, U[kU5];
+            for (int c = 0; c < 2; c++) rx[c] = vs > 0.0 ? 1.0 / (sqrt(s2c[c]) * vs) : 0.0;
+            double y = 0.0, Q = 0.0, Q0 = 0.0, S2 = 0.0;
+            int nu = 0, nout = 0, rdc = 0;
+            const int rounds = st.robust ? st.n_rounds + 1 : 1, h = lane & 1;
+            for (int rnd = 0; rnd < rounds; rnd++) {
+                direct_sums(scr, n, nal, lane, !st.robust ? 2 : (rnd ? 1 : 0), rx, isd, d, st.weight_fn,
+                            rnd == rounds - 1, ww.red, sums, nout);
+                HalfSums H;
+                for (int c = 0; c < 2; c++)
+                    for (int k = 0; k < 10; k++) H.E[c][k] = sums[kSumVals * c + 10 * h + k];
+                for (int k = 0; k < 15; k++) H.AA[k] = sums[kSumVals * h + k];
+                for (int k = 0; k < 5; k++) H.Ah[k] = sums[kSumVals * h + 15 + k];
+                H.hh = sums[kSumVals * h + 20];
+                __syncwarp();
+                nu = n - nout - 5;
+                y = 0.0;
+                class_solve_pair(H, h, s2c, 0.0, st.pivot_tol, U, d, rdc, Q, S2);
+                Q0 = Q;
+                if (st.robust && nu > 0 && Q0 > (double)nu) {   // the same in every lane
+                    const double tol = 1e-12 * s2min;
+                    for (int it = 0; it < st.n_eps; it++) {
+                        const double dy = (1.0 - Q / (double)nu) * Q / (-S2);
+                        y = fmax(0.0, y + dy);
+                        class_solve_pair(H, h, s2c, y, st.pivot_tol, U, d, rdc, Q, S2);
+                        if (fabs(dy) <= tol) break;
+                    }
+                }
+                for (int c = 0; c < 2; c++) isd[c] = 1.0 / sqrt(s2c[c] + y);
+            }
+            const double iw[2] = {1.0 / (s2c[0] + y), 1.0 / (s2c[1] + y)};
+            for (int j = lane; j < n; j += kWarp) {
+                const double* e = scr + (size_t)j * kScr;
+                const int64_t o = o0 + __double_as_longlong(e[7]);
+                if (R_out) R_out[o] = e[0] - (e[1] * d[0] + e[2] * d[1] + e[3] * d[2] + e[4] * d[3] + e[5] * d[4]);
+                if (W_out) W_out[o] = e[6] * (j < nal ? iw[0] : iw[1]);
+            }
+            if (lane == 0) write_static(src, stats, n_src, i, s5, S.cosd, d, y, Q, Q0, nu, nout);
+            __syncwarp();
+            continue;
+        }
+        if (st.robust) {
             for (int j = lane; j < n; j += kWarp) {
                 double* e = scr + (size_t)j * kScr;
                 const double x = e[0] / sqrt(e[7]);
@@ -321,21 +449,7 @@ __global__ void __launch_bounds__(128) k_source_static(DevGeo G, Settings st, Ob
             if (R_out) R_out[o0 + j] = R;
             if (W_out) W_out[o0 + j] = e[6] / (e[7] + y);
         }
-        if (lane == 0) {
-            double* sp = src + 5 * (size_t)i;
-            sp[0] = s5[0] + d[0] / S.cosd;
-            sp[1] = s5[1] + d[1];
-            sp[2] = s5[2] + d[2];
-            sp[3] = s5[3] + d[3];
-            sp[4] = s5[4] + d[4];
-            if (stats) {
-                stats[i] = y;
-                stats[(size_t)n_src + i] = Q;
-                stats[2 * (size_t)n_src + i] = (double)nu;
-                stats[3 * (size_t)n_src + i] = (double)nout;
-                stats[4 * (size_t)n_src + i] = nu > 0 ? (Q0 - (double)nu) / sqrt(2.0 * (double)nu) : 0.0;
-            }
-        }
+        if (lane == 0) write_static(src, stats, n_src, i, s5, S.cosd, d, y, Q, Q0, nu, nout);
         __syncwarp();
     }
 }
