@@ -58,6 +58,7 @@ void launch_asi(int32_t n_src, int32_t stride, const double* hist, double lam_ma
 void launch_calgen(const DevGeo& G, int64_t n_groups, const ObsRec* rec, const double* mu, const CalGenWork& w,
                    double tol, double* cal, cudaStream_t s);
 int calgen_prepare();
+bool calgen_in_smem(int n_bin);
 void launch_cal_sums(int n_cal, const uint32_t* perm_c, const int64_t* cal_off, const ObsRec* rec, double* sums,
                      const Shapes& sh, cudaStream_t s);
 void launch_cal_from_sums(int n_cal, int n_days, const double* sums, double tol, double* dtil, int* rd, double* cal,
@@ -1006,12 +1007,17 @@ int agis_init(const agis_geometry* geo, const agis_config* cfg, const agis_obs* 
             if ((rc = dalloc(c, &perm, n)) || (rc = dalloc(c, &off, (size_t)(ncell + ng + 1))) ||
                 (rc = dalloc(c, &w.V, (size_t)ncell * 6 * nb)) || (rc = dalloc(c, &w.E, (size_t)ncell * nb)) ||
                 (rc = dalloc(c, &w.bs, (size_t)ncell * nb)) || (rc = dalloc(c, &w.cw, (size_t)ncell * 18)) ||
-                (rc = dalloc(c, &w.S, (size_t)ng * nb * nb)) || (rc = dalloc(c, &w.r, (size_t)ng * nb)) ||
-                (rc = dalloc(c, &w.Et, (size_t)ng * nb)) || (rc = dalloc(c, &w.H, (size_t)ng * 3 * nb)) ||
-                (rc = dalloc(c, &w.v, (size_t)ng * nb)) || (rc = dalloc(c, &w.idx, (size_t)ng * nb)) ||
-                (rc = dalloc(c, &cc2, 3 * (size_t)nb)) || (rc = dalloc(c, &w.d, (size_t)n_cal)) ||
+                (rc = dalloc(c, &w.v, (size_t)ng * nb)) || (rc = dalloc(c, &cc2, 3 * (size_t)nb)) || (rc = dalloc(c, &w.d, (size_t)n_cal)) ||
                 (rc = dalloc(c, &w.rd, (size_t)(ncell + 2 * ng))))
                 return bail(rc);
+            if (calgen_in_smem(nb)) {
+                if ((rc = dalloc(c, &w.bins, (size_t)ncell * nb)) || (rc = dalloc(c, &w.nbin, (size_t)ncell)))
+                    return bail(rc);
+            } else if ((rc = dalloc(c, &w.S, (size_t)ng * nb * nb)) || (rc = dalloc(c, &w.r, (size_t)ng * nb)) ||
+                       (rc = dalloc(c, &w.Et, (size_t)ng * nb)) || (rc = dalloc(c, &w.H, (size_t)ng * 3 * nb)) ||
+                       (rc = dalloc(c, &w.idx, (size_t)ng * nb))) {
+                return bail(rc);
+            }
             // cc2 weights: sum of L*_r((m + 14 - 13.5) / n_col) over the columns m of each bin
             std::vector<double> hw(3 * (size_t)nb, 0.0);
             for (int m = 0; m < AGIS_N_COL; m++) {

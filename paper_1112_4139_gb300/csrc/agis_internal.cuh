@@ -480,11 +480,14 @@ struct CalGenWork {
     double* V;                 // AL cell: 6 x n_bin, V_j = U_j'^-1 B_j
     double* E;                 // AL cell: n_bin, sum W per bin
     double* bs;                // AL cell: n_bin, -sum W R per bin
+    uint16_t* bins;            // AL cell: its observed bins, ascending (null: V, E and bs by bin, zeros
+    int* nbin;                 // elsewhere); their number: V, E and bs then hold those bins alone
     double* cw;                // AL cell: 18 = w_j (6) and the two upper 3x3 factors (6 + 6)
     double* S;                 // AL group: n_bin x n_bin reduced normals
     double* r;                 // AL group: n_bin reduced right-hand side
     double* Et;                // AL group: n_bin, sum of E over the group's cells
     double* H;                 // AL group: 3 x n_bin Householder vectors of the cc2 columns
+                               // (S, r, Et, H and idx only without bins: else in shared memory)
     double* v;                 // AL group: n_bin small-scale update
     int* idx;                  // AL group: n_bin observed bins (compacted)
     const double* cc2w;        // 3 x n_bin: sum of L*_r over the columns of each bin
