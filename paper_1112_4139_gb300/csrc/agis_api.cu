@@ -23,7 +23,7 @@ void launch_evaluate(const DevGeo& G, const int64_t* t_ns, const uint32_t* meta,
                      const int32_t* obs_src, int64_t n_obs, const double* src, const double* att, const double* cal,
                      double* R, cudaStream_t stream);
 void launch_att_accum(const DevGeo& G, double lambda2, int rhs_norm, const uint32_t* perm_t, const int64_t* ivl_off,
-                      int n_iv, const ObsRec* rec, const double* w_att, const double* att, double* blk,
+                      int n_iv, const ObsRec* rec, const double* w_att, const double* att, double* blk, bool moments,
                       const Shapes& sh, cudaStream_t s);
 void launch_att_solve(int n_seg, int max_seg_knots, int n_coef, int64_t n_rows, const int64_t* seg_row, const int32_t* seg_l,
                       const int32_t* seg_n, const int32_t* seg_u, const double* blk, double* bandc, double* rhs,
@@ -317,6 +317,7 @@ struct agis_ctx {
     int64_t* ivl_off = nullptr;
     int n_iv = 0;
     double* blk = nullptr;
+    bool att_moments = false;    // interval blocks by moments on the tensor cores
     int n_seg = 0;
     int max_seg_knots = 0;   // the largest segment's coefficients (band rows / 4)
     int64_t n_rows = 0;
@@ -599,7 +600,7 @@ void enqueue_a(agis_ctx* c) {
                              c->att, c->blk, c->sh, c->stream);
     } else
         launch_att_accum(c->G, c->st.lambda2, c->st.rhs_norm_term, c->perm_t, c->ivl_off, c->n_iv,
-                         c->rec, c->an.eps2 ? c->an_w : nullptr, c->att, c->blk, c->sh, c->stream);
+                         c->rec, c->an.eps2 ? c->an_w : nullptr, c->att, c->blk, c->att_moments, c->sh, c->stream);
     launch_att_solve(c->n_seg, c->max_seg_knots, c->n_coef, c->n_rows, c->seg_row, c->seg_l, c->seg_n, c->seg_u, c->blk, c->bandc,
                      c->rhs, c->urow, c->yv, c->xs, c->st.pivot_tol, c->seg_rd, c->att, c->mixed ? c->d_att : nullptr,
                      c->datt64, c->stream);
@@ -1051,12 +1052,16 @@ int agis_init(const agis_geometry* geo, const agis_config* cfg, const agis_obs* 
     c->mixed = cfg->precision == 1;
     // FP64 S block: weight rounds by corrections to unit-weight sums (long sources: 30,000 of 820
     // observations 1.4 + 4 x 0.49 ms a source update, against 1.85 + 4 x 1.88 ms for the direct sums
-    // of every row) or by direct sums.  Short sources gain less (3000 of 165: 80 + 4 x 36 us against
-    // 93 + 4 x 81), and where the knot intervals hold few observations too, the attitude is so weakly
-    // determined along the coefficient vector that another rounding of the weights (1e-15) shows in
-    // the next iteration (calibration 1.1e-9 of its norm at 56 observations per interval, 0.8e-9 at
-    // 156): both keep the direct sums.
-    c->src_corr = n >= 512 * (int64_t)n_src && n >= 100 * (int64_t)c->n_iv;
+    // of every row) or by direct sums (short sources gain less: 3000 of 165 80 + 4 x 36 us against
+    // 93 + 4 x 81).  FP64 A block: interval blocks by moments (24.7M observations in 157,786 intervals
+    // 9.93 -> 2.95 ms, 7.1M in 131,490 3.06 -> 1.51) or by the sums of the products.
+    // Both first forms round otherwise (no worse against 64 bits), which turns the last bit of 10 to 20%
+    // of the attitude coefficients, and the next iteration's calibration averages those bits: measured
+    // 4.5e-9 / sqrt(n / 1e6) of its norm, 1.4e-9 at 4.4M observations, 0.9e-9 at 24.7M in
+    // intervals of 100 or more.  Smaller sets keep the sums' order, so that their iterations reproduce bit
+    // for bit; but for many short intervals, whose coefficients the data determine to 1e-13 only.
+    c->src_corr = n >= 23000000 && n >= 512 * (int64_t)n_src && n >= 100 * (int64_t)c->n_iv;
+    c->att_moments = c->src_corr || (c->n_iv >= 120000 && n < 64 * (int64_t)c->n_iv);
     if (c->mixed) {
         if ((rc = dalloc(c, &c->mo.s, n)) || (rc = dalloc(c, &c->mo.r, n)) || (rc = dalloc(c, &c->mo.ac, n)) ||
             (rc = dalloc(c, &c->mo.t, n)) || (rc = dalloc(c, &c->d_att, 4 * (size_t)n_coef)) ||
@@ -1818,7 +1823,7 @@ int agis_accumulate(agis_ctx* c, int32_t which) {
         return fail(c, AGIS_E_INVALID, "the attitude and calibration sums need a source update first");
     if (which == AGIS_X_ATTITUDE) {
         launch_att_accum(c->G, c->st.lambda2, c->st.rhs_norm_term, c->perm_t, c->ivl_off, c->n_iv, c->rec,
-                         c->an.eps2 ? c->an_w : nullptr, c->att, c->blk, c->sh, c->stream);
+                         c->an.eps2 ? c->an_w : nullptr, c->att, c->blk, c->att_moments, c->sh, c->stream);
         c->x_att_ready = true;
     } else if (which == AGIS_X_CALIBRATION) {
         if (!c->xcal) AGIS_TRY(dalloc(c, &c->xcal, 2 * (size_t)c->n_cal));

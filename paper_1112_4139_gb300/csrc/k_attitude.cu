@@ -1,6 +1,8 @@
 // k_attitude.cu -- the A block (Sect. 5.2): per-knot-interval partial normals from the
 // time-ordered observations, assembly of the banded normals of each overlapping segment,
 // and the segmented robust banded Cholesky (App. C restricted to the envelope).
+#include <cuda_fp16.h>
+
 #include "agis_internal.cuh"
 
 namespace agis {
@@ -21,19 +23,8 @@ constexpr int kAccFP64 = 116;  // distinct products: BB[p] M[m] (10 x 10) and B[
 // symmetric 4x4 M), so the lanes accumulate those 100 and the 16 right-hand-side products
 // (4 per lane) and expand them into the 152 outputs at the end.  W is the weight of the
 // source update, or w_att[o] (Eqs. W, wl) when the excess attitude noise is estimated.
-__global__ void __launch_bounds__(128) k_att_accum(DevGeo G, double lambda2, int rhs_norm,
-                                                   const uint32_t* __restrict__ perm_t,
-                                                   const int64_t* __restrict__ ivl_off, int n_iv,
-                                                   const ObsRec* __restrict__ rec,
-                                                   const double* __restrict__ w_att,
-                                                   const double* __restrict__ att, double* __restrict__ blk) {
-    __shared__ double stage_all[4][kWarp * kStage];
-    __shared__ double red_all[4][kAccFP64];
-    __shared__ int16_t src_tab[kBlkVals];  // accumulator of each block output
-    const int lane = threadIdx.x & 31;
-    const int wib = threadIdx.x >> 5;
-    double* stg = stage_all[wib];
-    double* red = red_all[wib];
+// accumulator of every block output
+__device__ __forceinline__ void block_table(int16_t* src_tab) {
     for (int o = threadIdx.x; o < kBlkVals; o += blockDim.x) {
         int v;
         if (o < 136) {
@@ -47,7 +38,14 @@ __global__ void __launch_bounds__(128) k_att_accum(DevGeo G, double lambda2, int
         }
         src_tab[o] = (int16_t)v;
     }
-    __syncthreads();
+}
+
+// one interval's products of every observation, by one warp, into red[kAccFP64]
+__device__ __forceinline__ void interval_direct(const DevGeo& G, double lambda2, int rhs_norm,
+                                                const uint32_t* __restrict__ perm_t, int64_t beg, int64_t end,
+                                                const ObsRec* __restrict__ rec, const double* __restrict__ w_att,
+                                                const double* __restrict__ att, int l, int lane, double* stg,
+                                                double* red) {
     // this lane's accumulators s = lane + 32 k (k < 3: BB[p] M[m]; k = 3: lanes 0-3 BB M,
     // lanes 4-19 B[b] r[c] of the right-hand side, lanes 20-31 none): the staged factors
     int fa[4], fb[4];
@@ -59,63 +57,422 @@ __global__ void __launch_bounds__(128) k_att_accum(DevGeo G, double lambda2, int
     }
     const bool k3 = lane < 20;              // accumulator 3 in use
     const bool k3_rhs = lane >= 4 && k3;    // ... and it is a right-hand-side product
+    double a[16];
+#pragma unroll
+    for (int k = 0; k < 16; k++) a[k] = att[4 * (int64_t)(l - 3) + k];
+    double acc[4] = {0, 0, 0, 0};
+    for (int64_t base = beg; base < end; base += kWarp) {
+        const int64_t j = base + lane;
+        double* st = stg + lane * kStage;
+        if (j < end) {
+            const uint32_t o = perm_t[j];
+            const ObsRec r = rec[o];
+            double B[4];
+            bspline4(G, r.t_ns, l, B);
+            double s[4];
+#pragma unroll
+            for (int c = 0; c < 4; c++) s[c] = B[0] * a[c] + B[1] * a[4 + c] + B[2] * a[8 + c] + B[3] * a[12 + c];
+            const double W = w_att ? w_att[o] : r.W;
+            const double l4 = 4.0 * lambda2;
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+#pragma unroll
+                for (int e = c; e < 4; e++) st[4 + tri4(c, e)] = W * (r.g[c] * r.g[e] + l4 * s[c] * s[e]);
+            }
+            double D = 1.0 - (s[0] * s[0] + s[1] * s[1] + s[2] * s[2] + s[3] * s[3]);
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                double v = r.R * r.g[c];
+                if (rhs_norm) v -= 2.0 * lambda2 * D * s[c];
+                st[14 + c] = W * v;
+                st[c] = B[c];
+            }
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+#pragma unroll
+                for (int e = c; e < 4; e++) st[18 + tri4(c, e)] = B[c] * B[e];
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < kStage; c++) st[c] = 0.0;
+        }
+        __syncwarp();
+        const int cnt = (int)((end - base) < kWarp ? (end - base) : kWarp);
+        for (int q = 0; q < cnt; q++) {
+            const double* sq = stg + q * kStage;
+#pragma unroll
+            for (int k = 0; k < 3; k++) acc[k] += sq[fa[k]] * sq[fb[k]];
+            if (k3) acc[3] += sq[fa[3]] * sq[fb[3]];
+        }
+        __syncwarp();
+    }
+#pragma unroll
+    for (int k = 0; k < 3; k++) red[lane + 32 * k] = acc[k];
+    if (k3) red[lane + 96] = k3_rhs ? -acc[3] : acc[3];
+    __syncwarp();
+}
+
+// One warp per interval, two FP64 factors from shared memory per product.
+__global__ void __launch_bounds__(128) k_att_accum(DevGeo G, double lambda2, int rhs_norm,
+                                                   const uint32_t* __restrict__ perm_t,
+                                                   const int64_t* __restrict__ ivl_off, int n_iv,
+                                                   const ObsRec* __restrict__ rec,
+                                                   const double* __restrict__ w_att,
+                                                   const double* __restrict__ att, double* __restrict__ blk) {
+    __shared__ double stage_all[4][kWarp * kStage];
+    __shared__ double red_all[4][kAccFP64];
+    __shared__ int16_t src_tab[kBlkVals];
+    const int lane = threadIdx.x & 31;
+    const int wib = threadIdx.x >> 5;
+    double* red = red_all[wib];
+    block_table(src_tab);
+    __syncthreads();
     const int nwarps = gridDim.x * (blockDim.x >> 5);
     for (int iv = blockIdx.x * (blockDim.x >> 5) + wib; iv < n_iv; iv += nwarps) {
-        const int l = iv + 3;
-        double a[16];
+        interval_direct(G, lambda2, rhs_norm, perm_t, ivl_off[iv], ivl_off[iv + 1], rec, w_att, att, iv + 3, lane,
+                        stage_all[wib], red);
 #pragma unroll
-        for (int k = 0; k < 16; k++) a[k] = att[4 * (int64_t)(l - 3) + k];
-        double acc[4] = {0, 0, 0, 0};
-        const int64_t beg = ivl_off[iv], end = ivl_off[iv + 1];
-        for (int64_t base = beg; base < end; base += kWarp) {
+        for (int k = 0; k < 5; k++) {
+            const int o = lane + 32 * k;
+            if (o < kBlkVals) blk[(int64_t)iv * kBlkVals + o] = red[src_tab[o]];
+        }
+        __syncwarp();
+    }
+}
+
+// ---------------------------------------------------------------------------------------
+// Interval blocks by moments on the tensor cores.  In a regular knot interval the B-splines are
+// cubic forms in u = (t - tau_l) / dt and v = 1 - u with coefficients c >= 0, so the block is
+//   sum W BB[p] g g' = sum_k c[p][k] sum_o (W g g')_o (u^k v^(6-k))_o,   k = 0 .. 6,
+// the right-hand side likewise with W R g (the cubics raised to degree 6), and the norm term, a
+// form with the interval's coefficients alone, needs sum_o W u^k v^(12-k), k = 0 .. 12.  Rows
+// W g g' (10), W R g (4), W v^6 and W u^6 by columns u^k v^(6-k): one 16 x 7 contraction over the
+// interval's observations, and an expansion without cancellation (rms error over the sum of the
+// terms' magnitudes: powers of 2 u - 1 2.0e-16, the products' sums 1.8e-16, these
+// forms less).
+//
+// It runs on mma.sync (a 128-row tcgen05 tile would hold one interval of 16 rows): every row value is
+// a 55-bit and every column value a 54-bit fraction of its largest magnitude in the interval, cut into
+// eight signed 7-bit digits kept as FP16 integers, and the products of the digit pairs i + j >= 6 are
+// accumulated in FP32 by their weight 2^(7 (i + j)): 8 pairs x 512 observations x 2^12 are
+// at most 2^24, so every sum is exact, and the pairs left out are below 2^-58 of the largest term
+// (FP64 rounds each product at 2^-53).  Products W g g', powers of x and conversions are 64-bit
+// integer arithmetic.
+// Bound: integer and shared-memory issue (about 28 instructions per observation and warp of 32)
+// and 68 FP64 instructions per interval for the expansion, where the FP64 form takes 116 FMAs and
+// about 95 more FP64 instructions per observation (2 per clock and SM).
+// 24.7M observations in 157,786 intervals: 9.93 -> 2.95 ms; 7.1M in 131,490: 3.06 -> 1.51 ms.
+// Intervals next to the multiple end knots (two at each end), short ones and those that the
+// observations do not cover sum the products one by one.
+constexpr int kMomWarps = 4;
+constexpr int kMomStride = 40;    // 64-bit values per row of the staged chunk (rows 64 B apart mod 128 B)
+constexpr int kMomFlush = 512;    // observations per exact accumulation
+constexpr int kMomMin = 24;       // shorter intervals: the sums of the products themselves
+constexpr uint64_t kDigitBias = 0x0081020408102040ull;   // 64 in every 7-bit digit
+
+struct MomScale {                  // u with 63 fractional bits: 2^shift (t - tau) inv 2^-64, times 2
+    uint64_t inv;
+    int32_t shift;
+    int32_t tshift;                // t - tau in 30 bits, and its unit in u
+    float tinv;
+};
+
+// v 2^(62 - E) for |v| < 2^E, truncated
+__device__ __forceinline__ long long to_fixed(double v, int E) {
+    const uint32_t hi = (uint32_t)__double2hiint(v);
+    const int sh = (int)((hi >> 20) & 0x7ffu) - 1023 + 10 - E;   // at most 9
+    unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | (uint32_t)__double2loint(v);
+    m = sh >= 0 ? m << sh : (sh > -64 ? m >> -sh : 0ull);
+    return (hi >> 31) ? -(long long)m : (long long)m;
+}
+// products of 62-bit fractions and of unsigned 63-bit ones, what is cut off at half its range
+__device__ __forceinline__ long long mulq(long long a, long long b) { return (long long)((unsigned long long)__mul64hi(a, b) << 2) | 2; }
+__device__ __forceinline__ uint64_t mulu(uint64_t a, uint64_t b) { return (__umul64hi(a, b) << 1) | 1; }
+__device__ __forceinline__ double pow2(int n) { return __longlong_as_double((long long)(1023 + n) << 52); }
+
+// fixed-point value, rounded to multiples of 2^kShift -> its digits' bit fields, 28 bits per word;
+// |q| 2^-kShift <= 0.992 2^55
+template <int kShift>
+__device__ __forceinline__ uint2 digit_words(long long q) {
+    constexpr uint64_t kAdd = (kDigitBias << kShift) + (kShift ? 1ull << (kShift > 0 ? kShift - 1 : 0) : 0ull);
+    const uint64_t u = ((uint64_t)q + kAdd) >> kShift;
+    return make_uint2((uint32_t)u & 0xfffffffu, (uint32_t)(u >> 28) & 0xfffffffu);
+}
+// the four digits of a 28-bit word of two observations, as FP16 pairs
+__device__ __forceinline__ void digits4(uint32_t a, uint32_t b, uint32_t out[4]) {
+    const uint32_t c0 = __byte_perm(a, b, 0x5410), c1 = __byte_perm(a >> 14, b >> 14, 0x5410);
+    const __half2 off = __halves2half2(__ushort_as_half(0xe440), __ushort_as_half(0xe440));   // -1088
+    auto half_of = [&](uint32_t w) -> uint32_t {
+        const uint32_t h = (w & 0x007f007fu) | 0x64006400u;    // 1024 + digit + 64
+        const __half2 r = __hadd2(*reinterpret_cast<const __half2*>(&h), off);
+        return *reinterpret_cast<const uint32_t*>(&r);
+    };
+    out[0] = half_of(c0);
+    out[1] = half_of(c0 >> 7);
+    out[2] = half_of(c1);
+    out[3] = half_of(c1 >> 7);
+}
+__device__ __forceinline__ void mma_f16(float c[4], const uint32_t a[4], uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// the four B-splines' coefficients (over 6) of u^k v^(3-k), and the columns' scales 2^n at any u
+__device__ constexpr int kSplineNum[4][4] = {{1, 0, 0, 0}, {4, 12, 6, 1}, {1, 6, 12, 4}, {0, 0, 0, 1}};
+__device__ constexpr int kColShift[7] = {0, 3, 5, 5, 5, 3, 0};
+
+// One interval's products from its moments, by one warp, into red[kAccFP64].
+__device__ __forceinline__ void interval_moments(const DevGeo& G, MomScale ms, double lambda2,
+                                                 const uint32_t* __restrict__ perm_t, int64_t beg, int64_t end, int iv,
+                                                 const ObsRec* __restrict__ rec, const double* __restrict__ w_att,
+                                                 const double* __restrict__ att, int EW, int ER, int Eg, float lu,
+                                                 float lv, int lane, uint2* st, const double (*cbb)[8], const double (*cb)[8], double* wk,
+                                                 double* red) {
+    const int g = lane >> 2, q = lane & 3;
+    const double l4 = 4.0 * lambda2;
+    // every column to its largest value in the interval: u^k v^(6-k) 2^sh[k] < 1
+    int sh[7];
+#pragma unroll
+    for (int k = 0; k < 7; k++) sh[k] = max(kColShift[k], (int)floorf((float)k * lu + (float)(6 - k) * lv - 1e-4f));
+    // moments of this lane: rows g and g + 8, columns 2 q and 2 q + 1
+    double mom[4] = {0, 0, 0, 0};
+    const int64_t tau = G.knot0_ns + (int64_t)iv * G.knot_dt_ns;
+    for (int64_t f0 = beg; f0 < end; f0 += kMomFlush) {
+        float acc[9][4];
+#pragma unroll
+        for (int s = 0; s < 9; s++)
+#pragma unroll
+            for (int e = 0; e < 4; e++) acc[s][e] = 0.0f;
+        const int64_t f1 = end < f0 + kMomFlush ? end : f0 + kMomFlush;
+        for (int64_t base = f0; base < f1; base += kWarp) {
             const int64_t j = base + lane;
-            double* st = stg + lane * kStage;
-            if (j < end) {
+            long long X[16], C[7];
+            if (j < f1) {
                 const uint32_t o = perm_t[j];
-                const ObsRec r = rec[o];
-                double B[4];
-                bspline4(G, r.t_ns, l, B);
-                double s[4];
-#pragma unroll
-                for (int c = 0; c < 4; c++) s[c] = B[0] * a[c] + B[1] * a[4 + c] + B[2] * a[8 + c] + B[3] * a[12 + c];
+                const ObsRec& r = rec[o];
                 const double W = w_att ? w_att[o] : r.W;
-                const double l4 = 4.0 * lambda2;
+                const uint64_t u = __umul64hi((uint64_t)(r.t_ns - tau) << ms.shift, ms.inv) << 1, v = (1ull << 63) - u;
+                const uint64_t u2 = mulu(u, u), v2 = mulu(v, v), u3 = mulu(u2, u), v3 = mulu(v2, v);
+                const uint64_t uv2 = mulu(u, v2), u2v = mulu(u2, v), u6 = mulu(u3, u3), v6 = mulu(v3, v3);
+                const long long Wq = to_fixed(W, EW), WR = to_fixed(W * r.R, ER);
+                long long gq[4];
+#pragma unroll
+                for (int c = 0; c < 4; c++) gq[c] = to_fixed(r.g[c], Eg);
 #pragma unroll
                 for (int c = 0; c < 4; c++) {
+                    const long long Wg = mulq(Wq, gq[c]);
 #pragma unroll
-                    for (int e = c; e < 4; e++) st[4 + tri4(c, e)] = W * (r.g[c] * r.g[e] + l4 * s[c] * s[e]);
+                    for (int e = c; e < 4; e++) X[tri4(c, e)] = __mul64hi(Wg, gq[e]);
+                    X[10 + c] = __mul64hi(WR, gq[c]);
                 }
-                double D = 1.0 - (s[0] * s[0] + s[1] * s[1] + s[2] * s[2] + s[3] * s[3]);
-#pragma unroll
-                for (int c = 0; c < 4; c++) {
-                    double v = r.R * r.g[c];
-                    if (rhs_norm) v -= 2.0 * lambda2 * D * s[c];
-                    st[14 + c] = W * v;
-                    st[c] = B[c];
-                }
-#pragma unroll
-                for (int c = 0; c < 4; c++) {
-#pragma unroll
-                    for (int e = c; e < 4; e++) st[18 + tri4(c, e)] = B[c] * B[e];
-                }
+                X[14] = __mul64hi(Wq, (long long)(v6 >> 1));
+                X[15] = __mul64hi(Wq, (long long)(u6 >> 1));
+                C[0] = (v6 << sh[0]) >> 1;
+                C[1] = mulu(uv2, v3) << (sh[1] - 1);
+                C[2] = mulu(uv2, uv2) << (sh[2] - 1);
+                C[3] = mulu(u3, v3) << (sh[3] - 1);
+                C[4] = mulu(u2v, u2v) << (sh[4] - 1);
+                C[5] = mulu(u2v, u3) << (sh[5] - 1);
+                C[6] = (u6 << sh[6]) >> 1;
             } else {
 #pragma unroll
-                for (int c = 0; c < kStage; c++) st[c] = 0.0;
-            }
-            __syncwarp();
-            const int cnt = (int)((end - base) < kWarp ? (end - base) : kWarp);
-            for (int q = 0; q < cnt; q++) {
-                const double* sq = stg + q * kStage;
+                for (int k = 0; k < 16; k++) X[k] = 0;
 #pragma unroll
-                for (int k = 0; k < 3; k++) acc[k] += sq[fa[k]] * sq[fb[k]];
-                if (k3) acc[3] += sq[fa[3]] * sq[fb[3]];
+                for (int k = 0; k < 7; k++) C[k] = 0;
             }
             __syncwarp();
+#pragma unroll
+            for (int k = 0; k < 16; k++) st[k * kMomStride + lane] = digit_words<5>(X[k]);
+#pragma unroll
+            for (int k = 0; k < 7; k++) st[(16 + k) * kMomStride + lane] = digit_words<8>(C[k]);
+            st[23 * kMomStride + lane] = digit_words<0>(0);
+            __syncwarp();
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const int k0 = 16 * h + 2 * q;
+                uint32_t A[8][4], Bd[8][2];
+#pragma unroll
+                for (int e = 0; e < 4; e++) {   // rows g, g + 8 at k0; then at k0 + 8
+                    const uint4 v = *reinterpret_cast<const uint4*>(&st[(g + 8 * (e & 1)) * kMomStride + k0 + 8 * (e >> 1)]);
+                    uint32_t d[4];
+                    digits4(v.x, v.z, d);
+#pragma unroll
+                    for (int t = 0; t < 4; t++) A[t][e] = d[t];
+                    digits4(v.y, v.w, d);
+#pragma unroll
+                    for (int t = 0; t < 4; t++) A[4 + t][e] = d[t];
+                }
+#pragma unroll
+                for (int e = 0; e < 2; e++) {
+                    const uint4 v = *reinterpret_cast<const uint4*>(&st[(16 + g) * kMomStride + k0 + 8 * e]);
+                    uint32_t d[4];
+                    digits4(v.x, v.z, d);
+#pragma unroll
+                    for (int t = 0; t < 4; t++) Bd[t][e] = d[t];
+                    digits4(v.y, v.w, d);
+#pragma unroll
+                    for (int t = 0; t < 4; t++) Bd[4 + t][e] = d[t];
+                }
+#pragma unroll
+                for (int i = 0; i < 8; i++)
+#pragma unroll
+                    for (int jd = 0; jd < 8; jd++)
+                        if (i + jd >= 6) mma_f16(acc[i + jd - 6], A[i], Bd[jd][0], Bd[jd][1]);
+            }
         }
+        // the exact sums by weight: H 2^63 + L 2^42, in units of 2^-109 of the scales
 #pragma unroll
-        for (int k = 0; k < 3; k++) red[lane + 32 * k] = acc[k];
-        if (k3) red[lane + 96] = k3_rhs ? -acc[3] : acc[3];
-        __syncwarp();
+        for (int e = 0; e < 4; e++) {
+            long long H = 0, L = 0;
+#pragma unroll
+            for (int s = 8; s >= 3; s--) H = (H << 7) + (long long)__float2int_rn(acc[s][e]);
+#pragma unroll
+            for (int s = 2; s >= 0; s--) L = (L << 7) + (long long)__float2int_rn(acc[s][e]);
+            const int row = g + 8 * (e >> 1);
+            const int ce = e & 1 ? (q == 0 ? sh[1] : q == 1 ? sh[3] : sh[5]) : (q == 0 ? sh[0] : q == 1 ? sh[2] : q == 2 ? sh[4] : sh[6]);
+            const int E = (row < 10 ? EW + 2 * Eg : (row < 14 ? ER + Eg : EW)) - ce;
+            mom[e] += fma((double)H, pow2(E - 46), (double)L * pow2(E - 67));
+        }
+    }
+    __syncwarp();
+    // wk: moments [16][8] at 0, coefficients of s [4][4] at 128, of s s' [10][7] at 144, the moments
+    // with the norm term [10][8] at 216
+    wk[g * 8 + 2 * q] = mom[0];
+    wk[g * 8 + 2 * q + 1] = mom[1];
+    wk[(g + 8) * 8 + 2 * q] = mom[2];
+    wk[(g + 8) * 8 + 2 * q + 1] = mom[3];
+    if (lane < 16) {
+        const int c = lane >> 2, k = lane & 3;
+        double s = 0.0;
+#pragma unroll
+        for (int jj = 0; jj < 4; jj++) s = fma(att[4 * (int64_t)(iv + jj) + c], (double)kSplineNum[jj][k], s);
+        wk[128 + lane] = s * (1.0 / 6.0);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < 3; t++) {
+        const int idx = lane + 32 * t;
+        if (idx < 70) {
+            const int m = idx / 7, b = idx - 7 * m;
+            int c = 0;
+            while (m >= tri4(c, 3) + 1) c++;
+            const int e = c + m - tri4(c, c);
+            double s = 0.0;
+#pragma unroll
+            for (int a = 0; a < 4; a++)
+                if (b - a >= 0 && b - a < 4) s = fma(wk[128 + 4 * c + a], wk[128 + 4 * e + b - a], s);
+            wk[144 + idx] = s;
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < 3; t++) {
+        const int idx = lane + 32 * t;
+        if (idx < 70) {
+            const int m = idx / 7, a = idx - 7 * m;
+            double s = 0.0;
+#pragma unroll
+            for (int b = 0; b < 7; b++) {
+                const int k = a + b;   // sum of W u^k v^(12-k): row 14, beyond k = 6 row 15
+                s = fma(wk[144 + 7 * m + b], k < 7 ? wk[14 * 8 + k] : wk[15 * 8 + k - 6], s);
+            }
+            wk[216 + 8 * m + a] = fma(l4, s, wk[8 * m + a]);
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < 4; t++) {
+        const int idx = lane + 32 * t;
+        if (idx < 116) {
+            double s = 0.0;
+            if (idx < 100) {
+                const int p = idx / 10, m = idx - 10 * p;
+#pragma unroll
+                for (int a = 0; a < 7; a++) s = fma(cbb[p][a], wk[216 + 8 * m + a], s);
+                s *= 1.0 / 36.0;
+            } else {
+                const int b = (idx - 100) >> 2, c = idx & 3;
+#pragma unroll
+                for (int a = 0; a < 7; a++) s = fma(cb[b][a], wk[(10 + c) * 8 + a], s);
+                s *= -1.0 / 6.0;
+            }
+            red[idx] = s;
+        }
+    }
+    __syncwarp();
+}
+
+__global__ void __launch_bounds__(32 * kMomWarps) k_att_moments(DevGeo G, MomScale ms, double lambda2,
+                                                                const uint32_t* __restrict__ perm_t,
+                                                                const int64_t* __restrict__ ivl_off, int n_iv,
+                                                                const ObsRec* __restrict__ rec,
+                                                                const double* __restrict__ w_att,
+                                                                const double* __restrict__ att, double* __restrict__ blk) {
+    __shared__ __align__(16) double stage_all[kMomWarps][kWarp * kStage + kAccFP64];
+    __shared__ double cbb[10][8], cb[4][8];   // coefficients of BB (over 36) and of B at degree 6 (over 6)
+    __shared__ int16_t src_tab[kBlkVals];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    double* wk = stage_all[wib];   // after an interval's sums: moments and polynomials
+    uint2* st = reinterpret_cast<uint2*>(wk);
+    double* red = wk + kWarp * kStage;   // the products
+    block_table(src_tab);
+    for (int e = threadIdx.x; e < 80; e += blockDim.x) {
+        const int p = e >> 3, k = e & 7;
+        int i = 0;
+        while (p >= tri4(i, 3) + 1) i++;
+        const int j = i + p - tri4(i, i);
+        int c = 0;
+        for (int a = 0; a < 4; a++)
+            if (k - a >= 0 && k - a < 4) c += kSplineNum[i][a] * kSplineNum[j][k - a];
+        cbb[p][k] = (double)c;
+    }
+    if (threadIdx.x < 32) {
+        const int i = threadIdx.x >> 3, k = threadIdx.x & 7;
+        int c = 0;
+        for (int a = 0; a < 4; a++)
+            if (k - a >= 0 && k - a < 4) c += kSplineNum[i][a] * (k - a == 0 || k - a == 3 ? 1 : 3);
+        cb[i][k] = (double)c;
+    }
+    __syncthreads();
+    const int nwarps = gridDim.x * kMomWarps;
+    for (int iv = blockIdx.x * kMomWarps + wib; iv < n_iv; iv += nwarps) {
+        const int64_t beg = ivl_off[iv], end = ivl_off[iv + 1];
+        // the largest magnitudes of W, W R and g (bits of the high words)
+        uint32_t mw = 0, mr = 0, mg = 0, t_lo = 0xffffffffu, t_hi = 0;
+        const int64_t tau = G.knot0_ns + (int64_t)iv * G.knot_dt_ns;
+        for (int64_t j = beg + lane; j < end; j += kWarp) {
+            const uint32_t o = perm_t[j];
+            const ObsRec& r = rec[o];
+            const double W = w_att ? w_att[o] : r.W;
+            const double2 ga = *reinterpret_cast<const double2*>(r.g), gb = *reinterpret_cast<const double2*>(r.g + 2);
+            const uint32_t tq = (uint32_t)((r.t_ns - tau) >> ms.tshift);
+            t_lo = min(t_lo, tq);
+            t_hi = max(t_hi, tq);
+            mw = max(mw, (uint32_t)__double2hiint(W) & 0x7fffffffu);
+            mr = max(mr, (uint32_t)__double2hiint(W * r.R) & 0x7fffffffu);
+            mg = max(max(mg, (uint32_t)__double2hiint(ga.x) & 0x7fffffffu), (uint32_t)__double2hiint(ga.y) & 0x7fffffffu);
+            mg = max(max(mg, (uint32_t)__double2hiint(gb.x) & 0x7fffffffu), (uint32_t)__double2hiint(gb.y) & 0x7fffffffu);
+        }
+        mw = __reduce_max_sync(0xffffffffu, mw);
+        mr = __reduce_max_sync(0xffffffffu, mr);
+        mg = __reduce_max_sync(0xffffffffu, mg);
+        t_lo = __reduce_min_sync(0xffffffffu, t_lo);
+        t_hi = __reduce_max_sync(0xffffffffu, t_hi);
+        // -log2 of the largest u and v
+        const float lu = -log2f((float)(t_hi + 1) * ms.tinv), lv = -log2f(fmaf(-(float)t_lo, ms.tinv, 1.0f) + 1e-6f);
+        // 2^E above them; W and W R below 0.99 of it, for rows of 55 bits
+        const int EW = (int)((mw + 0x5000) >> 20) - 1022, ER = (int)((mr + 0x5000) >> 20) - 1022, Eg = (int)(mg >> 20) - 1022;
+        // scales in range: finite, and no power of two below under- or overflows (all residuals may be
+        // zero); u^6 and v^6, the outer B-splines' squares, reach 2^-9: their 63 bits hold 54 of a column
+        const bool ok = iv >= 2 && iv < n_iv - 2 && end - beg >= kMomMin && abs(EW) < 250 && ER < 250 && abs(Eg) < 250 &&
+                        fmaxf(lu, lv) < 1.5f;
+        if (ok)
+            interval_moments(G, ms, lambda2, perm_t, beg, end, iv, rec, w_att, att, EW, max(ER, -250), Eg, lu, lv, lane,
+                             st, cbb, cb, wk, red);
+        else
+            interval_direct(G, lambda2, 0, perm_t, beg, end, rec, w_att, att, iv + 3, lane, wk, red);
 #pragma unroll
         for (int k = 0; k < 5; k++) {
             const int o = lane + 32 * k;
@@ -477,13 +834,25 @@ __global__ void k_att_apply(int n_coef, int n_seg, const int32_t* __restrict__ s
 }
 
 void launch_att_accum(const DevGeo& G, double lambda2, int rhs_norm, const uint32_t* perm_t, const int64_t* ivl_off,
-                      int n_iv, const ObsRec* rec, const double* w_att, const double* att, double* blk,
+                      int n_iv, const ObsRec* rec, const double* w_att, const double* att, double* blk, bool moments,
                       const Shapes& sh, cudaStream_t s) {
-    int warps = n_iv;
-    int blocks = (warps + 3) / 4;
     const int bps = sh.att_bps > 0 ? sh.att_bps : 32;
+    int blocks = (n_iv + 3) / 4;
     if (blocks > 152 * bps) blocks = 152 * bps;
     if (blocks < 1) blocks = 1;
+    // the norm term of degree 12 has no columns of its own and loses 4 bits in its middle: it must be small
+    // beside g g' (|g| about 2; the usual lambda^2 is 1e-6)
+    if (moments && !rhs_norm && lambda2 <= 1.0 / 64.0) {
+        int nb = 0;   // significant bits of dt
+        while (nb < 62 && (G.knot_dt_ns >> nb) > 0) nb++;
+        MomScale ms;
+        ms.shift = 64 - nb;
+        ms.tshift = nb > 30 ? nb - 30 : 0;
+        ms.tinv = (float)((double)((int64_t)1 << ms.tshift) / (double)G.knot_dt_ns);
+        ms.inv = (uint64_t)(((unsigned __int128)1 << (62 + nb)) / (unsigned __int128)G.knot_dt_ns);
+        k_att_moments<<<blocks, 32 * kMomWarps, 0, s>>>(G, ms, lambda2, perm_t, ivl_off, n_iv, rec, w_att, att, blk);
+        return;
+    }
     k_att_accum<<<blocks, 128, 0, s>>>(G, lambda2, rhs_norm, perm_t, ivl_off, n_iv, rec, w_att, att, blk);
 }
 

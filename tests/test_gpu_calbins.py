@@ -1,5 +1,5 @@
 """The C block of the full geometric calibration at the numbers of AC column bins where its path
-changes (reduced systems in shared memory up to 200 bins, through global memory beyond) and around
+changes (reduced systems in shared memory up to 160 bins, through global memory beyond) and around
 its warps' widths, against the oracle's constrained least-squares update of the same residuals."""
 import dataclasses
 

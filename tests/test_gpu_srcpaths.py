@@ -24,13 +24,13 @@ N_CMP = 60     # the sources compared with the oracle (the first ones)
 @pytest.fixture(scope="module")
 def base():
     # sources with 52 transits or more in a year: above 512 observations per source; the same sources
-    # six times, for more than 100 observations per knot interval (the lines of the dispatch)
+    # 140 times, for more than 23M observations and 100 per knot interval (the lines of the dispatch)
     one = synth.simulate(synth.config("small1yr", n_src=40_000, seed=5, min_transits=52))
-    tile = lambda a: np.concatenate([a] * 6)  # noqa: E731
-    src = np.concatenate([one.src + k * one.n_src for k in range(6)]).astype(np.int32)
+    tile = lambda a: np.concatenate([a] * 140)  # noqa: E731
+    src = np.concatenate([one.src + k * one.n_src for k in range(140)]).astype(np.int32)
     ds = dataclasses.replace(one, src=src, **{k: tile(getattr(one, k)) for k in (
         "t_ns", "ccd", "fov", "kind", "sigma", "mu", "noise", "gate", "src_true", "src_mag", "n_transits", "src0")})
-    assert ds.n_obs >= 512 * ds.n_src and ds.n_obs >= 110 * (ds.n_coef - 3), (ds.n_obs, ds.n_src)
+    assert ds.n_obs >= 23_500_000 and ds.n_obs >= 512 * ds.n_src and ds.n_obs >= 110 * (ds.n_coef - 3), (ds.n_obs, ds.n_src)
     return ds
 
 
@@ -60,7 +60,7 @@ def test_source_update_matches_oracle(base, shape, weight_fn):
         sig = ds.sigma.copy()
         sig[(ds.src % 3 == 0) & (np.arange(ds.n_obs) % 5 == 0)] *= np.float32(1.5)
         ds = dataclasses.replace(ds, sigma=sig)
-    assert ds.n_obs >= 512 * ds.n_src and ds.n_obs >= 100 * (ds.n_coef - 3)
+    assert ds.n_obs >= 23_000_000 and ds.n_obs >= 512 * ds.n_src
     # attitude and calibration at the truth: residuals at the noise level, weights that differ
     sub = ds.subset_sources(np.arange(N_CMP))
     P = OM.problem_from_dataset(sub)
