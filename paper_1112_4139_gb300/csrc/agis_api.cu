@@ -1051,9 +1051,9 @@ int agis_init(const agis_geometry* geo, const agis_config* cfg, const agis_obs* 
     }
     c->mixed = cfg->precision == 1;
     // FP64 S block: weight rounds by corrections to unit-weight sums (long sources: 30,000 of 820
-    // observations 1.4 + 4 x 0.49 ms a source update, against 1.85 + 4 x 1.88 ms for the direct sums
+    // observations 1.4 + 4 x 0.49 ms a source update, against 0.5 + 5 x 1.7 ms for the direct sums
     // of every row) or by direct sums (short sources gain less: 3000 of 165 80 + 4 x 36 us against
-    // 93 + 4 x 81).  FP64 A block: interval blocks by moments (24.7M observations in 157,786 intervals
+    // 29 + 5 x 61).  FP64 A block: interval blocks by moments (24.7M observations in 157,786 intervals
     // 9.93 -> 2.95 ms, 7.1M in 131,490 3.06 -> 1.51) or by the sums of the products.
     // Both first forms round otherwise (no worse against 64 bits), which turns the last bit of 10 to 20%
     // of the attitude coefficients, and the next iteration's calibration averages those bits: measured

@@ -6,6 +6,7 @@
 //   k_src_first   sigma per class, robust scale and round 0's class sums
 //   k_src_solve5  the 5x5 algebra of the excess-noise steps
 //   k_src_round   the next round's class sums, and the weights of the last round
+//   k_src_sums    class sums of every row, a block per source, in place of the above where the set is small
 //   k_src_final   the hand-over records (t, R = h - A d, W, g, meta) that the time-ordered
 //                 attitude pass and the calibration pass gather
 //   k_src_general sources whose sigma differs within a class: all rounds in one warp
@@ -17,8 +18,8 @@
 // on its error), and only the rows that may exceed 2 are gathered, 32 to a warp, for the FP64
 // weight and the 27 products that (1 - w) takes off again: a round then costs about a fifth of
 // the FP64 work of the direct sums.
-// Measured, source solves of the S block: 24.7M observations of 30,000 sources 14.2 -> 4.5 ms (9.9
-// with direct sums), 0.5M of 3000 sources 1.68 -> 0.7 ms (direct sums).  Before, one persistent
+// Measured, source solves of the S block: 24.7M observations of 30,000 sources 14.2 -> 4.5 ms; with
+// direct sums 6.7M of 8000 sources 4.75 -> 2.9, 0.5M of 3000 sources 1.68 -> 0.57.  Before, one persistent
 // kernel ran all rounds of a batch of sources in a warp, with the 5x5 solves in one lane each.
 #include <type_traits>
 
@@ -256,12 +257,7 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_first(Settings st, cons
                                                                const uint64_t* __restrict__ skey,
                                                                SrcWork* __restrict__ work) {
     extern __shared__ __align__(16) unsigned char first_smem[];
-    union FirstWork {
-        SelWork sel;
-        double red[kDirect ? kRedVals * kRedStride : 1];
-    };
-    FirstWork& fw = reinterpret_cast<FirstWork*>(first_smem)[threadIdx.x >> 5];
-    SelWork& sw = fw.sel;
+    SelWork& sw = reinterpret_cast<SelWork*>(first_smem)[threadIdx.x >> 5];
     __shared__ uint32_t list_all[kPassWarps][32];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     uint32_t* list = list_all[wib];
@@ -278,7 +274,9 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_first(Settings st, cons
             }
             double* scr = scratch + (size_t)o0 * kScr;
             // unit-weight sums and sigma of each class; sums only while its sigma is one value
-            double s2c[2] = {1.0, 1.0}, s2min = 1e300;
+            // (bit patterns: variances are not negative, and comparisons hold the FP64 unit)
+            double s2c[2] = {1.0, 1.0};
+            uint64_t s2m = __double_as_longlong(1e300);
             bool uni = true;
             for (int c = 0; c < 2; c++) {
                 const int lo = c ? nal : 0, hi = c ? n : nal;
@@ -287,14 +285,15 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_first(Settings st, cons
                 for (int k = 0; k < kSumVals; k++) v[k] = 0.0;
                 if (lo < hi) {
                     const double s2 = scr[(size_t)lo * kScr + 7];
-                    bool same = true;
+                    const uint64_t s2b = __double_as_longlong(s2);
+                    bool same = s2 == s2;
                     for (int j0 = lo; j0 < hi; j0 += kWarp) {
                         const int j = j0 + lane;
                         if (j < hi) {
                             const double* e = scr + (size_t)j * kScr;
-                            const double sj = e[7];
-                            s2min = fmin(s2min, sj);
-                            same = same && sj == s2;
+                            const uint64_t sj = __double_as_longlong(e[7]);
+                            s2m = sj < s2m ? sj : s2m;
+                            same = same && sj == s2b;
                             if (!kDirect && uni) {
                                 double h, A[5];
                                 row_load(e, h, A);
@@ -313,7 +312,7 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_first(Settings st, cons
                 }
                 if (!kDirect && uni) reduce_vals(v, lane, w.T[c]);
             }
-            s2min = warp_min(s2min);
+            const double s2min = warp_min(__longlong_as_double(s2m));
             double vs = 0.0;
             const bool in_smem = n <= kKeyCap64;
             const uint64_t* keys = in_smem ? sw.keys : skey + o0;
@@ -358,13 +357,9 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_first(Settings st, cons
             const bool last = st.robust ? st.n_rounds == 0 : true;
             int nout = 0;
             if (kDirect) {
-                double rx[2];
-                for (int c = 0; c < 2; c++) rx[c] = vs > 0.0 ? 1.0 / (sqrt(s2c[c]) * vs) : 0.0;
-                direct_sums(scr, n, nal, lane, st.robust ? 0 : 2, rx, nullptr, nullptr, st.weight_fn, last, fw.red,
-                            &w.T[0][0], nout);
-                if (lane == 0) w.nout = nout;
+                // round 0's weights are wfun(h rx); all 1 for a robust scale of 0
+                if (lane < 2) w.isd[lane] = vs > 0.0 ? 1.0 / (sqrt(lane ? s2c[1] : s2c[0]) * vs) : 0.0;
                 for (int k = lane; k < kRedVals; k += kWarp) (&w.C[0][0])[k] = 0.0;
-                __syncwarp();
                 continue;
             }
             for (int c = 0; c < 2; c++) {
@@ -476,31 +471,166 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_round(Settings st, int 
         }
 }
 
-__global__ void __launch_bounds__(32 * kPassWarps) k_src_round_direct(Settings st, int last,
-                                                                      const int64_t* __restrict__ src_off,
-                                                                      const int32_t* __restrict__ src_nal,
-                                                                      const int32_t* __restrict__ src_order,
-                                                                      int32_t n_src, int batch,
-                                                                      double* __restrict__ scratch,
-                                                                      SrcWork* __restrict__ work) {
-    __shared__ double red_all[kPassWarps][kRedVals * kRedStride];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int step = gridDim.x * kPassWarps * batch;
-    for (int base = (blockIdx.x * kPassWarps + wib) * batch; base < n_src; base += step)
-        for (int q = base; q < min(base + batch, n_src); q++) {
-            const int i = src_order[q];
-            SrcWork& w = work[i];
-            if (w.flags != 1) continue;
-            const int64_t o0 = src_off[i];
-            double d[5];
+// Direct class sums of one round, a block per source.  Every row is weighted: w = wfun(h rx) in
+// round 0 (kSumFirst, rx in SrcWork::isd), wfun((h - A d) isd) later (kSumLater), 1 for plain
+// weights (kSumOne).  Lane partials over the rows lane, lane + 32, ... of each class, then the 32
+// partials of a value are added in lane order.  last: w goes to the scratch row.
+//
+// Bound by FP64 instructions (64 cycles each on a sub-partition, whatever the active lanes), so
+// the four warps split them without doing any twice: the arguments z by chunks of 32 rows, the
+// products by the row of A that they share.  Only rows with |z| >= 2 are listed for the weight
+// function, for full warps of its polynomial, exponential and division.  With a warp per
+// source and the weight function in every row: 800 sources of 165 45 us a round (the largest one's
+// chain), 3000 81, 8000 of 840 512; so 28, 61, 470
+// (10,000 of 165: 181).
+enum SumMode { kSumFirst, kSumLater, kSumOne };
+constexpr int kSumChunks = 16;     // chunks of 32 rows between two flushes of the list
+struct SumShared {
+    double red[kRedVals * kRedStride];
+    double w[kSumChunks * kWarp];      // weights of the group's rows
+    double z[kSumChunks * kWarp];      // listed arguments and their rows
+    uint16_t slot[kSumChunks * kWarp];
+    int m[2], nout;
+};
+
+// the products of one row of A (kRole = 0, 1, 2 with sum w h^2, or 3 with row 4) over a group's chunks
+template <int kRole>
+__device__ __forceinline__ void sum_role(double* scr, SumShared& sh, int q0, int q1, int n_al, int nal, int n, int lane,
+                                         bool last, double (&v)[7]) {
+    for (int q = q0; q < q1; q++) {
+        const bool ac = q >= n_al;
+        if (q == n_al) {
+            // the AL class is complete
+            int k = 0;
 #pragma unroll
-            for (int k = 0; k < 5; k++) d[k] = w.d[k];
-            const double isd[2] = {w.isd[0], w.isd[1]};
-            int nout;
-            direct_sums(scratch + (size_t)o0 * kScr, (int)(src_off[i + 1] - o0), src_nal[i], lane, 1, nullptr, isd, d,
-                        st.weight_fn, last, red_all[wib], &w.T[0][0], nout);
-            if (lane == 0) w.nout = nout;
+            for (int b = kRole; b < 5; b++) sh.red[up5(kRole, b) * kRedStride + lane] = v[k++];
+            sh.red[(15 + kRole) * kRedStride + lane] = v[k++];
+            if (kRole == 2) sh.red[20 * kRedStride + lane] = v[k++];
+            if (kRole == 3) {
+                sh.red[up5(4, 4) * kRedStride + lane] = v[k++];
+                sh.red[19 * kRedStride + lane] = v[k++];
+            }
+#pragma unroll
+            for (int e = 0; e < 7; e++) v[e] = 0.0;
         }
+        const int j = (ac ? nal + (q - n_al) * kWarp : q * kWarp) + lane;
+        if (j < (ac ? n : nal)) {
+            double* e = scr + (size_t)j * kScr;
+            const double w = sh.w[(q - q0) * kWarp + lane], h = e[0];
+            if (kRole == 0 && last) e[6] = w;
+            const double wa = w * e[1 + kRole];
+            int k = 0;
+#pragma unroll
+            for (int b = kRole; b < 5; b++, k++) v[k] += wa * e[1 + b];
+            v[k++] += wa * h;
+            if (kRole == 2) v[k++] += w * h * h;
+            if (kRole == 3) {
+                const double w4 = w * e[5];
+                v[k++] += w4 * e[5];
+                v[k++] += w4 * h;
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(128) k_src_sums(Settings st, int mode, int last, const int64_t* __restrict__ src_off,
+                                                  const int32_t* __restrict__ src_nal,
+                                                  const int32_t* __restrict__ src_order, int32_t n_src,
+                                                  double* __restrict__ scratch, SrcWork* __restrict__ work) {
+    __shared__ SumShared sh;
+    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
+    if (tid < 2) sh.m[tid] = 0;
+    if (tid == 2) sh.nout = 0;
+    __syncthreads();
+    int par = 0;
+    for (int q_ = blockIdx.x; q_ < n_src; q_ += gridDim.x) {
+        const int i = src_order[q_];
+        SrcWork& w = work[i];
+        if (w.flags != 1) continue;
+        const int64_t o0 = src_off[i];
+        const int n = (int)(src_off[i + 1] - o0), nal = src_nal[i];
+        double* scr = scratch + (size_t)o0 * kScr;
+        const int n_al = (nal + kWarp - 1) / kWarp, n_chunk = n_al + (n - nal + kWarp - 1) / kWarp;
+        const double isd0 = w.isd[0], isd1 = w.isd[1];
+        double d[5], v[7];
+#pragma unroll
+        for (int k = 0; k < 5; k++) d[k] = w.d[k];
+#pragma unroll
+        for (int k = 0; k < 7; k++) v[k] = 0.0;
+        int cnt = 0;
+        for (int q0 = 0; q0 < n_chunk; q0 += kSumChunks, par ^= 1) {
+            const int q1 = min(q0 + kSumChunks, n_chunk);
+            for (int e = tid; e < (q1 - q0) * kWarp; e += 128) sh.w[e] = 1.0;
+            if (mode != kSumOne)
+                for (int q = q0 + wib; q < q1; q += 4) {
+                    const bool ac = q >= n_al;
+                    const int j = (ac ? nal + (q - n_al) * kWarp : q * kWarp) + lane;
+                    double z = 0.0;
+                    if (j < (ac ? n : nal)) {
+                        double h, A[5];
+                        row_load(scr + (size_t)j * kScr, h, A);
+                        const double f = ac ? isd1 : isd0;
+                        if (mode == kSumFirst) z = h * f;
+                        else z = (h - row_dot(A, d)) * f;
+                    }
+                    const bool cand = (__double2hiint(z) & 0x7fffffff) >= 0x40000000;   // |z| >= 2, or not a number
+                    const unsigned ball = __ballot_sync(0xffffffffu, cand);
+                    if (ball) {
+                        int pos = 0;
+                        if (lane == 0) pos = atomicAdd(&sh.m[par], __popc(ball));
+                        pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(ball & ((1u << lane) - 1u));
+                        if (cand) {
+                            sh.z[pos] = z;
+                            sh.slot[pos] = (uint16_t)((q - q0) * kWarp + lane);
+                        }
+                    }
+                }
+            __syncthreads();
+            const int m = sh.m[par];
+            for (int e = tid; e < m; e += 128) {
+                const double wt = wfun(sh.z[e], st.weight_fn);
+                sh.w[sh.slot[e]] = wt;
+                cnt += wt < 0.2;
+            }
+            if (tid == 0) sh.m[par ^ 1] = 0;
+            __syncthreads();
+            if (wib == 0) sum_role<0>(scr, sh, q0, q1, n_al, nal, n, lane, last, v);
+            else if (wib == 1) sum_role<1>(scr, sh, q0, q1, n_al, nal, n, lane, last, v);
+            else if (wib == 2) sum_role<2>(scr, sh, q0, q1, n_al, nal, n, lane, last, v);
+            else sum_role<3>(scr, sh, q0, q1, n_al, nal, n, lane, last, v);
+            __syncthreads();
+        }
+        // the last class (AL, with AC zero, if no AC rows follow)
+        const int base = n_chunk > n_al ? kSumVals : 0;
+        auto put = [&](int val, double x) {
+            sh.red[(base + val) * kRedStride + lane] = x;
+            if (base == 0) sh.red[(kSumVals + val) * kRedStride + lane] = 0.0;
+            else if (n_al == 0) sh.red[val * kRedStride + lane] = 0.0;
+        };
+        int k = 0;
+        for (int b = wib; b < 5; b++) put(up5(wib, b), v[k++]);
+        put(15 + wib, v[k++]);
+        if (wib == 2) put(20, v[k++]);
+        if (wib == 3) {
+            put(up5(4, 4), v[k++]);
+            put(19, v[k++]);
+        }
+        cnt = warp_sum_int(cnt);
+        if (lane == 0 && cnt) atomicAdd(&sh.nout, cnt);
+        __syncthreads();
+        // the partials of lanes without rows are zeros: one addition stands for them
+        if (tid < 64 && lane < kSumVals) {
+            const int cls = tid >> 5, val = cls * kSumVals + lane, rows = cls ? n - nal : nal, cols = min(rows, kWarp);
+            const double* col = sh.red + val * kRedStride;
+            double t = col[0];
+            for (int e = 1; e < cols; e++) t += col[e];
+            (&w.T[0][0])[val] = t + 0.0;
+        } else if (tid == 64) {
+            w.nout = sh.nout;
+        }
+        __syncthreads();
+        if (tid == 64) sh.nout = 0;
+    }
 }
 
 // the 5x5 algebra of one round, one thread (kPair: two neighbouring lanes) per source: y = 0 first,
@@ -889,19 +1019,21 @@ void launch_source_solve(const Settings& st, bool corrections, const int64_t* sr
     // lane 48), one lane beyond (30,000 sources: 100 us)
     const bool pair = n_src <= 152 * 4 * 16;
     constexpr size_t first_smem = kPassWarps * sizeof(SelWork);
-    static_assert(sizeof(SelWork) <= kRedVals * kRedStride * sizeof(double), "shared memory of the direct first pass");
     for (int r = 0; r < rounds; r++) {
         const int last = r == rounds - 1;
         if (r == 0 && corrections)
             k_src_first<false><<<nb, th, first_smem, stream>>>(st, src_off, src_nal, src_order, n_src, batch, scratch, skey,
                                                                work);
-        else if (r == 0)
-            k_src_first<true><<<nb, th, kPassWarps * kRedVals * kRedStride * sizeof(double), stream>>>(
-                st, src_off, src_nal, src_order, n_src, batch, scratch, skey, work);
         else if (corrections)
             k_src_round<<<nb, th, 0, stream>>>(st, last, src_off, src_nal, src_order, n_src, batch, scratch, work);
-        else
-            k_src_round_direct<<<nb, th, 0, stream>>>(st, last, src_off, src_nal, src_order, n_src, batch, scratch, work);
+        else {
+            if (r == 0)
+                k_src_first<true><<<nb, th, first_smem, stream>>>(st, src_off, src_nal, src_order, n_src, batch, scratch,
+                                                                  skey, work);
+            const int mode = !st.robust ? kSumOne : (r == 0 ? kSumFirst : kSumLater);
+            k_src_sums<<<n_src < 152 * 64 ? n_src : 152 * 64, 128, 0, stream>>>(st, mode, last, src_off, src_nal,
+                                                                                src_order, n_src, scratch, work);
+        }
         if (pair) k_src_solve5<true><<<(2 * n_src + 31) / 32, 32, 0, stream>>>(st, last, src_off, n_src, out, work);
         else k_src_solve5<false><<<(n_src + 127) / 128, 128, 0, stream>>>(st, last, src_off, n_src, out, work);
     }
