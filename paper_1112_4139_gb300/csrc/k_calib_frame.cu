@@ -80,25 +80,45 @@ __global__ void k_cal_solve_sums(int n_cal, const double* __restrict__ sums, dou
 
 // Constraint projection d = d~ - C (C'C)^-1 C' d~ (Eq. calCon).  The columns of C for
 // Eqs. cc1 (per interval: all 124 AL offsets) and cc3 (per interval and field: 7 AC offsets)
-// have disjoint supports, so within each column's support d = d~ - mean(d~).  One thread
-// per constraint column; then c += d.
-__global__ void k_cal_project(int n_days, const double* __restrict__ dtil, double* __restrict__ cal) {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= 3 * n_days) return;
-    int64_t k0;
-    int cnt;
-    if (g < n_days) {
-        k0 = (int64_t)g * 124;
-        cnt = 124;
-    } else {
-        const int h = g - n_days;  // (day, field)
-        k0 = (int64_t)n_days * 124 + (int64_t)h * 7;
-        cnt = 7;
+// have disjoint supports, so within each column's support d = d~ - mean(d~).  Then c += d.
+// AL columns by blocks of kProjDays: their values are staged (a thread on its own loads 124 one after
+// another: 41 us of 365 intervals, so 11) and summed by a lane in order; then the AC columns.
+constexpr int kProjDays = 8;
+__global__ void __launch_bounds__(128) k_cal_project(int n_days, const double* __restrict__ dtil, double* __restrict__ cal) {
+    const int al_blocks = (n_days + kProjDays - 1) / kProjDays, tid = threadIdx.x;
+    if ((int)blockIdx.x >= al_blocks) {
+        const int h = (blockIdx.x - al_blocks) * blockDim.x + tid;   // (interval, field)
+        if (h >= 2 * n_days) return;
+        const int64_t k0 = (int64_t)n_days * 124 + (int64_t)h * 7;
+        double v[7], s = 0.0;
+#pragma unroll
+        for (int i = 0; i < 7; i++) v[i] = dtil[k0 + i];
+#pragma unroll
+        for (int i = 0; i < 7; i++) s += v[i];
+        const double m = s / 7.0;
+#pragma unroll
+        for (int i = 0; i < 7; i++) cal[k0 + i] += v[i] - m;
+        return;
     }
-    double s = 0.0;
-    for (int i = 0; i < cnt; i++) s += dtil[k0 + i];
-    const double m = s / (double)cnt;
-    for (int i = 0; i < cnt; i++) cal[k0 + i] += dtil[k0 + i] - m;
+    __shared__ double sh[kProjDays * 124], mean[kProjDays];
+    const int g0 = blockIdx.x * kProjDays, nv = min(kProjDays, n_days - g0) * 124;
+    const int64_t k0 = (int64_t)g0 * 124;
+#pragma unroll
+    for (int e = 0; e < (kProjDays * 124 + 127) / 128; e++)
+        if (tid + 128 * e < nv) sh[tid + 128 * e] = dtil[k0 + tid + 128 * e];
+    __syncthreads();
+    if (tid * 124 < nv) {
+        double s = 0.0;
+#pragma unroll 4
+        for (int i = 0; i < 124; i++) s += sh[tid * 124 + i];
+        mean[tid] = s / 124.0;
+    }
+    __syncthreads();
+    for (int e = tid; e < nv; e += 128) cal[k0 + e] += sh[e] - mean[e / 124];
+}
+static void launch_cal_project(int n_days, const double* dtil, double* cal, cudaStream_t s) {
+    const int blocks = (n_days + kProjDays - 1) / kProjDays + (2 * n_days + 127) / 128;
+    if (blocks > 0) k_cal_project<<<blocks, 128, 0, s>>>(n_days, dtil, cal);
 }
 
 void launch_cal(int n_cal, int n_days, const uint32_t* perm_c, const int64_t* cal_off, const ObsRec* rec, double tol,
@@ -108,7 +128,7 @@ void launch_cal(int n_cal, int n_days, const uint32_t* perm_c, const int64_t* ca
     if (blocks > 152 * sh.cal_bps) blocks = 152 * sh.cal_bps;
     if (blocks < 1) blocks = 1;
     k_cal_accum<<<blocks, sh.cal_threads, 0, s>>>(n_cal, perm_c, cal_off, rec, tol, dtil, rd, nullptr);
-    k_cal_project<<<(3 * n_days + 127) / 128, 128, 0, s>>>(n_days, dtil, cal);
+    launch_cal_project(n_days, dtil, cal, s);
 }
 
 // partitioned sources: the local (N_kk, b_k) sums, and the update from reduced sums
@@ -126,7 +146,32 @@ void launch_cal_from_sums(int n_cal, int n_days, const double* sums, double tol,
     if (blocks > 152 * 16) blocks = 152 * 16;
     if (blocks < 1) blocks = 1;
     k_cal_solve_sums<<<blocks, 256, 0, s>>>(n_cal, sums, tol, dtil, rd);
-    k_cal_project<<<(3 * n_days + 127) / 128, 128, 0, s>>>(n_days, dtil, cal);
+    launch_cal_project(n_days, dtil, cal, s);
+}
+
+// Sums of kN values over a block of 256 threads in the order of a binary tree (thread t adds that of
+// t + 128, then t + 64, ...), every value by one warp: lane partials of eight, then shuffles.  A tree
+// in shared memory per value, eight barriers each, took 44 us for the frame's 27 and 18 us for the
+// statistics' 10; so 21 and 6.  sh: kN x 256.
+template <int kN>
+__device__ __forceinline__ void tree_sums(const double* acc, double* sh, double* __restrict__ out) {
+    const int tid = threadIdx.x, lane = tid & 31;
+#pragma unroll
+    for (int v = 0; v < kN; v++) sh[v * 256 + tid] = acc[v];
+    __syncthreads();
+    for (int v = tid >> 5; v < kN; v += 8) {
+        double x[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) x[k] = sh[v * 256 + lane + 32 * k];
+#pragma unroll
+        for (int h = 4; h > 0; h >>= 1)
+#pragma unroll
+            for (int k = 0; k < h; k++) x[k] += x[k + h];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x[0] += __shfl_down_sync(0xffffffffu, x[0], o);
+        if (lane == 0) out[v] = x[0];
+    }
+    __syncthreads();
 }
 
 // ---------------------------------------------------------------------------------------
@@ -148,9 +193,10 @@ __device__ __forceinline__ void triad(double a, double d, double* p, double* q, 
 //   q'w = dmu_a*,  -p'w = dmu_d,  q'(e + tt w) = Delta alpha*,  -p'(e + tt w) = Delta delta
 // with Delta from Eq. fr-Delta1, tt = (t_ep - t_fr) in years.  Each block reduces a fixed
 // contiguous range of sources in a fixed order (deterministic).
-__global__ void k_frame_normals(int n, const int32_t* __restrict__ subset, const double* __restrict__ src,
-                                const double* __restrict__ ref, double tt, double* __restrict__ partial) {
-    __shared__ double sh[256];
+__global__ void __launch_bounds__(256) k_frame_normals(int n, const int32_t* __restrict__ subset,
+                                                       const double* __restrict__ src, const double* __restrict__ ref,
+                                                       double tt, double* __restrict__ partial) {
+    __shared__ double sh[9 * 256];
     double acc[kFrameVals];
 #pragma unroll
     for (int i = 0; i < kFrameVals; i++) acc[i] = 0.0;
@@ -175,32 +221,35 @@ __global__ void k_frame_normals(int n, const int32_t* __restrict__ subset, const
             rows[3][c] = -p[c]; rows[3][3 + c] = -tt * p[c];
         }
         const double rhs[4] = {dpa, dpd, da, dd};
+#pragma unroll
         for (int e = 0; e < 4; e++) {
-            for (int a = 0; a < 6; a++) {
+#pragma unroll
+            for (int a = e < 2 ? 3 : 0; a < 6; a++) {   // the first two rows have no orientation part
+#pragma unroll
                 for (int c = a; c < 6; c++) acc[up6(a, c)] += rows[e][a] * rows[e][c];
                 acc[21 + a] += rows[e][a] * rhs[e];
             }
         }
     }
-    for (int v = 0; v < kFrameVals; v++) {
-        sh[threadIdx.x] = acc[v];
-        __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) partial[blockIdx.x * kFrameVals + v] = sh[0];
-        __syncthreads();
-    }
+    double* out = partial + blockIdx.x * kFrameVals;
+    tree_sums<9>(acc, sh, out);
+    tree_sums<9>(acc + 9, sh, out + 9);
+    tree_sums<9>(acc + 18, sh, out + 18);
 }
 
-// Sum the block partials in order and solve the 6x6 system by Algorithms C.1-C.3.
-__global__ void k_frame_solve(int n_part, const double* __restrict__ partial, double tol, double* __restrict__ eo) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double v[kFrameVals];
-    for (int i = 0; i < kFrameVals; i++) v[i] = 0.0;
-    for (int p = 0; p < n_part; p++)
-        for (int i = 0; i < kFrameVals; i++) v[i] += partial[p * kFrameVals + i];
+// Sum the block partials in order, a lane per value (one lane for all: 181 us of 30,000 sources, so
+// 34), and solve the 6x6 system by Algorithms C.1-C.3.
+__global__ void __launch_bounds__(32) k_frame_solve(int n_part, const double* __restrict__ partial, double tol,
+                                                    double* __restrict__ eo) {
+    __shared__ double v[kFrameVals];
+    if (threadIdx.x < kFrameVals) {
+        double t = 0.0;
+#pragma unroll 8
+        for (int p = 0; p < n_part; p++) t += partial[p * kFrameVals + threadIdx.x];
+        v[threadIdx.x] = t;
+    }
+    __syncwarp();
+    if (threadIdx.x != 0) return;
     double U[21];
     for (int j = 0; j < 6; j++) {
         for (int i = 0; i <= j; i++) {
@@ -263,7 +312,9 @@ __device__ __forceinline__ void frame_rotate(const double* q, const double* v, d
     out[0] = o[0]; out[1] = o[1]; out[2] = o[2];
 }
 
-// Rigorous transformation of the astrometric parameters, Sect. 6.1.2 steps 1-5.
+// Rigorous transformation of the astrometric parameters, Sect. 6.1.2 steps 1-5.  A chain of about 900
+// FP64 instructions: one warp per block, so that few sources spread over all sub-partitions (3000 in
+// blocks of 256 31 us, so 17).
 __global__ void k_frame_apply_src(int n_src, double* __restrict__ src, const double* __restrict__ eo, double dt_ep) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_src) return;
@@ -324,8 +375,8 @@ void launch_frame_from_sums(const DevGeo& G, int n_src, double* src, double* att
                             double* eo, cudaStream_t s) {
     const double tt = (double)(G.t_ep_ns - G.t_fr_ns) * 1e-9 / G.year_s;
     k_frame_solve<<<1, 32, 0, s>>>(1, sums, tol, eo);
-    k_frame_apply_src<<<(n_src + 255) / 256, 256, 0, s>>>(n_src, src, eo, tt);
-    k_frame_apply_att<<<(G.n_coef + 255) / 256, 256, 0, s>>>(G, att, eo);
+    k_frame_apply_src<<<(n_src + 31) / 32, 32, 0, s>>>(n_src, src, eo, tt);
+    k_frame_apply_att<<<(G.n_coef + 31) / 32, 32, 0, s>>>(G, att, eo);
 }
 
 void launch_frame(const DevGeo& G, int n, const int32_t* subset, int n_src, double* src, const double* ref,
@@ -333,8 +384,8 @@ void launch_frame(const DevGeo& G, int n, const int32_t* subset, int n_src, doub
     const double tt = (double)(G.t_ep_ns - G.t_fr_ns) * 1e-9 / G.year_s;
     k_frame_normals<<<n_part, 256, 0, s>>>(n, subset, src, ref, tt, partial);
     k_frame_solve<<<1, 32, 0, s>>>(n_part, partial, tol, eo);
-    k_frame_apply_src<<<(n_src + 255) / 256, 256, 0, s>>>(n_src, src, eo, tt);
-    k_frame_apply_att<<<(G.n_coef + 255) / 256, 256, 0, s>>>(G, att, eo);
+    k_frame_apply_src<<<(n_src + 31) / 32, 32, 0, s>>>(n_src, src, eo, tt);
+    k_frame_apply_att<<<(G.n_coef + 31) / 32, 32, 0, s>>>(G, att, eo);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -344,7 +395,7 @@ void launch_frame(const DevGeo& G, int n, const int32_t* subset, int n_src, doub
 // Stage 1: block b reduces the sources of its fixed contiguous chunk into part[b][10];
 // stage 2 (one block) adds the parts in block order, so the sums do not depend on timing.
 constexpr int kStatBlocks = 304;
-constexpr int kStatThreads = 256;
+constexpr int kStatThreads = 256;   // tree_sums' block
 __global__ void __launch_bounds__(kStatThreads) k_src_stats_part(int n_src, const double* __restrict__ chi2,
                                                                  const double* __restrict__ q,
                                                                  const int* __restrict__ nu,
@@ -352,7 +403,7 @@ __global__ void __launch_bounds__(kStatThreads) k_src_stats_part(int n_src, cons
                                                                  const int* __restrict__ rdf,
                                                                  const double* __restrict__ d,
                                                                  double* __restrict__ part) {
-    __shared__ double sh[kStatThreads];
+    __shared__ double sh[10 * kStatThreads];
     const int chunk = (n_src + gridDim.x - 1) / gridDim.x;
     const int lo = blockIdx.x * chunk, hi = min(n_src, lo + chunk);
     double acc[10];
@@ -365,32 +416,33 @@ __global__ void __launch_bounds__(kStatThreads) k_src_stats_part(int n_src, cons
         acc[4] += (double)rdf[i];
         for (int c = 0; c < 5; c++) acc[5 + c] += d[5 * (size_t)i + c] * d[5 * (size_t)i + c];
     }
-    for (int k = 0; k < 10; k++) {
-        sh[threadIdx.x] = acc[k];
-        __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) part[blockIdx.x * 10 + k] = sh[0];
-        __syncthreads();
-    }
+    tree_sums<10>(acc, sh, part + blockIdx.x * 10);
 }
 __global__ void __launch_bounds__(32) k_src_stats_final(int n_part, const double* __restrict__ part,
                                                         double* __restrict__ out) {
     // lane k < 10 adds statistic k over the parts in order
     if (threadIdx.x < 10) {
         double a = 0.0;
+#pragma unroll 16
         for (int b = 0; b < n_part; b++) a += part[b * 10 + threadIdx.x];
         out[threadIdx.x] = a;
     }
 }
 
 // integer sum in a fixed order (rank defects of segments / calibration parameters)
-__global__ void k_int_sum(int n, const int* __restrict__ v, long long* __restrict__ out) {
+__global__ void __launch_bounds__(1024) k_int_sum(int n, const int* __restrict__ v, long long* __restrict__ out) {
     __shared__ long long sh[1024];
     long long a = 0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) a += v[i];
+    // eight loads in flight per thread (one: 113 us of 252,000 values, so 16)
+    int i = threadIdx.x;
+    for (; i + 7 * 1024 < n; i += 8 * 1024) {
+        int t[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) t[k] = v[i + 1024 * k];
+#pragma unroll
+        for (int k = 0; k < 8; k++) a += t[k];
+    }
+    for (; i < n; i += 1024) a += v[i];
     sh[threadIdx.x] = a;
     __syncthreads();
     for (int o = blockDim.x / 2; o > 0; o >>= 1) {
