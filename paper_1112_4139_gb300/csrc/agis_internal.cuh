@@ -204,6 +204,7 @@ struct __align__(16) SrcWork {
     double d[5];       // solution of the latest round
     double isd[2];     // 1 / sqrt(sigma_c^2 + eps^2); after the last round 1 / (sigma_c^2 + eps^2)
     int32_t flags;     // 1: one sigma per class, 2: no observations, 0: the general path
+    int32_t all[2];    // per class: C is the weighted sums of all rows, T is not used
     int32_t nout;      // observations with w < 0.2
 };
 

@@ -209,6 +209,7 @@ __device__ __forceinline__ void reduce_vals(double* v, int lane, double* out) {
 // the rows listed in shared memory (m <= 32 of them), lane by lane.  first: w = wfun(h rx), the
 // initial downweighting by the robust scale; else w = wfun((h - A d) isd).  last: w goes to the
 // scratch row for the hand-over records.
+template <bool kAll = false>
 __device__ __forceinline__ void subtract_rows(double* scr, const uint32_t* list, int m, int lane, bool first,
                                               const double* d, double scale, int wfn, bool last, double* corr,
                                               int& nout) {
@@ -219,7 +220,7 @@ __device__ __forceinline__ void subtract_rows(double* scr, const uint32_t* list,
     const double w = wfun((first ? h : h - row_dot(A, d)) * scale, wfn);
     if (last) e[6] = w;
     nout += w < 0.2;
-    const double u = 1.0 - w;
+    const double u = kAll ? w : 1.0 - w;
 #pragma unroll
     for (int a = 0; a < 5; a++) {
         const double ua = u * A[a];
@@ -228,6 +229,20 @@ __device__ __forceinline__ void subtract_rows(double* scr, const uint32_t* list,
         corr[15 + a] = fma(ua, h, corr[15 + a]);
     }
     corr[20] = fma(u * h, h, corr[20]);
+}
+
+// Sums of w times the products over all rows of a class: where more than a third of them are
+// downweighted, the unit-weight sums would cancel against what is taken off.
+__device__ __noinline__ void direct_rows(double* scr, int lo, int hi, uint32_t* list, int lane, bool first, const double* d,
+                                         double scale, int wfn, bool last, double* sums, int& nout) {
+#pragma unroll
+    for (int k = 0; k < kSumVals; k++) sums[k] = 0.0;
+    for (int j0 = lo; j0 < hi; j0 += kWarp) {
+        list[lane] = (uint32_t)(j0 + lane);
+        __syncwarp();
+        subtract_rows<true>(scr, list, min(hi - j0, kWarp), lane, first, d, scale, wfn, last, sums, nout);
+        __syncwarp();
+    }
 }
 
 // Appends the row j of every lane with cand set to the list (n entries so far); a full list of 32
@@ -356,24 +371,25 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_first(Settings st, cons
             if (!uni) continue;
             const bool last = st.robust ? st.n_rounds == 0 : true;
             int nout = 0;
-            if (kDirect) {
+            if constexpr (kDirect) {
                 // round 0's weights are wfun(h rx); all 1 for a robust scale of 0
                 if (lane < 2) w.isd[lane] = vs > 0.0 ? 1.0 / (sqrt(lane ? s2c[1] : s2c[0]) * vs) : 0.0;
+                if (lane < 2) w.all[lane] = 0;
                 for (int k = lane; k < kRedVals; k += kWarp) (&w.C[0][0])[k] = 0.0;
                 continue;
-            }
+            } else
             for (int c = 0; c < 2; c++) {
                 const int lo = c ? nal : 0, hi = c ? n : nal;
                 double corr[kSumVals];
 #pragma unroll
                 for (int k = 0; k < kSumVals; k++) corr[k] = 0.0;
-                int m = 0;
-                bool any = false;
+                int m = 0, listed = 0;
+                const int nout0 = nout;
                 const double rx = vs > 0.0 ? 1.0 / (sqrt(s2c[c]) * vs) : 0.0;
                 const float ivs = (float)(1.0 / vs);
                 auto flush = [&](int k) {
                     subtract_rows(scr, list, k, lane, true, nullptr, rx, st.weight_fn, last, corr, nout);
-                    any = true;
+                    listed += k;
                 };
                 if (st.robust && rx > 0.0)
                     for (int j0 = lo; j0 < hi; j0 += kWarp) {
@@ -388,7 +404,17 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_first(Settings st, cons
                 __syncwarp();
                 if (m > 0) flush(m);
                 __syncwarp();
-                if (any) reduce_vals(corr, lane, w.C[c]);
+                const bool all = 3 * listed > hi - lo;
+                if (all) {
+                    double sums[kSumVals];   // (in memory: corr stays in registers)
+                    int cnt = 0;
+                    direct_rows(scr, lo, hi, list, lane, true, nullptr, rx, st.weight_fn, last, sums, cnt);
+                    nout = nout0 + cnt;
+#pragma unroll
+                    for (int k = 0; k < kSumVals; k++) corr[k] = sums[k];
+                }
+                if (lane == 0) w.all[c] = all;
+                if (listed) reduce_vals(corr, lane, w.C[c]);
                 else if (lane < kSumVals) w.C[c][lane] = 0.0;
             }
             nout = warp_sum_int(nout);
@@ -429,11 +455,11 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_round(Settings st, int 
                 double corr[kSumVals];
 #pragma unroll
                 for (int k = 0; k < kSumVals; k++) corr[k] = 0.0;
-                int m = 0;
-                bool any = false;
+                int m = 0, listed = 0;
+                const int nout0 = nout;
                 auto flush = [&](int k) {
                     subtract_rows(scr, list, k, lane, false, d, isd, st.weight_fn, last, corr, nout);
-                    any = true;
+                    listed += k;
                 };
                 auto screen = [&](double h, const double A[5]) {
                     const float hf = trunc_f32(h);
@@ -463,7 +489,17 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_round(Settings st, int 
                 __syncwarp();
                 if (m > 0) flush(m);
                 __syncwarp();
-                if (any) reduce_vals(corr, lane, w.C[c]);
+                const bool all = 3 * listed > hi - lo;
+                if (all) {
+                    double sums[kSumVals];   // (in memory: corr stays in registers)
+                    int cnt = 0;
+                    direct_rows(scr, lo, hi, list, lane, false, d, isd, st.weight_fn, last, sums, cnt);
+                    nout = nout0 + cnt;
+#pragma unroll
+                    for (int k = 0; k < kSumVals; k++) corr[k] = sums[k];
+                }
+                if (lane == 0) w.all[c] = all;
+                if (listed) reduce_vals(corr, lane, w.C[c]);
                 else if (lane < kSumVals) w.C[c][lane] = 0.0;
             }
             nout = warp_sum_int(nout);
@@ -657,20 +693,22 @@ __global__ void __launch_bounds__(128) k_src_solve5(Settings st, int last, const
     const int n = (int)(src_off[i + 1] - src_off[i]);
     ClassSums S;
     HalfSums H;
+    const int all[2] = {w.all[0], w.all[1]};
+    auto sum_of = [&](int c, int k) { return (c ? all[1] : all[0]) ? w.C[c][k] : w.T[c][k] - w.C[c][k]; };
     if (kPair) {
         for (int c = 0; c < 2; c++)
-            for (int k = 0; k < 10; k++) H.E[c][k] = w.T[c][10 * h + k] - w.C[c][10 * h + k];
-        for (int k = 0; k < 15; k++) H.AA[k] = w.T[h][k] - w.C[h][k];
-        for (int k = 0; k < 5; k++) H.Ah[k] = w.T[h][15 + k] - w.C[h][15 + k];
-        H.hh = w.T[h][20] - w.C[h][20];
+            for (int k = 0; k < 10; k++) H.E[c][k] = sum_of(c, 10 * h + k);
+        for (int k = 0; k < 15; k++) H.AA[k] = sum_of(h, k);
+        for (int k = 0; k < 5; k++) H.Ah[k] = sum_of(h, 15 + k);
+        H.hh = sum_of(h, 20);
     } else {
 #pragma unroll
         for (int c = 0; c < 2; c++) {
 #pragma unroll
-            for (int k = 0; k < 15; k++) S.AA[c][k] = w.T[c][k] - w.C[c][k];
+            for (int k = 0; k < 15; k++) S.AA[c][k] = sum_of(c, k);
 #pragma unroll
-            for (int k = 0; k < 5; k++) S.Ah[c][k] = w.T[c][15 + k] - w.C[c][15 + k];
-            S.hh[c] = w.T[c][20] - w.C[c][20];
+            for (int k = 0; k < 5; k++) S.Ah[c][k] = sum_of(c, 15 + k);
+            S.hh[c] = sum_of(c, 20);
         }
     }
     const double s2c[2] = {w.s2c[0], w.s2c[1]};
@@ -991,7 +1029,7 @@ void launch_obs_pass(const DevGeo& G, const AttNoise& an, const int64_t* t_ns, c
                      const double* mu, const int32_t* obs_src, int64_t n_obs, int32_t n_src, const double* src,
                      const double* att, const double* cal, ObsRec* rec, double* geo, double* scratch,
                      uint64_t* skey, const Shapes& sh, cudaStream_t stream) {
-    k_src_geo<<<(n_src + 255) / 256 > 0 ? (n_src + 255) / 256 : 1, 256, 0, stream>>>(n_src, src, geo);
+    k_src_geo<<<n_src > 0 ? (n_src + 31) / 32 : 1, 32, 0, stream>>>(n_src, src, geo);
     const int th = sh.obs_threads;
     int64_t fb = (n_obs + th - 1) / th;
     if (fb > 152 * (int64_t)sh.obs_bps) fb = 152 * (int64_t)sh.obs_bps;
@@ -1042,7 +1080,7 @@ void launch_source_solve(const Settings& st, bool corrections, const int64_t* sr
 }
 
 void launch_src_geo(int32_t n_src, const double* src, double* geo, cudaStream_t s) {
-    k_src_geo<<<(n_src + 255) / 256 > 0 ? (n_src + 255) / 256 : 1, 256, 0, s>>>(n_src, src, geo);
+    k_src_geo<<<n_src > 0 ? (n_src + 31) / 32 : 1, 32, 0, s>>>(n_src, src, geo);
 }
 
 void launch_evaluate(const DevGeo& G, const int64_t* t_ns, const uint32_t* meta, const double* mu,

@@ -41,7 +41,7 @@ def _cut(ds, keep):
 
 
 @pytest.mark.parametrize("weight_fn", ["agis", "huber"])
-@pytest.mark.parametrize("shape", ["long", "mixed", "tied", "varied"])
+@pytest.mark.parametrize("shape", ["long", "mixed", "tied", "varied", "offset"])
 def test_source_update_matches_oracle(base, shape, weight_fn):
     import paper_1112_4139_gb300 as pkg
     pkg.build()
@@ -64,9 +64,11 @@ def test_source_update_matches_oracle(base, shape, weight_fn):
     # attitude and calibration at the truth: residuals at the noise level, weights that differ
     sub = ds.subset_sources(np.arange(N_CMP))
     P = OM.problem_from_dataset(sub)
-    src1, sres, _ = OB.source_update(P, sub.src0, ds.att_true, ds.cal_true, OB.Settings(weight_fn=weight_fn))
+    # an offset of every residual by ten sigma: most rows are downweighted
+    cal = ds.cal_true + (10.0 * float(np.median(ds.sigma)) if shape == "offset" else 0.0)
+    src1, sres, _ = OB.source_update(P, sub.src0, ds.att_true, cal, OB.Settings(weight_fn=weight_fn))
     g = agis.from_dataset(ds, weight_fn=0 if weight_fn == "agis" else 1)
-    g.set_state(src=ds.src0, att=ds.att_true, cal=ds.cal_true)
+    g.set_state(src=ds.src0, att=ds.att_true, cal=cal)
     g.source_update()
     ss = {k: v[:N_CMP] for k, v in g.source_stats().items()}
     R, W = (v[:sub.n_obs] for v in g.residuals())
