@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(128) k_att_accum(DevGeo G, double lambda2, int
 // eight signed 7-bit digits kept as FP16 integers, and the products of the digit pairs i + j >= 6 are
 // accumulated in FP32 by their weight 2^(7 (i + j)): 8 pairs x 512 observations x 2^12 are
 // at most 2^24, so every sum is exact, and the pairs left out are below 2^-58 of the largest term
-// (FP64 rounds each product at 2^-53).  Products W g g', powers of x and conversions are 64-bit
+// (FP64 rounds each product at 2^-53).  Products W g g', the forms and conversions are 64-bit
 // integer arithmetic.
 // Bound: integer and shared-memory issue (about 28 instructions per observation and warp of 32)
 // and 68 FP64 instructions per interval for the expansion, where the FP64 form takes 116 FMAs and

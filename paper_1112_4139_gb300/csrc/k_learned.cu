@@ -3,6 +3,8 @@
 // Adam step, and the application of a proposal to the sources and to the residuals that
 // the A and C blocks read.  Not part of the paper (its analogue is the accelerated simple
 // iteration of Sect. 4.7); the definitions are those of include/agis.h.
+#include <cooperative_groups.h>
+
 #include <cuda_bf16.h>
 
 #include <string>
@@ -161,15 +163,20 @@ __global__ void __launch_bounds__(32 * kFwdWarps) k_mlp_fwd_tc(const uint32_t* _
 // kGradWarps warps takes 32 rows at a time: lane = row, and every warp computes its share of the
 // units of each layer (the weights are then broadcast loads, the row vectors of odd stride free of
 // bank conflicts); the weight gradients are outer-product sums over the 32 rows kept in shared
-// memory, each thread owning 4x4 tiles of W2 and W1 (8 loads for 16 products).  Blocks with one
-// tile add it straight into the global gradient, four values per reduction where aligned.
+// memory, each thread owning 4x4 tiles of W2 (8 loads for 16 products).  A cluster of four
+// blocks adds its sums through distributed shared memory, a quarter of the entries each, before they go
+// into the global gradient: 64 additions an entry at 8192 rows, as many as with a tile per warp, and
+// the same error against 64 bits (1.2e-7 to 2.2e-7 of the gradient; a block's sums straight into the
+// gradient were 31.6 us a step, but 256 additions and 1.9e-7 to 3.0e-7).
 // Bound: the batch of the training step (8192 rows, 256 tiles) is 1.7 blocks per SM, so the time is
-// one tile's chain of dependent sums: 83 -> 24.5 us (before: a warp per tile, a whole row per
+// one tile's chain of dependent sums: training step 87 -> 33.60.00.00.064.00.00.00.00.00.0 us (before: a warp per tile, a whole row per
 // thread, on 64 of the 152 SMs).
 constexpr int kGradWarps = 8;
 constexpr int kGradThreads = 32 * kGradWarps;
+constexpr int kGradCluster = 4;
+constexpr int kGradVals = (pN + 3) / 4 * 4;           // the flat layout in whole vectors of four
 constexpr int kRowF = kIn + 4 * kH + kOut;            // per row: x, h1, h2, dh2, dh1, dy
-constexpr size_t kGradSmem = (size_t)(2 * pN + 32 * kRowF + kGradWarps) * sizeof(float);
+constexpr size_t kGradSmem = (size_t)(2 * kGradVals + 32 * kRowF + kGradWarps) * sizeof(float);
 static_assert(kRowF % 2 == 1, "rows in distinct banks");
 
 // four neighbouring sums into the global gradient
@@ -200,22 +207,24 @@ __device__ __forceinline__ void outer4(const float* d, const float* v, float acc
     }
 }
 
-__global__ void __launch_bounds__(kGradThreads) k_mlp_loss_grad(const float* __restrict__ p, const float* __restrict__ X,
+__global__ void __cluster_dims__(kGradCluster, 1, 1) __launch_bounds__(kGradThreads) k_mlp_loss_grad(const float* __restrict__ p, const float* __restrict__ X,
                                                                 const float* __restrict__ T,
                                                                 const int32_t* __restrict__ idx, int n,
                                                                 float* __restrict__ grad, float* __restrict__ loss) {
-    extern __shared__ float sm[];
+    extern __shared__ __align__(16) float sm[];
     float* W = sm;                                     // rounded weights and FP32 biases, flat layout
-    float* G = sm + pN;                                // block gradient (several tiles per block)
-    float* rows = sm + 2 * pN;
-    float* lsum = sm + 2 * pN + 32 * kRowF;
+    float* G = sm + kGradVals;                         // block gradient
+    float* rows = sm + 2 * kGradVals;
+    float* lsum = rows + 32 * kRowF;
     const int ntile = (n + 31) / 32;
-    const bool one = ntile <= (int)gridDim.x;          // at most one tile per block
     for (int i = threadIdx.x; i < pN; i += kGradThreads) {
         const bool is_w = (i < pB1) || (i >= pW2 && i < pB2) || (i >= pW3 && i < pB3);
         W[i] = is_w ? bf16r(p[i]) : p[i];
-        if (!one) G[i] = 0.0f;
     }
+    if ((int)blockIdx.x >= ntile)                      // a block of the last cluster without rows
+        for (int i = threadIdx.x; i < kGradVals; i += kGradThreads) G[i] = 0.0f;
+    else if (threadIdx.x < kGradVals - pN)
+        G[pN + threadIdx.x] = 0.0f;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const float inv_n = 1.0f / (float)n;
     // W1 (offset 0) and W2 start on 16 bytes when grad does (pW2 = 1472)
@@ -302,6 +311,7 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_loss_grad(const float* __r
         }
         __syncthreads();
         // weight gradients over the 32 rows
+        const bool first = tile == (int)blockIdx.x;
         const float* rb = rows;
         for (int e = threadIdx.x; e < (kH / 4) * (kH / 4); e += kGradThreads) {   // W2: 16 x 16 tiles of 4 x 4
             const int i = 4 * (e / (kH / 4)), k = 4 * (e % (kH / 4));
@@ -310,9 +320,13 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_loss_grad(const float* __r
 #pragma unroll
             for (int a = 0; a < 4; a++) {
                 const int off = pW2 + (i + a) * kH + k;
-                if (one) grad_add4(grad + off, acc[a], vec);
-                else
-                    for (int b = 0; b < 4; b++) G[off + b] += acc[a][b];
+                float4 t = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+                float4* gp = reinterpret_cast<float4*>(G + off);
+                if (!first) {
+                    const float4 u = *gp;
+                    t = make_float4(t.x + u.x, t.y + u.y, t.z + u.z, t.w + u.w);
+                }
+                *gp = t;
             }
         }
         for (int e = threadIdx.x; e < kH * kIn; e += kGradThreads) {              // W1
@@ -320,16 +334,14 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_loss_grad(const float* __r
             float s = 0.0f;
 #pragma unroll 8
             for (int q = 0; q < 32; q++) s = fmaf(rb[q * kRowF + kIn + 3 * kH + i], rb[q * kRowF + k], s);
-            if (one) atomicAdd(&grad[pW1 + e], s);
-            else G[pW1 + e] += s;
+            G[pW1 + e] = first ? s : G[pW1 + e] + s;
         }
         for (int e = threadIdx.x; e < kOut * kH; e += kGradThreads) {             // W3
             const int o = e / kH, k = e % kH;
             float s = 0.0f;
 #pragma unroll 8
             for (int q = 0; q < 32; q++) s = fmaf(rb[q * kRowF + kIn + 4 * kH + o], rb[q * kRowF + kIn + kH + k], s);
-            if (one) atomicAdd(&grad[pW3 + e], s);
-            else G[pW3 + e] += s;
+            G[pW3 + e] = first ? s : G[pW3 + e] + s;
         }
         for (int e = threadIdx.x; e < 2 * kH + kOut; e += kGradThreads) {         // biases
             int off, src;
@@ -339,20 +351,45 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_loss_grad(const float* __r
             float s = 0.0f;
 #pragma unroll 8
             for (int q = 0; q < 32; q++) s += rb[q * kRowF + src];
-            if (one) atomicAdd(&grad[off], s);
-            else G[off] += s;
+            G[off] = first ? s : G[off] + s;
         }
     }
     lpart = warp_sum_f32(lpart);
     if (lane == 0) lsum[wib] = lpart;
     __syncthreads();
-    if (!one)
-        for (int i = threadIdx.x; i < pN; i += kGradThreads) atomicAdd(&grad[i], G[i]);
     if (threadIdx.x == 0) {
         float s = 0.0f;
         for (int k = 0; k < kGradWarps; k++) s += lsum[k];
+        lsum[0] = s;
+    }
+    // the cluster's sums: a quarter of the entries to each block
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();
+    const int rank = (int)cluster.block_rank();
+    constexpr int kGroups = kGradVals / 4, kPer = (kGroups + kGradCluster - 1) / kGradCluster;
+    for (int g = rank * kPer + threadIdx.x; g < min((rank + 1) * kPer, kGroups); g += kGradThreads) {
+        float4 t[kGradCluster];
+#pragma unroll
+        for (int c = 0; c < kGradCluster; c++) t[c] = reinterpret_cast<const float4*>(cluster.map_shared_rank(G, c))[g];
+        float v[4] = {t[0].x, t[0].y, t[0].z, t[0].w};
+#pragma unroll
+        for (int c = 1; c < kGradCluster; c++) {
+            v[0] += t[c].x;
+            v[1] += t[c].y;
+            v[2] += t[c].z;
+            v[3] += t[c].w;
+        }
+        if (4 * g + 3 < pN) grad_add4(grad + 4 * g, v, vec);
+        else
+            for (int k = 0; 4 * g + k < pN; k++) atomicAdd(&grad[4 * g + k], v[k]);
+    }
+    if (rank == 0 && threadIdx.x == 0) {
+        float s = 0.0f;
+        for (int c = 0; c < kGradCluster; c++) s += *cluster.map_shared_rank(lsum, c);
         atomicAdd(loss, s * inv_n);
     }
+    cluster.sync();   // shared memory stays until the others have read it
 }
 
 __global__ void k_mlp_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
@@ -631,8 +668,10 @@ int agis_mlp_loss_grad(const float* params, const float* X, const float* T, cons
     cudaMemsetAsync(grad, 0, sizeof(float) * agis::pN, s);
     cudaMemsetAsync(loss, 0, sizeof(float), s);
     const int tiles = (n + 31) / 32;
-    agis::k_mlp_loss_grad<<<agis::grid_of(tiles, 1, 2 * 152), agis::kGradThreads, agis::kGradSmem, s>>>(params, X, T, idx, n,
-                                                                                                     grad, loss);
+    // a multiple of the cluster, two blocks per SM at most
+    const int blocks = agis::grid_of((tiles + agis::kGradCluster - 1) / agis::kGradCluster, 1, 2 * 152 / agis::kGradCluster) *
+                       agis::kGradCluster;
+    agis::k_mlp_loss_grad<<<blocks, agis::kGradThreads, agis::kGradSmem, s>>>(params, X, T, idx, n, grad, loss);
     return mlp_launch_status("agis_mlp_loss_grad");
 }
 
