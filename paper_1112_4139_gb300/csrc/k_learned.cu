@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(32 * kFwdWarps) k_mlp_fwd_tc(const uint32_t* _
 // the same error against 64 bits (1.2e-7 to 2.2e-7 of the gradient; a block's sums straight into the
 // gradient were 31.6 us a step, but 256 additions and 1.9e-7 to 3.0e-7).
 // Bound: the batch of the training step (8192 rows, 256 tiles) is 1.7 blocks per SM, so the time is
-// one tile's chain of dependent sums: training step 87 -> 33.60.00.00.064.00.00.00.00.00.0 us (before: a warp per tile, a whole row per
+// one tile's chain of dependent sums: training step 87 -> 33.6 us (before: a warp per tile, a whole row per
 // thread, on 64 of the 152 SMs).
 constexpr int kGradWarps = 8;
 constexpr int kGradThreads = 32 * kGradWarps;
