@@ -928,6 +928,9 @@ static __device__ bool select_quantiles(const uint64_t* __restrict__ keys, int n
         const int m = sw.hist[bin[2 * p]] + (bin[2 * p + 1] != bin[2 * p] ? sw.hist[bin[2 * p + 1]] : 0);
         ok = ok && m <= kSelCap;
     }
+    // the radix select that follows a refusal clears this histogram: no lane may still be reading it
+    ok = __all_sync(0xffffffffu, ok);
+    __syncwarp();
     if (!ok) return false;
     for (int j = lane; j < n; j += kWarp) {
         const uint64_t key = keys[j];
