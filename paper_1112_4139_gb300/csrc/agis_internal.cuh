@@ -197,8 +197,8 @@ struct SrcOutPtrs {
 
 // Per-source state of the FP64 S block between its kernels (class-sum path).
 struct __align__(16) SrcWork {
-    double T[2][21];   // unit-weight sums per class: 15 AA, 5 Ah, hh
-    double C[2][21];   // what the round's weights take off: sums of (1 - w) times the same products
+    double T[2][21];   // unit-weight sums per class over the rows within two robust scales: 15 AA, 5 Ah, hh
+    double C[2][21];   // what the round's weights add: (w - 1) times the same products, w for the other rows
     double s2c[2];     // sigma^2 of the AL and AC observations (one value per class)
     double s2min, vs;  // smallest sigma^2; robust scale of x = h / sigma
     double d[5];       // solution of the latest round

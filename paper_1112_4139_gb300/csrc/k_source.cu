@@ -14,9 +14,9 @@
 // What bounds it: FP64 issue (2 FMA per clock and SM).  A 5x5 solve of one lane costs a warp as
 // many FP64 cycles as 32 of them, hence a thread per source there.  Downweighting leaves w = 1
 // wherever |z| <= 2 (Eqs. dw, dwH), about 95% of the observations, so for long sources the 21
-// products of a row are summed once, with unit weights; a round evaluates z in FP32 (with a bound
-// on its error), and only the rows that may exceed 2 are gathered, 32 to a warp, for the FP64
-// weight and the 27 products that (1 - w) takes off again: a round then costs about a fifth of
+// products of a row within two robust scales are summed once, with unit weights; a round evaluates z in
+// FP32 (with a bound on its error), and only the rows that may exceed 2 or that those sums do not hold are
+// gathered, 32 to a warp, for the FP64 weight and 27 products: a round then costs about a fifth of
 // the FP64 work of the direct sums.
 // Measured, source solves of the S block: 24.7M observations of 30,000 sources 14.2 -> 4.5 ms; with
 // direct sums 6.7M of 8000 sources 4.75 -> 2.9, 0.5M of 3000 sources 1.68 -> 0.57.  Before, one persistent
@@ -137,7 +137,7 @@ __global__ void k_src_geo(int32_t n_src, const double* __restrict__ src, double*
 }
 
 // Observation pass, one thread per observation (source order): residual h, design row A and
-// attitude partial g at the current parameters.  Scratch row: h, A[5], key(h/sigma), sigma^2;
+// attitude partial g at the current parameters.  Scratch row: h, A[5], weight 1, sigma^2;
 // with the excess attitude noise on, sigma~^2 = sigma^2 + eps_a^2(t) in place of sigma^2 (Eq. W).
 __global__ void __launch_bounds__(256) k_obs_forward(DevGeo G, AttNoise an, int64_t n_obs, const int64_t* __restrict__ t_ns,
                                                      const uint32_t* __restrict__ meta,
@@ -166,6 +166,7 @@ __global__ void __launch_bounds__(256) k_obs_forward(DevGeo G, AttNoise an, int6
         e[0] = ob.R;
         e[1] = ob.A[0]; e[2] = ob.A[1]; e[3] = ob.A[2]; e[4] = ob.A[3]; e[5] = ob.A[4];
         skey[o] = dkey(x);
+        e[6] = 1.0;
         e[7] = s2;
         ObsRec* r = rec + o;
         r->t_ns = t;
@@ -205,22 +206,24 @@ __device__ __forceinline__ void reduce_vals(double* v, int lane, double* out) {
     if (cnt > 0) out[off] = v[0];
 }
 
-// What a round subtracts from the unit-weight sums of one class: (1 - w) times the products of
-// the rows listed in shared memory (m <= 32 of them), lane by lane.  first: w = wfun(h rx), the
-// initial downweighting by the robust scale; else w = wfun((h - A d) isd).  last: w goes to the
-// scratch row for the hand-over records.
-template <bool kAll = false>
-__device__ __forceinline__ void subtract_rows(double* scr, const uint32_t* list, int m, int lane, bool first,
-                                              const double* d, double scale, int wfn, bool last, double* corr,
-                                              int& nout) {
+// Adds u times the products of the rows listed in shared memory (m <= 32 of them) to corr, lane by
+// lane.  first: w = wfun(h rx), the initial downweighting by the robust scale; else w = wfun((h - A d)
+// isd).  kAll: u = w.  Otherwise a row that the unit-weight sums hold (weight slot 1) takes u = w - 1
+// and counts into what is taken off (sub_n rows, sub_hh of h^2), one that they do not hold (weight
+// slot 0) takes u = w.  last: w goes to the scratch row for the hand-over records.
+template <bool kAll>
+__device__ __forceinline__ void weigh_rows(double* scr, const uint32_t* list, int m, int lane, bool first,
+                                           const double* d, double scale, int wfn, bool last, double* corr, int& nout,
+                                           int& sub_n, double& sub_hh) {
     if (lane >= m) return;
     double* e = scr + (size_t)list[lane] * kScr;
     double h, A[5];
     row_load(e, h, A);
     const double w = wfun((first ? h : h - row_dot(A, d)) * scale, wfn);
+    const bool held = !kAll && e[6] != 0.0;
     if (last) e[6] = w;
     nout += w < 0.2;
-    const double u = kAll ? w : 1.0 - w;
+    const double u = held ? w - 1.0 : w;
 #pragma unroll
     for (int a = 0; a < 5; a++) {
         const double ua = u * A[a];
@@ -228,19 +231,26 @@ __device__ __forceinline__ void subtract_rows(double* scr, const uint32_t* list,
         for (int b = a; b < 5; b++) corr[up5(a, b)] = fma(ua, A[b], corr[up5(a, b)]);
         corr[15 + a] = fma(ua, h, corr[15 + a]);
     }
-    corr[20] = fma(u * h, h, corr[20]);
+    const double uh = u * h;
+    corr[20] = fma(uh, h, corr[20]);
+    if (held) {
+        sub_n++;
+        sub_hh = fma(-uh, h, sub_hh);
+    }
 }
 
-// Sums of w times the products over all rows of a class: where more than a third of them are
-// downweighted, the unit-weight sums would cancel against what is taken off.
-__device__ __noinline__ void direct_rows(double* scr, int lo, int hi, uint32_t* list, int lane, bool first, const double* d,
-                                         double scale, int wfn, bool last, double* sums, int& nout) {
+// Sums of w times the products over all rows of a class, for rounds that would take off too much of
+// the unit-weight sums.
+__device__ __noinline__ void direct_rows(double* scr, int lo, int hi, uint32_t* list, int lane, const double* d, double scale,
+                                         int wfn, bool last, double* sums, int& nout) {
+    int sub_n = 0;
+    double sub_hh = 0.0;
 #pragma unroll
     for (int k = 0; k < kSumVals; k++) sums[k] = 0.0;
     for (int j0 = lo; j0 < hi; j0 += kWarp) {
         list[lane] = (uint32_t)(j0 + lane);
         __syncwarp();
-        subtract_rows<true>(scr, list, min(hi - j0, kWarp), lane, first, d, scale, wfn, last, sums, nout);
+        weigh_rows<true>(scr, list, min(hi - j0, kWarp), lane, false, d, scale, wfn, last, sums, nout, sub_n, sub_hh);
         __syncwarp();
     }
 }
@@ -263,7 +273,10 @@ __device__ __forceinline__ void append_rows(bool cand, int j, uint32_t* list, in
 }
 
 // Per source: sigma per class, robust scale of x = h / sigma (Sect. 5.1.2: half the intersextile
-// range), unit-weight class sums, and round 0's downweighting.
+// range), unit-weight class sums, and round 0's downweighting.  The unit-weight sums hold the rows with
+// |x| below twice the robust scale and no others: a row further out (5 to 8% of them, however far) has
+// 0 in its weight slot and is added with its weight in every round, so that nothing large is ever
+// summed only to be taken off again.  A robust scale of 0 leaves all rows to be added.
 template <bool kDirect>
 __global__ void __launch_bounds__(32 * kPassWarps) k_src_first(Settings st, const int64_t* __restrict__ src_off,
                                                                const int32_t* __restrict__ src_nal,
@@ -288,46 +301,6 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_first(Settings st, cons
                 continue;
             }
             double* scr = scratch + (size_t)o0 * kScr;
-            // unit-weight sums and sigma of each class; sums only while its sigma is one value
-            // (bit patterns: variances are not negative, and comparisons hold the FP64 unit)
-            double s2c[2] = {1.0, 1.0};
-            uint64_t s2m = __double_as_longlong(1e300);
-            bool uni = true;
-            for (int c = 0; c < 2; c++) {
-                const int lo = c ? nal : 0, hi = c ? n : nal;
-                double v[kSumVals];
-#pragma unroll
-                for (int k = 0; k < kSumVals; k++) v[k] = 0.0;
-                if (lo < hi) {
-                    const double s2 = scr[(size_t)lo * kScr + 7];
-                    const uint64_t s2b = __double_as_longlong(s2);
-                    bool same = s2 == s2;
-                    for (int j0 = lo; j0 < hi; j0 += kWarp) {
-                        const int j = j0 + lane;
-                        if (j < hi) {
-                            const double* e = scr + (size_t)j * kScr;
-                            const uint64_t sj = __double_as_longlong(e[7]);
-                            s2m = sj < s2m ? sj : s2m;
-                            same = same && sj == s2b;
-                            if (!kDirect && uni) {
-                                double h, A[5];
-                                row_load(e, h, A);
-#pragma unroll
-                                for (int a = 0; a < 5; a++) {
-#pragma unroll
-                                    for (int b = a; b < 5; b++) v[up5(a, b)] = fma(A[a], A[b], v[up5(a, b)]);
-                                    v[15 + a] = fma(A[a], h, v[15 + a]);
-                                }
-                                v[20] = fma(h, h, v[20]);
-                            }
-                        }
-                        uni = __all_sync(0xffffffffu, uni && same);
-                    }
-                    s2c[c] = s2;
-                }
-                if (!kDirect && uni) reduce_vals(v, lane, w.T[c]);
-            }
-            const double s2min = warp_min(__longlong_as_double(s2m));
             double vs = 0.0;
             const bool in_smem = n <= kKeyCap64;
             const uint64_t* keys = in_smem ? sw.keys : skey + o0;
@@ -361,6 +334,55 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_first(Settings st, cons
                 vs = 0.5 * ((x[2] + g5 * (x[3] - x[2])) - (x[0] + g1 * (x[1] - x[0])));
                 __syncwarp();
             }
+            // x of the key, to 2^-22 relative: at or above 2 robust scales within that, or not finite
+            const float ivs = (float)(1.0 / vs);
+            auto beyond = [&](int j) {
+                return st.robust && !(fabsf(trunc_f32(dkey_inv(keys[j])) * ivs) < 1.99999f);
+            };
+            // unit-weight sums and sigma of each class; sums only while its sigma is one value
+            // (bit patterns: variances are not negative, and comparisons hold the FP64 unit)
+            double s2c[2] = {1.0, 1.0};
+            uint64_t s2m = __double_as_longlong(1e300);
+            bool uni = true;
+            for (int c = 0; c < 2; c++) {
+                const int lo = c ? nal : 0, hi = c ? n : nal;
+                double v[kSumVals];
+#pragma unroll
+                for (int k = 0; k < kSumVals; k++) v[k] = 0.0;
+                if (lo < hi) {
+                    const double s2 = scr[(size_t)lo * kScr + 7];
+                    const uint64_t s2b = __double_as_longlong(s2);
+                    bool same = s2 == s2;
+                    for (int j0 = lo; j0 < hi; j0 += kWarp) {
+                        const int j = j0 + lane;
+                        if (j < hi) {
+                            double* e = scr + (size_t)j * kScr;
+                            const uint64_t sj = __double_as_longlong(e[7]);
+                            s2m = sj < s2m ? sj : s2m;
+                            same = same && sj == s2b;
+                            if (!kDirect && uni) {
+                                double h, A[5];
+                                row_load(e, h, A);
+                                if (beyond(j)) {
+                                    e[6] = 0.0;
+                                } else {
+#pragma unroll
+                                    for (int a = 0; a < 5; a++) {
+#pragma unroll
+                                        for (int b = a; b < 5; b++) v[up5(a, b)] = fma(A[a], A[b], v[up5(a, b)]);
+                                        v[15 + a] = fma(A[a], h, v[15 + a]);
+                                    }
+                                    v[20] = fma(h, h, v[20]);
+                                }
+                            }
+                        }
+                        uni = __all_sync(0xffffffffu, uni && same);
+                    }
+                    s2c[c] = s2;
+                }
+                if (!kDirect && uni) reduce_vals(v, lane, w.T[c]);
+            }
+            const double s2min = warp_min(__longlong_as_double(s2m));
             if (lane == 0) {
                 w.s2c[0] = s2c[0];
                 w.s2c[1] = s2c[1];
@@ -383,37 +405,22 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_first(Settings st, cons
                 double corr[kSumVals];
 #pragma unroll
                 for (int k = 0; k < kSumVals; k++) corr[k] = 0.0;
-                int m = 0, listed = 0;
-                const int nout0 = nout;
+                int m = 0, listed = 0, sub_n = 0;
+                double sub_hh = 0.0;
                 const double rx = vs > 0.0 ? 1.0 / (sqrt(s2c[c]) * vs) : 0.0;
-                const float ivs = (float)(1.0 / vs);
                 auto flush = [&](int k) {
-                    subtract_rows(scr, list, k, lane, true, nullptr, rx, st.weight_fn, last, corr, nout);
+                    weigh_rows<true>(scr, list, k, lane, true, nullptr, rx, st.weight_fn, last, corr, nout, sub_n, sub_hh);
                     listed += k;
                 };
-                if (st.robust && rx > 0.0)
+                if (st.robust)
                     for (int j0 = lo; j0 < hi; j0 += kWarp) {
                         const int j = j0 + lane;
-                        // x of the key, to 2^-22 relative: at or above 2 within that, or not finite
-                        const bool cand = j < hi && !(fabsf(trunc_f32(dkey_inv(keys[j])) * ivs) < 1.99999f);
-                        if (last && j < hi && !cand) scr[(size_t)j * kScr + 6] = 1.0;
-                        append_rows(cand, j, list, m, lane, flush);
+                        append_rows(j < hi && beyond(j), j, list, m, lane, flush);
                     }
-                else if (last)
-                    for (int j = lo + lane; j < hi; j += kWarp) scr[(size_t)j * kScr + 6] = 1.0;
                 __syncwarp();
                 if (m > 0) flush(m);
                 __syncwarp();
-                const bool all = 3 * listed > hi - lo;
-                if (all) {
-                    double sums[kSumVals];   // (in memory: corr stays in registers)
-                    int cnt = 0;
-                    direct_rows(scr, lo, hi, list, lane, true, nullptr, rx, st.weight_fn, last, sums, cnt);
-                    nout = nout0 + cnt;
-#pragma unroll
-                    for (int k = 0; k < kSumVals; k++) corr[k] = sums[k];
-                }
-                if (lane == 0) w.all[c] = all;
+                if (lane == 0) w.all[c] = 0;
                 if (listed) reduce_vals(corr, lane, w.C[c]);
                 else if (lane < kSumVals) w.C[c][lane] = 0.0;
             }
@@ -425,7 +432,11 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_first(Settings st, cons
 
 // Class sums of a later round: w = wfun((h - A d) / sqrt(sigma_c^2 + y)) with the previous round's
 // (d, y).  z = (h - A d) isd in FP32 from truncated values: its error is below
-// 2^-19 isd (|h| + sum |A_k d_k|) (truncation 2^-23 of each factor, ten roundings of 2^-24).
+// 2^-19 isd (|h| + sum |A_k d_k|) (truncation 2^-23 of each factor, ten roundings of 2^-24).  Rows that
+// the unit-weight sums do not hold are added with their weights, the others that may exceed 2 have
+// (1 - w) taken off.  Their |h| is below two robust scales, but the rounds may still reject many of
+// them: where more than a third of a class's rows or a quarter of its sum of h^2 is taken off, the class is
+// summed over all its rows instead, so that the difference loses less than a bit.
 __global__ void __launch_bounds__(32 * kPassWarps) k_src_round(Settings st, int last, const int64_t* __restrict__ src_off,
                                                                const int32_t* __restrict__ src_nal,
                                                                const int32_t* __restrict__ src_order, int32_t n_src,
@@ -455,10 +466,11 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_round(Settings st, int 
                 double corr[kSumVals];
 #pragma unroll
                 for (int k = 0; k < kSumVals; k++) corr[k] = 0.0;
-                int m = 0, listed = 0;
+                int m = 0, listed = 0, sub_n = 0;
+                double sub_hh = 0.0;
                 const int nout0 = nout;
                 auto flush = [&](int k) {
-                    subtract_rows(scr, list, k, lane, false, d, isd, st.weight_fn, last, corr, nout);
+                    weigh_rows<false>(scr, list, k, lane, false, d, isd, st.weight_fn, last, corr, nout, sub_n, sub_hh);
                     listed += k;
                 };
                 auto screen = [&](double h, const double A[5]) {
@@ -475,25 +487,28 @@ __global__ void __launch_bounds__(32 * kPassWarps) k_src_round(Settings st, int 
                 for (int j0 = lo; j0 < hi; j0 += 2 * kWarp) {   // two rows in flight per lane
                     const int ja = j0 + lane, jb = ja + kWarp;
                     double ha = 0.0, hb = 0.0, Aa[5], Ab[5];
-                    if (ja < hi) row_load(scr + (size_t)ja * kScr, ha, Aa);
-                    if (jb < hi) row_load(scr + (size_t)jb * kScr, hb, Ab);
-                    const bool ca = ja < hi && screen(ha, Aa);
-                    const bool cb = jb < hi && screen(hb, Ab);
-                    if (last) {
-                        if (ja < hi && !ca) scr[(size_t)ja * kScr + 6] = 1.0;
-                        if (jb < hi && !cb) scr[(size_t)jb * kScr + 6] = 1.0;
+                    long long wa = 0, wb = 0;   // weight slots: 1, or 0 for a row beyond
+                    if (ja < hi) {
+                        row_load(scr + (size_t)ja * kScr, ha, Aa);
+                        wa = __double_as_longlong(scr[(size_t)ja * kScr + 6]);
                     }
+                    if (jb < hi) {
+                        row_load(scr + (size_t)jb * kScr, hb, Ab);
+                        wb = __double_as_longlong(scr[(size_t)jb * kScr + 6]);
+                    }
+                    const bool ca = ja < hi && (wa == 0 || screen(ha, Aa));
+                    const bool cb = jb < hi && (wb == 0 || screen(hb, Ab));
                     append_rows(ca, ja, list, m, lane, flush);
                     append_rows(cb, jb, list, m, lane, flush);
                 }
                 __syncwarp();
                 if (m > 0) flush(m);
                 __syncwarp();
-                const bool all = 3 * listed > hi - lo;
+                const bool all = 3 * warp_sum_int(sub_n) > hi - lo || 4.0 * warp_sum(sub_hh) > w.T[c][20];
                 if (all) {
                     double sums[kSumVals];   // (in memory: corr stays in registers)
                     int cnt = 0;
-                    direct_rows(scr, lo, hi, list, lane, false, d, isd, st.weight_fn, last, sums, cnt);
+                    direct_rows(scr, lo, hi, list, lane, d, isd, st.weight_fn, last, sums, cnt);
                     nout = nout0 + cnt;
 #pragma unroll
                     for (int k = 0; k < kSumVals; k++) corr[k] = sums[k];
@@ -694,7 +709,7 @@ __global__ void __launch_bounds__(128) k_src_solve5(Settings st, int last, const
     ClassSums S;
     HalfSums H;
     const int all[2] = {w.all[0], w.all[1]};
-    auto sum_of = [&](int c, int k) { return (c ? all[1] : all[0]) ? w.C[c][k] : w.T[c][k] - w.C[c][k]; };
+    auto sum_of = [&](int c, int k) { return (c ? all[1] : all[0]) ? w.C[c][k] : w.T[c][k] + w.C[c][k]; };
     if (kPair) {
         for (int c = 0; c < 2; c++)
             for (int k = 0; k < 10; k++) H.E[c][k] = sum_of(c, 10 * h + k);
@@ -1039,7 +1054,7 @@ void launch_obs_pass(const DevGeo& G, const AttNoise& an, const int64_t* t_ns, c
 }
 
 // The inner iteration of the S block on the scratch rows of the observation pass.  corrections:
-// rounds subtract (1 - w) terms from unit-weight sums; else each round sums every row.
+// rounds correct unit-weight sums by the rows beyond |z| = 2; else each round sums every row.
 void launch_source_solve(const Settings& st, bool corrections, const int64_t* src_off, const int32_t* src_nal,
                          const int32_t* src_order, int32_t n_src, const SrcOutPtrs& out, ObsRec* rec, double* scratch,
                          const uint64_t* skey, SrcWork* work, const Shapes& sh, cudaStream_t stream) {
