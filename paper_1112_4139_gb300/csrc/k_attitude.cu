@@ -439,10 +439,12 @@ __global__ void __launch_bounds__(32 * kMomWarps) k_att_moments(DevGeo G, MomSca
     const int nwarps = gridDim.x * kMomWarps;
     for (int iv = blockIdx.x * kMomWarps + wib; iv < n_iv; iv += nwarps) {
         const int64_t beg = ivl_off[iv], end = ivl_off[iv + 1];
+        // short intervals and the ends are not read for their scales first
+        const bool sized = iv >= 2 && iv < n_iv - 2 && end - beg >= kMomMin;
         // the largest magnitudes of W, W R and g (bits of the high words)
         uint32_t mw = 0, mr = 0, mg = 0, t_lo = 0xffffffffu, t_hi = 0;
         const int64_t tau = G.knot0_ns + (int64_t)iv * G.knot_dt_ns;
-        for (int64_t j = beg + lane; j < end; j += kWarp) {
+        for (int64_t j = sized ? beg + lane : end; j < end; j += kWarp) {
             const uint32_t o = perm_t[j];
             const ObsRec& r = rec[o];
             const double W = w_att ? w_att[o] : r.W;
@@ -466,7 +468,7 @@ __global__ void __launch_bounds__(32 * kMomWarps) k_att_moments(DevGeo G, MomSca
         const int EW = (int)((mw + 0x5000) >> 20) - 1022, ER = (int)((mr + 0x5000) >> 20) - 1022, Eg = (int)(mg >> 20) - 1022;
         // scales in range: finite, and no power of two below under- or overflows (all residuals may be
         // zero); u^6 and v^6, the outer B-splines' squares, reach 2^-9: their 63 bits hold 54 of a column
-        const bool ok = iv >= 2 && iv < n_iv - 2 && end - beg >= kMomMin && abs(EW) < 250 && ER < 250 && abs(Eg) < 250 &&
+        const bool ok = sized && abs(EW) < 250 && ER < 250 && abs(Eg) < 250 &&
                         fmaxf(lu, lv) < 1.5f;
         if (ok)
             interval_moments(G, ms, lambda2, perm_t, beg, end, iv, rec, w_att, att, EW, max(ER, -250), Eg, lu, lv, lane,
