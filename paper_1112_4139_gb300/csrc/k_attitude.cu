@@ -147,28 +147,29 @@ __global__ void __launch_bounds__(128) k_att_accum(DevGeo G, double lambda2, int
 // the right-hand side likewise with W R g (the cubics raised to degree 6), and the norm term, a
 // form with the interval's coefficients alone, needs sum_o W u^k v^(12-k), k = 0 .. 12.  Rows
 // W g g' (10), W R g (4), W v^6 and W u^6 by columns u^k v^(6-k): one 16 x 7 contraction over the
-// interval's observations, and an expansion without cancellation (rms error over the sum of the
-// terms' magnitudes: powers of 2 u - 1 2.0e-16, the products' sums 1.8e-16, these
-// forms less).
+// interval's observations, and an expansion without cancellation.  Root mean square error of an entry
+// relative to its place, against the products' sums: 0.54 of theirs with 24 observations in the interval, 0.36 with
+// 54, 0.25 with 156 (the worst entry 0.81, 0.62, 0.44).
 //
 // It runs on mma.sync (a 128-row tcgen05 tile would hold one interval of 16 rows): every row value is
-// a 55-bit and every column value a 54-bit fraction of its largest magnitude in the interval, cut into
-// eight signed 7-bit digits kept as FP16 integers, and the products of the digit pairs i + j >= 6 are
-// accumulated in FP32 by their weight 2^(7 (i + j)): 8 pairs x 512 observations x 2^12 are
-// at most 2^24, so every sum is exact, and the pairs left out are below 2^-58 of the largest term
+// a 62-bit and every column value a 61-bit fraction of its largest magnitude in the interval, cut into
+// nine signed 7-bit digits kept as FP16 integers, and the products of the digit pairs i + j >= 7 are
+// accumulated in FP32 by their weight 2^(7 (i + j)): 9 pairs x 448 observations x 2^12 are
+// below 2^24, so every sum is exact, and the pairs left out are about 2^-69 of the largest term
 // (FP64 rounds each product at 2^-53).  Products W g g', the forms and conversions are 64-bit
 // integer arithmetic.
-// Bound: integer and shared-memory issue (about 28 instructions per observation and warp of 32)
+// Bound by reading: integer and shared-memory issue
 // and 68 FP64 instructions per interval for the expansion, where the FP64 form takes 116 FMAs and
 // about 95 more FP64 instructions per observation (2 per clock and SM).
-// 24.7M observations in 157,786 intervals: 9.93 -> 2.95 ms; 7.1M in 131,490: 3.06 -> 1.51 ms.
-// Intervals next to the multiple end knots (two at each end), short ones and those that the
-// observations do not cover sum the products one by one.
+// Attitude update, the products' sums against this: 24.7M observations in 157,786 intervals 11.6 -> 5.3 ms, 7.1M in
+// 131,490 4.62 -> 3.81 (a fifth of these intervals of 54 takes the products), 14M in 131,490 7.3 -> 4.4.
+// Intervals next to the multiple end knots (two at each end), short ones, those that the
+// observations do not cover and those with a sum far below its digits' scale sum the products one by one.
 constexpr int kMomWarps = 4;
 constexpr int kMomStride = 40;    // 64-bit values per row of the staged chunk (rows 64 B apart mod 128 B)
-constexpr int kMomFlush = 512;    // observations per exact accumulation
+constexpr int kMomFlush = 448;    // observations per exact accumulation
 constexpr int kMomMin = 24;       // shorter intervals: the sums of the products themselves
-constexpr uint64_t kDigitBias = 0x0081020408102040ull;   // 64 in every 7-bit digit
+constexpr uint64_t kDigitBias = 0x4081020408102040ull;   // 64 in each of nine 7-bit digits
 
 struct MomScale {                  // u with 63 fractional bits: 2^shift (t - tau) inv 2^-64, times 2
     uint64_t inv;
@@ -188,29 +189,32 @@ __device__ __forceinline__ long long to_fixed(double v, int E) {
 // products of 62-bit fractions and of unsigned 63-bit ones, what is cut off at half its range
 __device__ __forceinline__ long long mulq(long long a, long long b) { return (long long)((unsigned long long)__mul64hi(a, b) << 2) | 2; }
 __device__ __forceinline__ uint64_t mulu(uint64_t a, uint64_t b) { return (__umul64hi(a, b) << 1) | 1; }
+__device__ __forceinline__ long long shifted(uint64_t x, int n) { return (long long)(n >= 0 ? x << n : x >> -n); }
 __device__ __forceinline__ double pow2(int n) { return __longlong_as_double((long long)(1023 + n) << 52); }
 
-// fixed-point value, rounded to multiples of 2^kShift -> its digits' bit fields, 28 bits per word;
-// |q| 2^-kShift <= 0.992 2^55
-template <int kShift>
-__device__ __forceinline__ uint2 digit_words(long long q) {
-    constexpr uint64_t kAdd = (kDigitBias << kShift) + (kShift ? 1ull << (kShift > 0 ? kShift - 1 : 0) : 0ull);
-    const uint64_t u = ((uint64_t)q + kAdd) >> kShift;
-    return make_uint2((uint32_t)u & 0xfffffffu, (uint32_t)(u >> 28) & 0xfffffffu);
+// fixed-point value -> its digits' bit fields; |q| <= 0.992 2^62
+__device__ __forceinline__ uint2 digit_bits(long long q) {
+    const uint64_t u = (uint64_t)q + kDigitBias;
+    return make_uint2((uint32_t)u, (uint32_t)(u >> 32));
 }
-// the four digits of a 28-bit word of two observations, as FP16 pairs
-__device__ __forceinline__ void digits4(uint32_t a, uint32_t b, uint32_t out[4]) {
-    const uint32_t c0 = __byte_perm(a, b, 0x5410), c1 = __byte_perm(a >> 14, b >> 14, 0x5410);
+// the nine digits of a value of two observations (low and high words of each), as FP16 pairs
+__device__ __forceinline__ uint32_t digit_half(uint32_t w) {   // digits in bits 0-6 and 16-22
+    const uint32_t h = (w & 0x007f007fu) | 0x64006400u;        // 1024 + digit + 64
     const __half2 off = __halves2half2(__ushort_as_half(0xe440), __ushort_as_half(0xe440));   // -1088
-    auto half_of = [&](uint32_t w) -> uint32_t {
-        const uint32_t h = (w & 0x007f007fu) | 0x64006400u;    // 1024 + digit + 64
-        const __half2 r = __hadd2(*reinterpret_cast<const __half2*>(&h), off);
-        return *reinterpret_cast<const uint32_t*>(&r);
-    };
-    out[0] = half_of(c0);
-    out[1] = half_of(c0 >> 7);
-    out[2] = half_of(c1);
-    out[3] = half_of(c1 >> 7);
+    const __half2 r = __hadd2(*reinterpret_cast<const __half2*>(&h), off);
+    return *reinterpret_cast<const uint32_t*>(&r);
+}
+__device__ __forceinline__ void digits4(uint32_t a, uint32_t b, uint32_t out[4]) {   // of bits 0 .. 27
+    const uint32_t c0 = __byte_perm(a, b, 0x5410), c1 = __byte_perm(a >> 14, b >> 14, 0x5410);
+    out[0] = digit_half(c0);
+    out[1] = digit_half(c0 >> 7);
+    out[2] = digit_half(c1);
+    out[3] = digit_half(c1 >> 7);
+}
+__device__ __forceinline__ void digits9(const uint4 v, uint32_t out[9]) {
+    digits4(v.x, v.z, out);
+    digits4(__funnelshift_l(v.x, v.y, 4), __funnelshift_l(v.z, v.w, 4), out + 4);
+    out[8] = digit_half(__byte_perm(v.y >> 24, v.w >> 24, 0x5410));
 }
 __device__ __forceinline__ void mma_f16(float c[4], const uint32_t a[4], uint32_t b0, uint32_t b1) {
     asm volatile(
@@ -222,27 +226,52 @@ __device__ __forceinline__ void mma_f16(float c[4], const uint32_t a[4], uint32_
 // the four B-splines' coefficients (over 6) of u^k v^(3-k), and the columns' scales 2^n at any u
 __device__ constexpr int kSplineNum[4][4] = {{1, 0, 0, 0}, {4, 12, 6, 1}, {1, 6, 12, 4}, {0, 0, 0, 1}};
 __device__ constexpr int kColShift[7] = {0, 3, 5, 5, 5, 3, 0};
+// components c <= e of row tri4(c, e) of W g g'
+__device__ __forceinline__ int row_first(int row) { return row < 4 ? 0 : row < 7 ? 1 : row < 9 ? 2 : 3; }
+__device__ __forceinline__ int row_second(int row) { return row < 4 ? row : row < 7 ? row - 3 : row < 9 ? row - 5 : 3; }
 
-// One interval's products from its moments, by one warp, into red[kAccFP64].
-__device__ __forceinline__ void interval_moments(const DevGeo& G, MomScale ms, double lambda2,
+// One interval's products from its moments, by one warp, into red[kAccFP64].  False (nothing written)
+// if a sum on the diagonal is small beside the scale of its digits.
+//
+// Every row and column has a scale of its own (W, W R and each component of g by their largest
+// values).  An observation's term is off by about 2^-63 of the row's largest value times the column's (two
+// products cut at 2^-62), by 2^amp of that for a column that is shifted up by amp bits more than over a
+// whole interval, and the sum by sqrt(n) of it.  The products' sums are off by 0.17 2^-52 sqrt(n) of a sum on the
+// diagonal, and by about 0.28 2^-52 of its place in the matrix (the root of its two diagonal sums) where signs
+// differ.  A diagonal sum of at least 2^(amp - 9) sqrt(n) of its two scales' product keeps the digits
+// below 0.25 2^-52 of either; a smaller one (large weights that meet small components or lie at the other end
+// of the interval) sends the interval to the products' sums.
+__device__ __forceinline__ bool interval_moments(const DevGeo& G, MomScale ms, double lambda2,
                                                  const uint32_t* __restrict__ perm_t, int64_t beg, int64_t end, int iv,
                                                  const ObsRec* __restrict__ rec, const double* __restrict__ w_att,
-                                                 const double* __restrict__ att, int EW, int ER, int Eg, float lu,
+                                                 const double* __restrict__ att, int EW, int ER, const int (&Eg)[4], float lu,
                                                  float lv, int lane, uint2* st, const double (*cbb)[8], const double (*cb)[8], double* wk,
                                                  double* red) {
     const int g = lane >> 2, q = lane & 3;
     const double l4 = 4.0 * lambda2;
-    // every column to its largest value in the interval: u^k v^(6-k) 2^sh[k] < 1
-    int sh[7];
+    // every column to its largest value in the interval: u^k v^(6-k) 2^sh[k] < 1.  They are formed from
+    // ua = u 2^a, vb = v 2^b and 4 u v, with cs[k] bits up to 61 fractional ones
+    int sh[7], cs[7];
+    const int a = (int)lu > 0, b = (int)lv > 0;
 #pragma unroll
-    for (int k = 0; k < 7; k++) sh[k] = max(kColShift[k], (int)floorf((float)k * lu + (float)(6 - k) * lv - 1e-4f));
+    for (int k = 0; k < 7; k++) {
+        sh[k] = max(kColShift[k], (int)floorf((float)k * lu + (float)(6 - k) * lv - 1e-4f));
+        const int m = k < 6 - k ? k : 6 - k;   // (4 u v)^m
+        cs[k] = sh[k] - 2 - 2 * m - (k > 3 ? (2 * k - 6) * a : (6 - 2 * k) * b);
+    }
     // moments of this lane: rows g and g + 8, columns 2 q and 2 q + 1
     double mom[4] = {0, 0, 0, 0};
+    auto eg = [&](int c) { return c == 0 ? Eg[0] : c == 1 ? Eg[1] : c == 2 ? Eg[2] : Eg[3]; };
+    auto unit = [&](int e) {   // power of two of mom[e]'s scale
+        const int row = g + 8 * (e >> 1);
+        const int ce = e & 1 ? (q == 0 ? sh[1] : q == 1 ? sh[3] : sh[5]) : (q == 0 ? sh[0] : q == 1 ? sh[2] : q == 2 ? sh[4] : sh[6]);
+        return (row < 10 ? EW + eg(row_first(row)) + eg(row_second(row)) : (row < 14 ? ER + eg(row - 10) : EW)) - ce;
+    };
     const int64_t tau = G.knot0_ns + (int64_t)iv * G.knot_dt_ns;
     for (int64_t f0 = beg; f0 < end; f0 += kMomFlush) {
-        float acc[9][4];
+        float acc[10][4];
 #pragma unroll
-        for (int s = 0; s < 9; s++)
+        for (int s = 0; s < 10; s++)
 #pragma unroll
             for (int e = 0; e < 4; e++) acc[s][e] = 0.0f;
         const int64_t f1 = end < f0 + kMomFlush ? end : f0 + kMomFlush;
@@ -254,28 +283,29 @@ __device__ __forceinline__ void interval_moments(const DevGeo& G, MomScale ms, d
                 const ObsRec& r = rec[o];
                 const double W = w_att ? w_att[o] : r.W;
                 const uint64_t u = __umul64hi((uint64_t)(r.t_ns - tau) << ms.shift, ms.inv) << 1, v = (1ull << 63) - u;
-                const uint64_t u2 = mulu(u, u), v2 = mulu(v, v), u3 = mulu(u2, u), v3 = mulu(v2, v);
-                const uint64_t uv2 = mulu(u, v2), u2v = mulu(u2, v), u6 = mulu(u3, u3), v6 = mulu(v3, v3);
+                const uint64_t ua = u << a, vb = v << b, p = mulu(ua, vb) << (2 - a - b), p2 = mulu(p, p);
+                const uint64_t u2 = mulu(ua, ua), v2 = mulu(vb, vb), u4 = mulu(u2, u2), v4 = mulu(v2, v2);
+                const uint64_t u6 = mulu(u4, u2), v6 = mulu(v4, v2);
                 const long long Wq = to_fixed(W, EW), WR = to_fixed(W * r.R, ER);
                 long long gq[4];
 #pragma unroll
-                for (int c = 0; c < 4; c++) gq[c] = to_fixed(r.g[c], Eg);
+                for (int c = 0; c < 4; c++) gq[c] = to_fixed(r.g[c], Eg[c]);
 #pragma unroll
                 for (int c = 0; c < 4; c++) {
                     const long long Wg = mulq(Wq, gq[c]);
 #pragma unroll
-                    for (int e = c; e < 4; e++) X[tri4(c, e)] = __mul64hi(Wg, gq[e]);
-                    X[10 + c] = __mul64hi(WR, gq[c]);
+                    for (int e = c; e < 4; e++) X[tri4(c, e)] = mulq(Wg, gq[e]);
+                    X[10 + c] = WR ? mulq(WR, gq[c]) : 0;   // zero residuals give zero sums
                 }
-                X[14] = __mul64hi(Wq, (long long)(v6 >> 1));
-                X[15] = __mul64hi(Wq, (long long)(u6 >> 1));
-                C[0] = (v6 << sh[0]) >> 1;
-                C[1] = mulu(uv2, v3) << (sh[1] - 1);
-                C[2] = mulu(uv2, uv2) << (sh[2] - 1);
-                C[3] = mulu(u3, v3) << (sh[3] - 1);
-                C[4] = mulu(u2v, u2v) << (sh[4] - 1);
-                C[5] = mulu(u2v, u3) << (sh[5] - 1);
-                C[6] = (u6 << sh[6]) >> 1;
+                X[14] = mulq(Wq, (long long)(v6 >> (6 * b + 1)));
+                X[15] = mulq(Wq, (long long)(u6 >> (6 * a + 1)));
+                C[0] = shifted(v6, cs[0]);
+                C[1] = shifted(mulu(p, v4), cs[1]);
+                C[2] = shifted(mulu(p2, v2), cs[2]);
+                C[3] = shifted(mulu(p2, p), cs[3]);
+                C[4] = shifted(mulu(p2, u2), cs[4]);
+                C[5] = shifted(mulu(p, u4), cs[5]);
+                C[6] = shifted(u6, cs[6]);
             } else {
 #pragma unroll
                 for (int k = 0; k < 16; k++) X[k] = 0;
@@ -284,58 +314,57 @@ __device__ __forceinline__ void interval_moments(const DevGeo& G, MomScale ms, d
             }
             __syncwarp();
 #pragma unroll
-            for (int k = 0; k < 16; k++) st[k * kMomStride + lane] = digit_words<5>(X[k]);
+            for (int k = 0; k < 16; k++) st[k * kMomStride + lane] = digit_bits(X[k]);
 #pragma unroll
-            for (int k = 0; k < 7; k++) st[(16 + k) * kMomStride + lane] = digit_words<8>(C[k]);
-            st[23 * kMomStride + lane] = digit_words<0>(0);
+            for (int k = 0; k < 7; k++) st[(16 + k) * kMomStride + lane] = digit_bits(C[k]);
+            st[23 * kMomStride + lane] = digit_bits(0);
             __syncwarp();
 #pragma unroll
             for (int h = 0; h < 2; h++) {
                 const int k0 = 16 * h + 2 * q;
-                uint32_t A[8][4], Bd[8][2];
+                uint32_t A[9][4], Bd[9][2];
 #pragma unroll
                 for (int e = 0; e < 4; e++) {   // rows g, g + 8 at k0; then at k0 + 8
-                    const uint4 v = *reinterpret_cast<const uint4*>(&st[(g + 8 * (e & 1)) * kMomStride + k0 + 8 * (e >> 1)]);
-                    uint32_t d[4];
-                    digits4(v.x, v.z, d);
+                    uint32_t d[9];
+                    digits9(*reinterpret_cast<const uint4*>(&st[(g + 8 * (e & 1)) * kMomStride + k0 + 8 * (e >> 1)]), d);
 #pragma unroll
-                    for (int t = 0; t < 4; t++) A[t][e] = d[t];
-                    digits4(v.y, v.w, d);
-#pragma unroll
-                    for (int t = 0; t < 4; t++) A[4 + t][e] = d[t];
+                    for (int t = 0; t < 9; t++) A[t][e] = d[t];
                 }
 #pragma unroll
                 for (int e = 0; e < 2; e++) {
-                    const uint4 v = *reinterpret_cast<const uint4*>(&st[(16 + g) * kMomStride + k0 + 8 * e]);
-                    uint32_t d[4];
-                    digits4(v.x, v.z, d);
+                    uint32_t d[9];
+                    digits9(*reinterpret_cast<const uint4*>(&st[(16 + g) * kMomStride + k0 + 8 * e]), d);
 #pragma unroll
-                    for (int t = 0; t < 4; t++) Bd[t][e] = d[t];
-                    digits4(v.y, v.w, d);
-#pragma unroll
-                    for (int t = 0; t < 4; t++) Bd[4 + t][e] = d[t];
+                    for (int t = 0; t < 9; t++) Bd[t][e] = d[t];
                 }
 #pragma unroll
-                for (int i = 0; i < 8; i++)
+                for (int i = 0; i < 9; i++)
 #pragma unroll
-                    for (int jd = 0; jd < 8; jd++)
-                        if (i + jd >= 6) mma_f16(acc[i + jd - 6], A[i], Bd[jd][0], Bd[jd][1]);
+                    for (int jd = 0; jd < 9; jd++)
+                        if (i + jd >= 7) mma_f16(acc[i + jd - 7], A[i], Bd[jd][0], Bd[jd][1]);
             }
         }
-        // the exact sums by weight: H 2^63 + L 2^42, in units of 2^-109 of the scales
+        // the exact sums by weight: H 2^84 + L 2^49, in units of 2^-123 of the scales
 #pragma unroll
         for (int e = 0; e < 4; e++) {
             long long H = 0, L = 0;
 #pragma unroll
-            for (int s = 8; s >= 3; s--) H = (H << 7) + (long long)__float2int_rn(acc[s][e]);
+            for (int s = 9; s >= 5; s--) H = (H << 7) + (long long)__float2int_rn(acc[s][e]);
 #pragma unroll
-            for (int s = 2; s >= 0; s--) L = (L << 7) + (long long)__float2int_rn(acc[s][e]);
-            const int row = g + 8 * (e >> 1);
-            const int ce = e & 1 ? (q == 0 ? sh[1] : q == 1 ? sh[3] : sh[5]) : (q == 0 ? sh[0] : q == 1 ? sh[2] : q == 2 ? sh[4] : sh[6]);
-            const int E = (row < 10 ? EW + 2 * Eg : (row < 14 ? ER + Eg : EW)) - ce;
-            mom[e] += fma((double)H, pow2(E - 46), (double)L * pow2(E - 67));
+            for (int s = 4; s >= 0; s--) L = (L << 7) + (long long)__float2int_rn(acc[s][e]);
+            const int E = unit(e);
+            mom[e] += fma((double)H, pow2(E - 39), (double)L * pow2(E - 74));
         }
     }
+    bool good = true;
+    const double root_n = (double)sqrtf((float)(end - beg));
+#pragma unroll
+    for (int e = 0; e < 4; e++) {   // rows 0, 4, 7 and 9, columns 0 .. 6
+        const int row = g + 8 * (e >> 1);
+        const int amp = e & 1 ? (q == 0 ? cs[1] + 1 : q == 1 ? cs[3] + 3 : cs[5] + 1) : (q == 0 ? cs[0] + 2 : q == 1 ? cs[2] + 1 : q == 2 ? cs[4] + 1 : cs[6] + 2);
+        if ((row == 0 || row == 4 || row == 7 || row == 9) && 2 * q + (e & 1) < 7) good = good && mom[e] >= root_n * pow2(unit(e) + max(amp, 0) - 9);
+    }
+    if (!__all_sync(0xffffffffu, good)) return false;
     __syncwarp();
     // wk: moments [16][8] at 0, coefficients of s [4][4] at 128, of s s' [10][7] at 144, the moments
     // with the norm term [10][8] at 216
@@ -402,9 +431,10 @@ __device__ __forceinline__ void interval_moments(const DevGeo& G, MomScale ms, d
         }
     }
     __syncwarp();
+    return true;
 }
 
-__global__ void __launch_bounds__(32 * kMomWarps) k_att_moments(DevGeo G, MomScale ms, double lambda2,
+__global__ void __launch_bounds__(32 * kMomWarps, 3) k_att_moments(DevGeo G, MomScale ms, double lambda2,
                                                                 const uint32_t* __restrict__ perm_t,
                                                                 const int64_t* __restrict__ ivl_off, int n_iv,
                                                                 const ObsRec* __restrict__ rec,
@@ -439,42 +469,51 @@ __global__ void __launch_bounds__(32 * kMomWarps) k_att_moments(DevGeo G, MomSca
     const int nwarps = gridDim.x * kMomWarps;
     for (int iv = blockIdx.x * kMomWarps + wib; iv < n_iv; iv += nwarps) {
         const int64_t beg = ivl_off[iv], end = ivl_off[iv + 1];
-        // short intervals and the ends are not read for their scales first
-        const bool sized = iv >= 2 && iv < n_iv - 2 && end - beg >= kMomMin;
-        // the largest magnitudes of W, W R and g (bits of the high words)
-        uint32_t mw = 0, mr = 0, mg = 0, t_lo = 0xffffffffu, t_hi = 0;
-        const int64_t tau = G.knot0_ns + (int64_t)iv * G.knot_dt_ns;
-        for (int64_t j = sized ? beg + lane : end; j < end; j += kWarp) {
-            const uint32_t o = perm_t[j];
-            const ObsRec& r = rec[o];
-            const double W = w_att ? w_att[o] : r.W;
-            const double2 ga = *reinterpret_cast<const double2*>(r.g), gb = *reinterpret_cast<const double2*>(r.g + 2);
-            const uint32_t tq = (uint32_t)((r.t_ns - tau) >> ms.tshift);
-            t_lo = min(t_lo, tq);
-            t_hi = max(t_hi, tq);
-            mw = max(mw, (uint32_t)__double2hiint(W) & 0x7fffffffu);
-            mr = max(mr, (uint32_t)__double2hiint(W * r.R) & 0x7fffffffu);
-            mg = max(max(mg, (uint32_t)__double2hiint(ga.x) & 0x7fffffffu), (uint32_t)__double2hiint(ga.y) & 0x7fffffffu);
-            mg = max(max(mg, (uint32_t)__double2hiint(gb.x) & 0x7fffffffu), (uint32_t)__double2hiint(gb.y) & 0x7fffffffu);
+        bool done = false;
+        if (iv >= 2 && iv < n_iv - 2 && end - beg >= kMomMin) {
+            // the largest magnitudes of W, W R and g (bits of the high words)
+            uint32_t mw = 0, mr = 0, mg[4] = {0, 0, 0, 0}, t_lo = 0xffffffffu, t_hi = 0;
+            const int64_t tau = G.knot0_ns + (int64_t)iv * G.knot_dt_ns;
+            for (int64_t j = beg + lane; j < end; j += kWarp) {
+                const uint32_t o = perm_t[j];
+                const ObsRec& r = rec[o];
+                const double W = w_att ? w_att[o] : r.W;
+                const double2 ga = *reinterpret_cast<const double2*>(r.g), gb = *reinterpret_cast<const double2*>(r.g + 2);
+                const uint32_t tq = (uint32_t)((r.t_ns - tau) >> ms.tshift);
+                t_lo = min(t_lo, tq);
+                t_hi = max(t_hi, tq);
+                mw = max(mw, (uint32_t)__double2hiint(W) & 0x7fffffffu);
+                mr = max(mr, (uint32_t)__double2hiint(W * r.R) & 0x7fffffffu);
+                mg[0] = max(mg[0], (uint32_t)__double2hiint(ga.x) & 0x7fffffffu);
+                mg[1] = max(mg[1], (uint32_t)__double2hiint(ga.y) & 0x7fffffffu);
+                mg[2] = max(mg[2], (uint32_t)__double2hiint(gb.x) & 0x7fffffffu);
+                mg[3] = max(mg[3], (uint32_t)__double2hiint(gb.y) & 0x7fffffffu);
+            }
+            mw = __reduce_max_sync(0xffffffffu, mw);
+            mr = __reduce_max_sync(0xffffffffu, mr);
+            t_lo = __reduce_min_sync(0xffffffffu, t_lo);
+            t_hi = __reduce_max_sync(0xffffffffu, t_hi);
+            // -log2 of the largest u and v
+            const float lu = -log2f((float)(t_hi + 1) * ms.tinv), lv = -log2f(fmaf(-(float)t_lo, ms.tinv, 1.0f) + 1e-6f);
+            // 2^E above them; W and W R below 0.99 of it, for rows of 55 bits
+            const int EW = (int)((mw + 0x5000) >> 20) - 1022, ER = (int)((mr + 0x5000) >> 20) - 1022;
+            // scales in range: finite, and no power of two below under- or overflows (all residuals may be
+            // zero); u and v each reach beyond 2^-1.5: columns near the outer B-splines' ends keep their bits
+            bool ok = abs(EW) < 250 && ER < 250 && fmaxf(lu, lv) < 1.5f;
+            int Eg[4];
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                Eg[c] = (int)(__reduce_max_sync(0xffffffffu, mg[c]) >> 20) - 1022;
+                ok = ok && abs(Eg[c]) < 250;
+            }
+            if (ok)
+                done = interval_moments(G, ms, lambda2, perm_t, beg, end, iv, rec, w_att, att, EW, max(ER, -250), Eg, lu, lv,
+                                        lane, st, cbb, cb, wk, red);
         }
-        mw = __reduce_max_sync(0xffffffffu, mw);
-        mr = __reduce_max_sync(0xffffffffu, mr);
-        mg = __reduce_max_sync(0xffffffffu, mg);
-        t_lo = __reduce_min_sync(0xffffffffu, t_lo);
-        t_hi = __reduce_max_sync(0xffffffffu, t_hi);
-        // -log2 of the largest u and v
-        const float lu = -log2f((float)(t_hi + 1) * ms.tinv), lv = -log2f(fmaf(-(float)t_lo, ms.tinv, 1.0f) + 1e-6f);
-        // 2^E above them; W and W R below 0.99 of it, for rows of 55 bits
-        const int EW = (int)((mw + 0x5000) >> 20) - 1022, ER = (int)((mr + 0x5000) >> 20) - 1022, Eg = (int)(mg >> 20) - 1022;
-        // scales in range: finite, and no power of two below under- or overflows (all residuals may be
-        // zero); u^6 and v^6, the outer B-splines' squares, reach 2^-9: their 63 bits hold 54 of a column
-        const bool ok = sized && abs(EW) < 250 && ER < 250 && abs(Eg) < 250 &&
-                        fmaxf(lu, lv) < 1.5f;
-        if (ok)
-            interval_moments(G, ms, lambda2, perm_t, beg, end, iv, rec, w_att, att, EW, max(ER, -250), Eg, lu, lv, lane,
-                             st, cbb, cb, wk, red);
-        else
+        if (!done) {
+            __syncwarp();
             interval_direct(G, lambda2, 0, perm_t, beg, end, rec, w_att, att, iv + 3, lane, wk, red);
+        }
 #pragma unroll
         for (int k = 0; k < 5; k++) {
             const int o = lane + 32 * k;
