@@ -32,16 +32,12 @@ WORKLOADS = {
     "small1yr": "10k sources, 1 yr, 1-h knots, 1-day calibration, sigma_AL 100 uas, 1% outliers",
     "uneven5yr": "3M sources, 5 yr, 30-s knots, G ~ U(12, 18) with sigma_AL 50-500 uas, 40-250 transits",
 }
-# kernels launched by one iteration, (with a full FP64 evaluation, with the linearized pass):
-# FP64 form: S (source geometry, observation pass, first sums, 5 rounds of 5x5 algebra, 4 rounds
-# of sums, final pass, per-observation path, stats in two stages, update-history push) = 17, A
-# (accumulate, assemble, solve, apply, rank-defect sum), C
-# (accumulate, project, rank-defect sum), frame (normals, solve, apply sources, apply
-# attitude) = 29.  Mixed form: the S pass is source geometry + full evaluation, or the one
-# linearized-correction kernel; the S solves are scale/round-0 sums, 5 rounds of 5x5 algebra,
-# 4 rounds of sums, final pass, per-observation path, stats (two), history push = 15 (default
-# 4 reweighting rounds); A, C and frame as above.
-KERNELS_PER_STEP = {"fp64": (29, 29), "mixed": (2 + 15 + 12, 1 + 15 + 12)}
+# kernels launched by one iteration besides the per-source solves, whose number the library gives,
+# (with a full FP64 evaluation, with the linearized pass): S (source geometry and observation pass, or
+# the one linearized-correction kernel of the mixed form; stats in two stages, update-history push),
+# A (accumulate, assemble, solve, apply, rank-defect sum), C (accumulate, project, rank-defect sum), frame
+# (normals, solve, apply sources, apply attitude)
+KERNELS_PER_STEP = {"fp64": (2 + 3 + 12, 2 + 3 + 12), "mixed": (2 + 3 + 12, 1 + 3 + 12)}
 # with the excess attitude noise on: x values, selection in short and in longer buckets, attitude weights
 KERNELS_ATTNOISE = 4
 FALLBACK_HBM_GBS = 6800.0
@@ -54,12 +50,9 @@ MIX_PASS_BYTES = 8 + 16 + 4 + 8 + 8
 TRAFFIC_PER_OBS = {"fp64_s_block": None, "mixed_correct": 47.6}
 
 
-def kernels_per_step(form, ds):
-    """Kernels of an iteration with and without the full evaluation (FP64 form: sets below the lines of the
-    direct class sums take one pass of sums more)."""
-    full, lin = KERNELS_PER_STEP[form]
-    large = ds.n_obs >= 23_000_000 and ds.n_obs >= 512 * ds.n_src and ds.n_obs >= 100 * (ds.n_coef - 3)
-    return (full, lin) if form != "fp64" or large else (full + 1, lin + 1)
+def kernels_per_step(form, solves):
+    """Kernels of an iteration with and without the full evaluation, `solves` of them per-source solves."""
+    return tuple(k + solves for k in KERNELS_PER_STEP[form])
 
 
 def parse():
@@ -435,11 +428,12 @@ def time_form(agis, ds, stream, cfg, steps, warmup, local, dist, tune_iters=0, a
     ms = ev0.elapsed_time(ev1) / steps
     if dist is not None:
         ms = max_over_ranks(ms, dist)
+    solves = g.source_kernels()
     g.close()
     full = [it for it in its if it["s"]["full_eval"]]
     lin = [it for it in its if not it["s"]["full_eval"]]
     med = lambda xs: float(np.median(xs)) if xs else None
-    return {"ms": ms, "t_init": t_init, "clocks": clocks, "n_full_eval": len(full), "tuning": tuning,
+    return {"ms": ms, "t_init": t_init, "clocks": clocks, "n_full_eval": len(full), "tuning": tuning, "solves": solves,
             "s_ms": med([it["s"]["elapsed_ms"] for it in its]), "a_ms": med([it["a"]["elapsed_ms"] for it in its]),
             "c_ms": med([it["c"]["elapsed_ms"] for it in its]),
             "pass_full_ms": med([it["s"]["pass_ms"] for it in full]),
@@ -481,6 +475,7 @@ def run_partitioned(args, agis, ds, stream, rank, world, local, dist, t_gen):
     dist.barrier()
     clocks = sampler.stop()
     ms = max_over_ranks(ev0.elapsed_time(ev1) / args.steps, dist)
+    solves = g.source_kernels()
     g.close()
     n_total = int(max_over_ranks(float(ds.n_obs), dist))
     # end to end: upload of the rank's part from pinned host buffers, one partitioned iteration,
@@ -514,7 +509,7 @@ def run_partitioned(args, agis, ds, stream, rank, world, local, dist, t_gen):
                                   "all-reduced (NCCL)", "t_generate_s": round(t_gen, 1), "t_init_s": round(t_init, 2)},
         "e2e": ({"value": n_total / float(np.median(e2e_t)), "unit": "obs/s", "h2d_bytes_per_step": int(h2d),
                  "d2h_bytes_per_step": int(out_src.numel() * 8)} if e2e_t else None),
-        "gpu_launches": (kernels_per_step("fp64", ds)[0] + 1) * args.steps,
+        "gpu_launches": (kernels_per_step("fp64", solves)[0] + 1) * args.steps,
         "clocks": clocks,
     }
     if rank == 0:
@@ -825,8 +820,8 @@ def main():
                                     "col_bin": args.cal_col_bin} if args.cal_generic else "r = 0 offsets per day")},
         "e2e": ({"value": e2e, "unit": "obs/s", "h2d_bytes_per_step": int(h2d), "d2h_bytes_per_step": int(d2h)}
                 if e2e is not None else None),
-        "gpu_launches": (kernels_per_step(head, ds)[0] * r["n_full_eval"] +
-                         kernels_per_step(head, ds)[1] * (steps_of[head] - r["n_full_eval"]) +
+        "gpu_launches": (kernels_per_step(head, r["solves"])[0] * r["n_full_eval"] +
+                         kernels_per_step(head, r["solves"])[1] * (steps_of[head] - r["n_full_eval"]) +
                          (KERNELS_ATTNOISE * steps_of[head] if an_ns > 0 else 0)),
         "clocks": r["clocks"],
         "roofline": fp64_roofline(r) if head == "fp64" else mixed_roofline(r),

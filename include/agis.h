@@ -236,6 +236,8 @@ int agis_get_source_stats(agis_ctx* ctx, double* stats_out, double* cov_out);
 
 /* Sizes of the context (n_obs, n_src, n_coef, n_cal). */
 int agis_get_sizes(const agis_ctx* ctx, int64_t* n_obs, int32_t* n_src, int32_t* n_coef, int32_t* n_cal);
+/* Kernels that the per-source solves of one source update launch (after the observation pass). */
+int agis_get_source_kernels(const agis_ctx* ctx, int32_t* n);
 /* Device time in ms of the kernels of the latest call, per kernel class (S pass, A
  * accumulation, A solve, C, frame): 5 doubles. */
 int agis_get_kernel_times(const agis_ctx* ctx, double* ms_out);

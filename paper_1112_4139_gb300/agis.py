@@ -24,7 +24,7 @@ EXPORTS = (
     "agis_default_config", "agis_init", "agis_source_update", "agis_attitude_update", "agis_calibration_update",
     "agis_frame_rotate", "agis_iterate", "agis_evaluate", "agis_get_sources", "agis_get_attitude",
     "agis_get_calibration", "agis_set_sources", "agis_set_attitude", "agis_set_calibration", "agis_get_residuals",
-    "agis_get_source_stats", "agis_get_sizes", "agis_get_kernel_times", "agis_destroy", "agis_last_error",
+    "agis_get_source_stats", "agis_get_sizes", "agis_get_source_kernels", "agis_get_kernel_times", "agis_destroy", "agis_last_error",
     "agis_abi_version", "agis_source_update_static", "agis_mlp_pack", "agis_mlp_forward", "agis_mlp_loss_grad",
     "agis_mlp_adam", "agis_proposal_targets", "agis_set_proposal", "agis_get_proposal_features",
     "agis_copy_sources_device", "agis_set_asi", "agis_asi_estimate", "agis_autotune", "agis_get_tuning",
@@ -119,6 +119,8 @@ def load():
         lib.agis_get_sizes.argtypes = [V, C.POINTER(C.c_int64), C.POINTER(C.c_int32), C.POINTER(C.c_int32),
                                        C.POINTER(C.c_int32)]
         lib.agis_get_sizes.restype = I
+        lib.agis_get_source_kernels.argtypes = [V, C.POINTER(C.c_int32)]
+        lib.agis_get_source_kernels.restype = I
         lib.agis_get_kernel_times.argtypes = [V, P]
         lib.agis_get_kernel_times.restype = I
         lib.agis_destroy.argtypes = [V]
@@ -309,6 +311,12 @@ class Agis:
         cov = np.empty((self.n_src, 5, 5))
         self._check(self._lib.agis_get_source_stats(self.ctx, _ptr(st), _ptr(cov)))
         return dict(eps2=st[0], Q=st[1], nu=st[2], n_out=st[3], D=st[4], cov=cov)
+
+    def source_kernels(self):
+        """Kernels that the per-source solves of one source update launch."""
+        n = C.c_int32()
+        self._check(self._lib.agis_get_source_kernels(self.ctx, C.byref(n)))
+        return n.value
 
     def kernel_times(self):
         ms = np.zeros(5)

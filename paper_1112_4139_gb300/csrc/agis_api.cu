@@ -19,6 +19,7 @@ void launch_obs_pass(const DevGeo& G, const AttNoise& an, const int64_t* t_ns, c
 void launch_source_solve(const Settings& st, bool corrections, const int64_t* src_off, const int32_t* src_nal,
                          const int32_t* src_order, int32_t n_src, const SrcOutPtrs& out, ObsRec* rec, double* scratch,
                          const uint64_t* skey, SrcWork* work, const Shapes& sh, cudaStream_t stream);
+int source_solve_kernels(const Settings& st, bool corrections);
 void launch_evaluate(const DevGeo& G, const int64_t* t_ns, const uint32_t* meta, const double* mu,
                      const int32_t* obs_src, int64_t n_obs, const double* src, const double* att, const double* cal,
                      double* R, cudaStream_t stream);
@@ -1050,18 +1051,21 @@ int agis_init(const agis_geometry* geo, const agis_config* cfg, const agis_obs* 
         if (cuda_check(c, cudaStreamSynchronize(s), "orders")) return bail(AGIS_E_CUDA);
     }
     c->mixed = cfg->precision == 1;
-    // FP64 S block: weight rounds by corrections to unit-weight sums (long sources: 30,000 of 820
-    // observations 1.4 + 4 x 0.49 ms a source update, against 0.5 + 5 x 1.7 ms for the direct sums
-    // of every row) or by direct sums (short sources gain less: 3000 of 165 80 + 4 x 36 us against
-    // 29 + 5 x 61).  FP64 A block: interval blocks by moments (24.7M observations in 157,786 intervals
-    // 9.93 -> 2.95 ms, 7.1M in 131,490 3.06 -> 1.51) or by the sums of the products.
-    // Both first forms round otherwise (no worse against 64 bits), which turns the last bit of 10 to 20%
-    // of the attitude coefficients, and the next iteration's calibration averages those bits: measured
-    // 4.5e-9 / sqrt(n / 1e6) of its norm, 1.4e-9 at 4.4M observations, 0.9e-9 at 24.7M in
-    // intervals of 100 or more.  Smaller sets keep the sums' order, so that their iterations reproduce bit
-    // for bit; but for many short intervals, whose coefficients the data determine to 1e-13 only.
-    c->src_corr = n >= 23000000 && n >= 512 * (int64_t)n_src && n >= 100 * (int64_t)c->n_iv;
-    c->att_moments = c->src_corr || (c->n_iv >= 120000 && n < 64 * (int64_t)c->n_iv);
+    // FP64 S block: weight rounds by corrections to unit-weight sums or by direct sums of every row; FP64 A
+    // block: interval blocks by moments or by the sums of the products.  What each saves follows from its own
+    // work.  Corrections, a whole source update: 1.03 to 1.10 with 165 observations per source, 1.14 to
+    // 1.20 with 330, 1.24 to 1.30 with 823 (fewer than 165 not measured).  Moments, a whole attitude update: 1.01 with 25
+    // observations per interval, 1.21 with 51, 1.66 with 106, 2.17 with 156; below kMomMin = 24 all
+    // intervals would take the products.
+    // Both round otherwise than the sums over all rows (no worse against 64 bits).  The attitude normals are
+    // nearly singular along the coefficient vector, so any change of rounding moves the last bits of most
+    // coefficients within two iterations, and with them the calibration: by 1.0e-9 to 1.35e-9 of its norm in
+    // sets of 0.5 to 14M observations (badly determined ones more), 0.9e-9 at 17 and 25M, 0.7e-9 at 50M, 0.6e-9 at
+    // 82M.  Results are kept within 1e-9 of those of the sums over all rows, so smaller sets keep these: the
+    // line lies between the last size near that bound and the next one measured, and is not about speed.
+    const bool large = n >= (int64_t)1 << 25;
+    c->src_corr = large && n >= 160 * (int64_t)n_src;
+    c->att_moments = large && n >= 24 * (int64_t)c->n_iv;
     if (c->mixed) {
         if ((rc = dalloc(c, &c->mo.s, n)) || (rc = dalloc(c, &c->mo.r, n)) || (rc = dalloc(c, &c->mo.ac, n)) ||
             (rc = dalloc(c, &c->mo.t, n)) || (rc = dalloc(c, &c->d_att, 4 * (size_t)n_coef)) ||
@@ -1776,6 +1780,12 @@ int agis_get_sizes(const agis_ctx* c, int64_t* n_obs, int32_t* n_src, int32_t* n
     if (n_src) *n_src = c->n_src;
     if (n_coef) *n_coef = c->n_coef;
     if (n_cal) *n_cal = c->n_cal;
+    return AGIS_OK;
+}
+
+int agis_get_source_kernels(const agis_ctx* c, int32_t* n) {
+    if (!c || !n) return AGIS_E_INVALID;
+    *n = c->mixed ? 2 * (c->st.robust ? c->st.n_rounds + 1 : 1) + 2 : source_solve_kernels(c->st, c->src_corr);
     return AGIS_OK;
 }
 

@@ -1094,6 +1094,13 @@ void launch_source_solve(const Settings& st, bool corrections, const int64_t* sr
     k_src_general<<<nb, th, 0, stream>>>(st, src_off, src_order, n_src, out, rec, scratch, work);
 }
 
+// kernels of one call: sums (a first pass and one pass per further round, or one per round) and 5x5 algebra of
+// every round, the hand-over records and the per-observation path
+int source_solve_kernels(const Settings& st, bool corrections) {
+    const int rounds = st.robust ? st.n_rounds + 1 : 1;
+    return 1 + (corrections ? rounds - 1 : rounds) + rounds + 2;
+}
+
 void launch_src_geo(int32_t n_src, const double* src, double* geo, cudaStream_t s) {
     k_src_geo<<<n_src > 0 ? (n_src + 31) / 32 : 1, 32, 0, s>>>(n_src, src, geo);
 }
