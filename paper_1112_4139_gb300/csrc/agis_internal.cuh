@@ -813,13 +813,14 @@ __device__ __forceinline__ double row_dot(const double A[5], const double* d) {
 
 // Direct class sums of one round: every row weighted (w = wfun(h rx) first, wfun((h - A d) isd)
 // later, 1 for plain weights), lane partials over the rows lane, lane + 32, ... of each class to
-// red[value][lane], then lane v adds the 32 partials of value v in lane order.  last: w goes to
-// the scratch row for the hand-over records.
+// red[value][lane], then lane v adds the 32 partials of value v in lane order.  about: the sums hold
+// h - A d in the place of h (so the solution is relative to d, and Q is formed without cancellation).
+// last: w goes to the scratch row for the hand-over records.
 constexpr int kRedVals = 2 * kSumVals;
 constexpr int kRedStride = 33;    // doubles per value row (odd: the column sums read distinct banks)
 __device__ __forceinline__ void direct_sums(double* scr, int n, int nal, int lane, int mode, const double* rx,
-                                            const double* isd, const double* d, int wfn, bool last, double* red,
-                                            double* out, int& nout) {
+                                            const double* isd, const double* d, bool about, int wfn, bool last,
+                                            double* red, double* out, int& nout) {
     int cnt = 0;
     for (int c = 0; c < 2; c++) {
         const int hi = c ? n : nal;
@@ -832,12 +833,14 @@ __device__ __forceinline__ void direct_sums(double* scr, int n, int nal, int lan
             double* e = scr + (size_t)j * kScr;
             double h, A[5];
             row_load(e, h, A);
+            const double t = mode == 1 || about ? h - row_dot(A, d) : h;
             double w = 1.0;
             if (mode == 0) {
                 if (rx[c] > 0.0) w = wfun(h * rx[c], wfn);
             } else if (mode == 1) {
-                w = wfun((h - row_dot(A, d)) * isd[c], wfn);
+                w = wfun(t * isd[c], wfn);
             }
+            if (about) h = t;
             if (last) e[6] = w;
             cnt += (w < 0.2);
 #pragma unroll

@@ -232,7 +232,8 @@ __device__ __forceinline__ void write_static(double* src, double* stats, int32_t
 // excess-noise step passes over the rows.
 // Bound: FP64 issue (64 cycles of a sub-partition per warp instruction).  2000 sources of 140
 // observations: 2.58 -> 1.29 ms (before: per-observation passes, two divisions each, for every step,
-// and 8-digit radix selects over the strided rows).
+// and 8-digit radix selects over the strided rows); 1.34 with the sums of the class path about the last solution, in
+// round 0 by a second pass where the start is far off.
 __global__ void __launch_bounds__(128) k_source_static(DevGeo G, Settings st, ObsPtrs ob, int64_t n_obs,
                                                        int32_t n_src, CcdRows rows, int64_t cal_t0, int64_t cal_dt,
                                                        int32_t n_days, double* __restrict__ src,
@@ -370,28 +371,50 @@ __global__ void __launch_bounds__(128) k_source_static(DevGeo G, Settings st, Ob
             int nu = 0, nout = 0, rdc = 0;
             const int rounds = st.robust ? st.n_rounds + 1 : 1, h = lane & 1;
             for (int rnd = 0; rnd < rounds; rnd++) {
-                direct_sums(scr, n, nal, lane, !st.robust ? 2 : (rnd ? 1 : 0), rx, isd, d, st.weight_fn,
-                            rnd == rounds - 1, ww.red, sums, nout);
-                HalfSums H;
-                for (int c = 0; c < 2; c++)
-                    for (int k = 0; k < 10; k++) H.E[c][k] = sums[kSumVals * c + 10 * h + k];
-                for (int k = 0; k < 15; k++) H.AA[k] = sums[kSumVals * h + k];
-                for (int k = 0; k < 5; k++) H.Ah[k] = sums[kSumVals * h + 15 + k];
-                H.hh = sums[kSumVals * h + 20];
-                __syncwarp();
-                nu = n - nout - 5;
-                y = 0.0;
-                class_solve_pair(H, h, s2c, 0.0, st.pivot_tol, U, d, rdc, Q, S2);
-                Q0 = Q;
-                if (st.robust && nu > 0 && Q0 > (double)nu) {   // the same in every lane
-                    const double tol = 1e-12 * s2min;
-                    for (int it = 0; it < st.n_eps; it++) {
-                        const double dy = (1.0 - Q / (double)nu) * Q / (-S2);
-                        y = fmax(0.0, y + dy);
-                        class_solve_pair(H, h, s2c, y, st.pivot_tol, U, d, rdc, Q, S2);
-                        if (fabs(dy) <= tol) break;
+                // Sums about the solution of the round before, and in round 0 about its own where the
+                // residuals fell to a sixteenth of their sum of squares or less (a start far off): Q, which
+                // the sums give as hh - 2 d'b + d'N d, then keeps the bits of sum w R^2.  Where a pivot fails, the
+                // zeroed parameters are those of d itself, so the sums are about zero.  All lanes agree.
+                const int mode = !st.robust ? 2 : (rnd ? 1 : 0);
+                double org[5], x[5];
+                for (int k = 0; k < 5; k++) org[k] = d[k];
+                bool about = rnd > 0, plain = false;
+                for (;;) {
+                    direct_sums(scr, n, nal, lane, mode, rx, isd, org, about, st.weight_fn, rnd == rounds - 1, ww.red, sums,
+                                nout);
+                    HalfSums H;
+                    for (int c = 0; c < 2; c++)
+                        for (int k = 0; k < 10; k++) H.E[c][k] = sums[kSumVals * c + 10 * h + k];
+                    for (int k = 0; k < 15; k++) H.AA[k] = sums[kSumVals * h + k];
+                    for (int k = 0; k < 5; k++) H.Ah[k] = sums[kSumVals * h + 15 + k];
+                    H.hh = sums[kSumVals * h + 20];
+                    const double all = sums[20] / s2c[0] + sums[kSumVals + 20] / s2c[1];
+                    __syncwarp();
+                    nu = n - nout - 5;
+                    y = 0.0;
+                    class_solve_pair(H, h, s2c, 0.0, st.pivot_tol, U, x, rdc, Q, S2);
+                    int defect = rdc;
+                    if (rnd == 0 && !about && !plain && defect == 0 && all > 16.0 * Q) {
+                        for (int k = 0; k < 5; k++) org[k] = x[k];
+                        about = true;
+                        continue;
                     }
+                    Q0 = Q;
+                    if (st.robust && nu > 0 && Q0 > (double)nu) {
+                        const double tol = 1e-12 * s2min;
+                        for (int it = 0; it < st.n_eps; it++) {
+                            const double dy = (1.0 - Q / (double)nu) * Q / (-S2);
+                            y = fmax(0.0, y + dy);
+                            class_solve_pair(H, h, s2c, y, st.pivot_tol, U, x, rdc, Q, S2);
+                            defect |= rdc;
+                            if (fabs(dy) <= tol) break;
+                        }
+                    }
+                    if (!about || defect == 0) break;
+                    about = false;
+                    plain = true;
                 }
+                for (int k = 0; k < 5; k++) d[k] = about ? org[k] + x[k] : x[k];
                 for (int c = 0; c < 2; c++) isd[c] = 1.0 / sqrt(s2c[c] + y);
             }
             const double iw[2] = {1.0 / (s2c[0] + y), 1.0 / (s2c[1] + y)};
