@@ -106,3 +106,33 @@ def test_far_rows_leave_no_trace(probe, robust, n_rounds, weight_fn, corrections
     assert probe.src_solve_eval(robust, n_rounds, 3, 0 if weight_fn == "agis" else 1, corrections, n_src, n,
                                 *[a.ctypes.data for a in (off, nal, rows, s, e, Q, nu, out, R, W)]) == 0
     compare(off, rows, ref, (R, W, s, e, Q, nu, out))
+
+
+@pytest.mark.parametrize("corrections", [0, 1])
+@pytest.mark.parametrize("start", [1e2, 1e3])
+def test_start_far_off(probe, start, corrections):
+    """Starting parameters far off (what a rejected proposal of 1000 sigma leaves): nothing becomes non-finite, and the
+    forms differ from the oracle by no more than the cancellation of the class sums, 2^-53 of sum W h^2 a row."""
+    off, nal, rows = rows_of()
+    rng = np.random.default_rng(5)
+    size = np.diff(off)
+    src = np.repeat(np.arange(len(size)), size)
+    rows[:, 0] += (rows[:, 1:6] * (start * SIGMA * rng.choice([-1.0, 1.0], (len(size), 5)))[src]).sum(1)
+    keep = np.isin(src, np.flatnonzero(size >= 64)) & (np.abs(rows[:, 0]) < 100 * start * SIGMA)
+    nal = np.array([np.count_nonzero(keep[off[i]:off[i] + nal[i]]) for i in range(len(size))], np.int32)
+    size = np.array([np.count_nonzero(keep[off[i]:off[i + 1]]) for i in range(len(size))])
+    rows, off = np.ascontiguousarray(rows[keep]), np.concatenate([[0], np.cumsum(size)]).astype(np.int64)
+    src = np.repeat(np.arange(len(size)), size)
+    n_src, n = len(nal), len(rows)
+    R0, W0, d0, e0, Q0, nu0, out0 = oracle_of(off, rows, OB.Settings())
+    s = np.zeros((n_src, 5))
+    e, Q, R, W = np.zeros(n_src), np.zeros(n_src), np.zeros(n), np.zeros(n)
+    nu, out = np.zeros(n_src, np.int32), np.zeros(n_src, np.int32)
+    assert probe.src_solve_eval(1, 4, 3, 0, corrections, n_src, n,
+                                *[a.ctypes.data for a in (off, nal, rows, s, e, Q, nu, out, R, W)]) == 0
+    assert all(np.isfinite(v).all() for v in (s, e, Q, R, W))
+    hh = np.bincount(src, W0 * rows[:, 0] ** 2, minlength=n_src)
+    # the sums of 21 products, their expansion and the three noise steps: 256 roundings
+    assert np.all(np.abs(Q - Q0) <= 256 * 2.0 ** -53 * hh + 1e-12 * Q0)
+    terms = np.abs(rows[:, 0]) + (np.abs(rows[:, 1:6]) * np.abs(d0)[src]).sum(1) + np.sqrt(rows[:, 6])
+    assert np.all(np.abs(R - R0) <= 1e-12 * terms)
