@@ -43,11 +43,12 @@ KERNELS_ATTNOISE = 4
 FALLBACK_HBM_GBS = 6800.0
 # algorithmic bytes per observation of the linearized observation pass (see time_form)
 MIX_PASS_BYTES = 8 + 16 + 4 + 8 + 8
-# DRAM bytes per observation (dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture
-# of 2.47e7 observations, scaled per observation; profiles/k_*_kernels_30k.md): the S block of
-# the FP64 form (observation pass + solves) and the mixed form's linearized pass.  None once
+# DRAM bytes per observation (dram__bytes_read.sum + dram__bytes_write.sum of ncu captures, scaled per
+# observation): the S block of the FP64 form (observation pass + solves in the form of large sets, 6.6e6
+# observations, profiles/launches_fp64_cases.md) and the mixed form's linearized pass (2.47e7,
+# profiles/k_mixed_kernels_30k.md).  None once
 # the kernel has changed since its capture.
-TRAFFIC_PER_OBS = {"fp64_s_block": None, "mixed_correct": 47.6}
+TRAFFIC_PER_OBS = {"fp64_s_block": 656.0, "mixed_correct": 47.6}
 
 
 def kernels_per_step(form, solves):

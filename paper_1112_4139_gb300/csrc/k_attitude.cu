@@ -158,8 +158,8 @@ __global__ void __launch_bounds__(128) k_att_accum(DevGeo G, double lambda2, int
 // below 2^24, so every sum is exact, and the pairs left out are about 2^-69 of the largest term
 // (FP64 rounds each product at 2^-53).  Products W g g', the forms and conversions are 64-bit
 // integer arithmetic.
-// Bound by reading: integer and shared-memory issue
-// and 68 FP64 instructions per interval for the expansion, where the FP64 form takes 116 FMAs and
+// Bound, by reading: integer and shared-memory issue (FP64 pipe 31% busy), and 68 FP64 instructions per
+// interval for the expansion, where the FP64 form takes 116 FMAs and
 // about 95 more FP64 instructions per observation (2 per clock and SM).
 // Attitude update, the products' sums against this: 24.7M observations in 157,786 intervals 11.6 -> 5.3 ms, 7.1M in
 // 131,490 4.62 -> 3.81 (a fifth of these intervals of 54 takes the products), 14M in 131,490 7.3 -> 4.4.

@@ -569,7 +569,7 @@ __global__ void __launch_bounds__(kSolveThreads) k_cg_solve(int nb, double tol, 
 // the reflections only the upper triangle is updated; the forward substitution rides along with
 // the factorisation as one more column.  Every entry receives the operations of the three kernels
 // in their order.
-// Bound: FP64 issue (m^3 / 6 FMAs of the trailing updates, the divisions of U's rows), one block per
+// Bound: two barriers per column (FP64 pipe 46% busy: m^3 / 6 FMAs of the trailing updates, U's rows), one block per
 // SM.  1612 groups of 123 bins and 30 cells: 11.3 (reduce 7.88, rhs 0.12, solve 3.32) -> 4.42 ms.
 constexpr int kSmemBins = 160;
 // a / b from the rounded reciprocal ib of b: the quotient's residual is exact in one FMA, and the

@@ -11,16 +11,18 @@
 //                 attitude pass and the calibration pass gather
 //   k_src_general sources whose sigma differs within a class: all rounds in one warp
 //
-// What bounds it: FP64 issue (2 FMA per clock and SM).  A 5x5 solve of one lane costs a warp as
+// What bounds it: the FP64 pipe (2 FMA per clock and SM; 86 to 92% busy in the passes over the rows, 63% in
+// k_src_round, which waits for rows at 12 warps an SM).  A 5x5 solve of one lane costs a warp as
 // many FP64 cycles as 32 of them, hence a thread per source there.  Downweighting leaves w = 1
 // wherever |z| <= 2 (Eqs. dw, dwH), about 95% of the observations, so for long sources the 21
 // products of a row within two robust scales are summed once, with unit weights; a round evaluates z in
 // FP32 (with a bound on its error), and only the rows that may exceed 2 or that those sums do not hold are
 // gathered, 32 to a warp, for the FP64 weight and 27 products: a round then costs about a fifth of
 // the FP64 work of the direct sums.
-// Measured, source solves of the S block: 24.7M observations of 30,000 sources 14.2 -> 4.5 ms; with
-// direct sums 6.7M of 8000 sources 4.75 -> 2.9, 0.5M of 3000 sources 1.68 -> 0.57.  Before, one persistent
-// kernel ran all rounds of a batch of sources in a warp, with the 5x5 solves in one lane each.
+// Measured, source solves of the S block: 6.6M observations of 8000 sources 4.75 -> 2.9 ms with direct
+// sums (first pass 0.12 ms, sums 5 x 0.47), 1.5 with corrections (first sums 0.37, rounds 4 x 0.175); 0.5M of
+// 3000 sources 1.68 -> 0.57 with direct sums.  Before, one persistent kernel ran all rounds of a batch of sources in a
+// warp, with the 5x5 solves in one lane each.
 #include <type_traits>
 
 #include "agis_internal.cuh"

@@ -230,7 +230,7 @@ __device__ __forceinline__ void write_static(double* src, double* stats, int32_t
 // source have one sigma each, the rows are laid out AL first and the inner iteration works on
 // class sums (one pass over the rows per round, the 5x5 algebra by pairs of lanes); otherwise every
 // excess-noise step passes over the rows.
-// Bound: FP64 issue (64 cycles of a sub-partition per warp instruction).  2000 sources of 140
+// Bound: FP64 instructions (64 cycles of a sub-partition each; pipe 75% busy) of one chain per warp.  2000 sources of 140
 // observations: 2.58 -> 1.29 ms (before: per-observation passes, two divisions each, for every step,
 // and 8-digit radix selects over the strided rows); 1.34 with the sums of the class path about the last solution, in
 // round 0 by a second pass where the start is far off.
