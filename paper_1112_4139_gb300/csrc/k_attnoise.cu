@@ -332,7 +332,7 @@ __global__ void k_an_weights(int64_t n, AttNoise an, const ObsRec* __restrict__ 
         const double s = (double)sigma[o];
         const double v = __dadd_rn(__dadd_rn(__dmul_rn(s, s), an.eps2[an_index(an, t, m)]), eps2_src[obs_src[o]]);
         const double iv = rcp_pos(v), z2 = R * R * iv;   // w is 1 up to |z| = 2: no root for most rows
-        w_att[o] = __double2hiint(z2) < 0x40100000 ? iv : wfun(sqrt(z2), weight_fn) * iv;
+        w_att[o] = (__double2hiint(z2) & 0x7fffffff) < 0x40100000 ? iv : wfun(sqrt(z2), weight_fn) * iv;
     }
 }
 

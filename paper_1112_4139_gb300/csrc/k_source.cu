@@ -886,7 +886,7 @@ __device__ __forceinline__ void pass_normals(double* scr, int n, int lane, doubl
                 if (kMode == kGenOne)
                     iv = rcp_pos(ws.y + y);
                 else
-                    cand = __double2hiint(z2_of(h, A, ws.y, iv)) >= 0x40100000;   // 4 and above, or not a number
+                    cand = (__double2hiint(z2_of(h, A, ws.y, iv)) & 0x7fffffff) >= 0x40100000;   // 4 and above, or not a number
                 if (!cand) {
                     e[6] = 1.0;
                     add(iv, h, A);

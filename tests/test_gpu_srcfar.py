@@ -136,3 +136,32 @@ def test_start_far_off(probe, start, corrections):
     assert np.all(np.abs(Q - Q0) <= 256 * 2.0 ** -53 * hh + 1e-12 * Q0)
     terms = np.abs(rows[:, 0]) + (np.abs(rows[:, 1:6]) * np.abs(d0)[src]).sum(1) + np.sqrt(rows[:, 6])
     assert np.all(np.abs(R - R0) <= 1e-12 * terms)
+
+
+@pytest.mark.parametrize("corrections", [0, 1])
+@pytest.mark.parametrize("sign", [1, -1])        # what inf - inf gives on the GPU has the sign bit set
+def test_a_row_that_is_not_a_number_has_no_weight(probe, sign, corrections):
+    """One such residual among those of a source of one sigma per class and of one whose sigma differs: its own weight is
+    not a number either (the pivots of its source fail, so the other rows keep theirs), and the other sources are as
+    without it."""
+    off, nal, rows = rows_of()
+    n_src, n = len(nal), len(rows)
+    hit = [10, 11]                                # 820 rows of one sigma per class, 840 that differ
+    assert list(np.diff(off)[hit]) == [820, 840]
+
+    def solve(rows):
+        s = np.zeros((n_src, 5))
+        e, Q, R, W = np.zeros(n_src), np.zeros(n_src), np.zeros(n), np.zeros(n)
+        nu, out = np.zeros(n_src, np.int32), np.zeros(n_src, np.int32)
+        assert probe.src_solve_eval(1, 4, 3, 0, corrections, n_src, n,
+                                    *[a.ctypes.data for a in (off, nal, rows, s, e, Q, nu, out, R, W)]) == 0
+        return s, Q, R, W
+    bad = rows.copy()
+    bad[off[hit] + 5, 0] = np.copysign(np.nan, sign)
+    a, b = solve(bad), solve(rows)
+    src = np.repeat(np.arange(n_src), np.diff(off))
+    own = np.isin(src, hit)
+    assert np.isnan(a[3][off[hit] + 5]).all() and np.isnan(a[2][off[hit] + 5]).all()
+    other = ~np.isin(np.arange(n_src), hit)
+    assert np.array_equal(a[0][other], b[0][other]) and np.array_equal(a[1][other], b[1][other])
+    assert np.array_equal(a[2][~own], b[2][~own]) and np.array_equal(a[3][~own], b[3][~own])
